@@ -442,8 +442,9 @@ typedef struct {
  *   both clamped to [-2^30, 2^30];
  * tile (a, b, c) is a candidate iff lo <= (a, b, c) <= hi per axis.  A
  * Gaussian with a non-finite mean or scale, a scale <= 0 or a zero quaternion
- * is nobody's candidate.  Each voxel sums its tile's candidates in increasing
- * Gaussian index (float32; the results are deterministic).
+ * is nobody's candidate.  Each voxel's float32 sum over its tile's candidates
+ * is taken in a fixed order (the results are deterministic); close to theta,
+ * in increasing Gaussian index.
  *   out_density: device float32 [n_voxels] (required);
  *   out_occ / out_surf: device uint8 [n_voxels] (0/1), either may be NULL;
  *   stats: may be NULL (see fgl_density_stats for its one input field).

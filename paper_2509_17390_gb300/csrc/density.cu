@@ -14,9 +14,9 @@
 //                  every tile's candidates end up in increasing Gaussian
 //                  index and the float32 sums are deterministic;
 //   k_tile_bounds  begin/end of every tile's candidate run;
-//   k_density<B>   one block per tile: candidates staged in shared memory in
-//                  chunks, each thread accumulates one x-row of voxels over
-//                  them in packed f32x2 arithmetic (one ex2 per evaluation);
+//   k_density<B>   one block per tile: each warp stages candidates in shared
+//                  memory and sums them over the tile's x-rows, a row's voxels
+//                  from three exponentials;
 //   k_occ_surf     D > theta and the 6-neighbour surface test.
 //
 // The paper finds the candidates of a tile with an LBVH query over Gaussian
@@ -223,94 +223,276 @@ __global__ void k_tile_bounds(const uint32_t* __restrict__ keys, int64_t n,
 }
 
 // ---------------------------------------------------------------------------
-// density: one block per tile of B^3 voxels; each thread owns one x-row of
-// the tile (B voxels sharing the y/z part of the quadratic form) and works on
-// voxel pairs with packed f32x2 arithmetic
+// density: one block per tile of B^3 voxels.  Each warp of the block sums
+// every S-th batch of 32 candidates over the whole tile (two x-rows a lane, so
+// that a staged candidate is read once for 64 rows); the warps' sums are added
+// in warp order.  Bound by instruction issue and the FMA pipe about equally
+// (36 warp instructions for a candidate and 32 rows, of which 3 exponentials;
+// one exponential a voxel took 40, and 8 of them held the MUFU pipe longest).
+// 720 k Gaussians, 10,304 tiles of 2.5 cm voxels: 2.22 -> 1.51 ms; 85 k
+// Gaussians, 630 tiles of 5 cm: 0.63 -> 0.20 ms.
 // ---------------------------------------------------------------------------
-template <int B>
-struct DensityCfg {
-  static constexpr int THREADS = B * B;  // one x-row each: 64 for B = 8, 16 for B = 4
-  static constexpr int CHUNK = 128;      // candidates staged per pass
-};
-
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   uint64_t d;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
+// A row's exponent is a parabola in x: about the row's middle xm,
+//   q(xm + d) = q(xm) + g d + M00 d^2,
+// so its B values are E P^j c_j with E = 2^q(xm), P = 2^(g h / 2) and
+// c_j = alpha^2 2^(M00 (j h / 2)^2), j = +-1, +-3, .. the voxel's distance
+// from the middle in half voxels: three exponentials a row (E, P, 1 / P) and
+// two packed operations a voxel pair instead of one exponential a voxel.
+// Taken when the parabola falls by at most 2^kRowFall from the middle to the
+// end of the row: E P^j then stays below 2^kRowFall, and where E underflows
+// (below 2^-126) the row's largest value is below 2^-45.  P^2 has to stay
+// finite too (|g h / 2| <= kRowSlope), so that a row far from the Gaussian adds
+// 0 and not 0 times infinity.  A Gaussian outside these limits (steep) is
+// evaluated voxel by voxel.
+constexpr float kRowFall = 20.f, kRowSlope = 60.f;
+
+// Voxels whose density falls this close to theta (relative) are summed again
+// voxel by voxel in candidate order, so that the masks never hang on the
+// rounding of the factored form or of the warps' partial sums: they differ
+// from those sums by a few 1e-6 (a term's exponent by a few units of 2^-24 of
+// its partial sums).
+constexpr float kThetaBand = 1e-4f;
+
+// One staged candidate.  bx = M01 dy + M02 dz is the x coefficient and
+// syz = M11 dy^2 + M12 dy dz + M22 dz^2 the y/z part of the exponent.
+struct __align__(16) StagedGauss {
+  float4 at;     // dY, dZ (tile corner minus mean), xm, M00 xm; steep: dX in z, 0 in w
+  float4 m;      // M11, M22, M12, M01
+  float4 n;      // M02, M00 xm h / 2, alpha^2, M00
+  float4 c[2];   // c_1, c_1, c_3, c_3 | c_5, c_5, c_7, c_7
+};
 
 template <int B>
-__global__ void __launch_bounds__(DensityCfg<B>::THREADS)
+struct DensityCfg {
+  static constexpr int ROWS = B * B;
+  static constexpr int LANES = ROWS / 2;    // lanes that cover the tile, two rows each
+  static constexpr int SUB = 32 / LANES;    // candidates a warp takes at once
+};
+
+template <int B, int S>
+__global__ void __launch_bounds__(32 * S)
     k_density(const GaussParams* __restrict__ params, const uint32_t* __restrict__ cand,
-              const uint32_t* __restrict__ begin, const uint32_t* __restrict__ end, GridArgs g,
+              const uint32_t* __restrict__ begin, const uint32_t* __restrict__ end, GridArgs g, float theta,
               float* __restrict__ out) {
   using C = DensityCfg<B>;
-  // staged candidate k:  s0 = (dX, dX, M00, M00), s1 = (a2, a2, dY, dZ),
-  // s2 = (M11, M22, M01, M02), s3 = M12, with (dX, dY, dZ) = tile corner - mu
-  __shared__ float4 s0[C::CHUNK], s1[C::CHUNK], s2[C::CHUNK];
-  __shared__ float s3[C::CHUNK];
+  constexpr int NT = 32 * S;
+  __shared__ StagedGauss stage[S][32];
+  __shared__ float s_sum[S > 1 ? S - 1 : 1][C::ROWS * B];
+  const unsigned FULL = 0xFFFFFFFFu;
   const int tile = blockIdx.x;
   const int tx = tile % g.ntiles[0], ty = (tile / g.ntiles[0]) % g.ntiles[1],
             tz = tile / (g.ntiles[0] * g.ntiles[1]);
   const uint32_t b0 = begin[tile], b1 = end[tile];
-  const int t = threadIdx.x;
-  const int y = t % B, z = t / B;
-  uint64_t ox2[B / 2];
-#pragma unroll
-  for (int p = 0; p < B / 2; ++p)
-    ox2[p] = dev::pack2f(((float)(2 * p) + 0.5f) * g.h, ((float)(2 * p + 1) + 0.5f) * g.h);
-  const float oy = ((float)y + 0.5f) * g.h, oz = ((float)z + 0.5f) * g.h;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int slot = lane % C::LANES, sub = lane / C::LANES, y = slot % B, z = slot / B;  // rows (y, z), (y, z + B / 2)
+  StagedGauss* st = stage[warp];
   // tile corner in FP64 (the offsets to the means are formed there, then
   // rounded once: |tile corner - mu| is small, so the float offset is accurate)
   const double cx = (double)g.o[0] + (double)(tx * B) * (double)g.h;
   const double cy = (double)g.o[1] + (double)(ty * B) * (double)g.h;
   const double cz = (double)g.o[2] + (double)(tz * B) * (double)g.h;
-  uint64_t acc2[B / 2];
+  const double mid = (double)(B / 2) * (double)g.h;
+  const float hh = 0.5f * g.h, end_d = (float)(B - 1) * hh;
+  const float oy = ((float)y + 0.5f) * g.h;
+  const float oz[2] = {((float)z + 0.5f) * g.h, ((float)(z + B / 2) + 0.5f) * g.h};
+  uint64_t acc[2][B / 2];  // voxel pairs mirrored about the row's middle, innermost first
 #pragma unroll
-  for (int p = 0; p < B / 2; ++p) acc2[p] = 0ull;
-  for (uint32_t c0 = b0; c0 < b1; c0 += C::CHUNK) {
-    const uint32_t m = min((uint32_t)C::CHUNK, b1 - c0);
-    __syncthreads();
-    for (uint32_t k = t; k < m; k += C::THREADS) {
-      const GaussParams P = params[cand[c0 + k]];
-      const float dX = (float)(cx - (double)P.a.x);
-      s0[k] = make_float4(dX, dX, P.b.x, P.b.x);
-      s1[k] = make_float4(P.a.w, P.a.w, (float)(cy - (double)P.a.y), (float)(cz - (double)P.a.z));
-      s2[k] = make_float4(P.b.y, P.b.z, P.b.w, P.c.x);
-      s3[k] = P.c.y;
+  for (int r = 0; r < 2; ++r)
+#pragma unroll
+    for (int p = 0; p < B / 2; ++p) acc[r][p] = 0ull;
+  // a batch's parameters travel while the one before it is summed, its
+  // candidate numbers one batch earlier
+  GaussParams P = {};
+  uint32_t next = 0;
+  if (b0 + 32 * warp + lane < b1) P = params[cand[b0 + 32 * warp + lane]];
+  if (b0 + 32 * (warp + S) + lane < b1) next = cand[b0 + 32 * (warp + S) + lane];
+  for (uint32_t c0 = b0 + 32 * warp; c0 < b1; c0 += 32 * S) {
+    __syncwarp();  // the batch before this one is summed
+    const bool valid = c0 + lane < b1;
+    const float dX = (float)(cx - (double)P.a.x), dY = (float)(cy - (double)P.a.y), dZ = (float)(cz - (double)P.a.z);
+    // |g h / 2| over the tile's rows, from above: P^2 stays finite
+    const float most = 2.f * end_d + g.h;  // the tile's edge
+    const float slope = hh * (fabsf(P.b.w) * (fabsf(dY) + most) + fabsf(P.c.x) * (fabsf(dZ) + most) +
+                              2.f * fabsf(P.b.x) * (fabsf(dX) + most));
+    const bool fast = valid && fabsf(P.b.x) * (end_d * end_d) <= kRowFall && slope <= kRowSlope;
+    // the factored ones first, steep ones from the end
+    const unsigned fm = __ballot_sync(FULL, fast), sm = __ballot_sync(FULL, valid && !fast);
+    const unsigned below = (1u << lane) - 1u;
+    const int nf = __popc(fm), ns = __popc(sm);
+    if (valid) {
+      StagedGauss& q = st[fast ? __popc(fm & below) : 31 - __popc(sm & below)];
+      const float xm = (float)((cx + (fast ? mid : 0.0)) - (double)P.a.x), u = fast ? P.b.x * xm : 0.f;
+      q.at = make_float4(dY, dZ, xm, u);
+      q.m = make_float4(P.b.y, P.b.z, P.c.y, P.b.w);
+      q.n = make_float4(P.c.x, u * hh, P.a.w, P.b.x);
+      if (fast) {
+        const float k1 = P.b.x * hh * hh;
+        const float c1 = P.a.w * exp2f(k1), c3 = P.a.w * exp2f(9.f * k1), c5 = P.a.w * exp2f(25.f * k1),
+                    c7 = P.a.w * exp2f(49.f * k1);
+        q.c[0] = make_float4(c1, c1, c3, c3);
+        q.c[1] = make_float4(c5, c5, c7, c7);
+      }
     }
-    __syncthreads();
-    for (uint32_t k = 0; k < m; ++k) {
-      const float4 A = s0[k], W = s1[k], M = s2[k];
-      const float m12 = s3[k];
-      const float dy = W.z + oy, dz = W.w + oz;
-      // y/z part M11 dy^2 + M12 dy dz + M22 dz^2 and x coefficient M01 dy + M02 dz
-      const float syz = fmaf(fmaf(M.x, dy, m12 * dz), dy, (M.y * dz) * dz);
-      const float bx = fmaf(M.z, dy, M.w * dz);
-      const uint64_t dX2 = dev::pack2f(A.x, A.y), M002 = dev::pack2f(A.z, A.w);
-      const uint64_t a22 = dev::pack2f(W.x, W.y);
-      const uint64_t bx2 = dev::pack2f(bx, bx), syz2 = dev::pack2f(syz, syz);
+    __syncwarp();
+    if (c0 + 32 * S + lane < b1) P = params[next];
+    if (c0 + 64 * S + lane < b1) next = cand[c0 + 64 * S + lane];
+#pragma unroll 1
+    for (int i = sub; i < nf; i += C::SUB) {
+      const float4 at = st[i].at, m = st[i].m, n = st[i].n;
+      const float4 w0 = st[i].c[0], w1 = st[i].c[1];
+      const float dy = at.x + oy;
+      const float ay = (m.x * dy) * dy, by = fmaf(m.w, dy, at.w);
+      uint64_t t2[2], PP[2];
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const float dz = at.y + oz[r];
+        const float a = fmaf(n.x, dz, by);
+        const float qm = fmaf(a, at.z, fmaf(fmaf(m.z, dy, m.y * dz), dz, ay));
+        const float gh = fmaf(a, hh, n.y);
+        const float E = dev::ex2_approx(qm), Pl = dev::ex2_approx(-gh), Pr = dev::ex2_approx(gh);
+        t2[r] = dev::pack2f(E * Pl, E * Pr);
+        PP[r] = dev::pack2f(Pl * Pl, Pr * Pr);
+      }
 #pragma unroll
       for (int p = 0; p < B / 2; ++p) {
-        const uint64_t dx2 = add2(dX2, ox2[p]);
-        const uint64_t q2 = dev::ffma2(dev::ffma2(M002, dx2, bx2), dx2, syz2);  // <= 0
-        float q0, q1;
-        dev::unpack2f(q2, q0, q1);
-        acc2[p] = dev::ffma2(a22, dev::pack2f(dev::ex2_approx(q0), dev::ex2_approx(q1)), acc2[p]);
+        const float4 w = p < 2 ? w0 : w1;
+        const uint64_t w2 = (p & 1) ? dev::pack2f(w.z, w.w) : dev::pack2f(w.x, w.y);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          if (p) t2[r] = mul2(t2[r], PP[r]);
+          acc[r][p] = dev::ffma2(t2[r], w2, acc[r][p]);
+        }
+      }
+    }
+#pragma unroll 1
+    for (int i = 31 - sub; i > 31 - ns; i -= C::SUB) {
+      const float4 at = st[i].at, m = st[i].m, n = st[i].n;
+      const float dy = at.x + oy;
+      const float ay = (m.x * dy) * dy, by = m.w * dy;
+      const uint64_t M002 = dev::pack2f(n.w, n.w), dX2 = dev::pack2f(at.z, at.z), a22 = dev::pack2f(n.z, n.z);
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const float dz = at.y + oz[r];
+        const float bx = fmaf(n.x, dz, by), syz = fmaf(fmaf(m.z, dy, m.y * dz), dz, ay);
+        const uint64_t bx2 = dev::pack2f(bx, bx), syz2 = dev::pack2f(syz, syz);
+#pragma unroll
+        for (int p = 0; p < B / 2; ++p) {
+          const uint64_t dx2 =
+              add2(dX2, dev::pack2f(((float)(B / 2 - 1 - p) + 0.5f) * g.h, ((float)(B / 2 + p) + 0.5f) * g.h));
+          float q0, q1;
+          dev::unpack2f(dev::ffma2(dev::ffma2(M002, dx2, bx2), dx2, syz2), q0, q1);  // <= 0
+          acc[r][p] = dev::ffma2(a22, dev::pack2f(dev::ex2_approx(q0), dev::ex2_approx(q1)), acc[r][p]);
+        }
       }
     }
   }
-  const int gx = tx * B, gy = ty * B + y, gz = tz * B + z;
-  if (gy < g.dims[1] && gz < g.dims[2]) {
-    float* row = out + ((int64_t)gz * g.dims[1] + gy) * g.dims[0];
+  float d[2][B];  // the rows' densities, complete in warp 0's lanes of sub 0
 #pragma unroll
-    for (int p = 0; p < B / 2; ++p) {
-      float a0, a1;
-      dev::unpack2f(acc2[p], a0, a1);
-      if (gx + 2 * p < g.dims[0]) row[gx + 2 * p] = a0;
-      if (gx + 2 * p + 1 < g.dims[0]) row[gx + 2 * p + 1] = a1;
+  for (int r = 0; r < 2; ++r)
+#pragma unroll
+    for (int p = 0; p < B / 2; ++p) dev::unpack2f(acc[r][p], d[r][B / 2 - 1 - p], d[r][B / 2 + p]);
+#pragma unroll
+  for (int o = C::LANES; o < 32; o <<= 1)
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+      for (int i = 0; i < B; ++i) d[r][i] += __shfl_xor_sync(FULL, d[r][i], o);
+  if (S > 1) {
+    if (warp > 0 && sub == 0) {
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int i = 0; i < B; ++i) s_sum[warp - 1][(r * B + i) * C::LANES + slot] = d[r][i];
+    }
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll 1
+      for (int v = 0; v + 1 < S; ++v)
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+          for (int i = 0; i < B; ++i) d[r][i] += s_sum[v][(r * B + i) * C::LANES + slot];
     }
   }
+  const int gx = tx * B, gy = ty * B + y;
+  const bool owner = warp == 0 && sub == 0 && gy < g.dims[1];
+  // voxels close to theta: their terms, a candidate a thread, then one
+  // thread's sum in candidate order
+  uint32_t close = 0;
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+#pragma unroll
+    for (int i = 0; i < B; ++i)
+      if (owner && tz * B + z + r * (B / 2) < g.dims[2] &&
+          fabsf(d[r][i] - theta) <= kThetaBand * (fabsf(d[r][i]) + fabsf(theta)))
+        close |= 1u << (r * B + i);
+  if (__syncthreads_or(close != 0u && b1 > b0)) {
+    __shared__ uint32_t s_close[C::LANES];
+    float* s_q = reinterpret_cast<float*>(stage);  // alpha^2 and 2^q of a batch of candidates
+    if (threadIdx.x < C::LANES) s_close[threadIdx.x] = close;
+    __syncthreads();
+    for (int o = 0; o < C::LANES; ++o) {
+      for (uint32_t left = s_close[o]; left; left &= left - 1) {  // the same for the whole block
+        const int bit = __ffs(left) - 1, i = bit % B;
+        const float vx = __fmul_rn((float)i + 0.5f, g.h), vy = __fmul_rn((float)(o % B) + 0.5f, g.h),
+                    vz = __fmul_rn((float)(o / B + (bit / B) * (B / 2)) + 0.5f, g.h);
+        float sum = 0.f;
+        for (uint32_t c0 = b0; c0 < b1; c0 += NT) {
+          if (c0 + threadIdx.x < b1) {
+            const GaussParams Q = params[cand[c0 + threadIdx.x]];
+            const float dx = __fadd_rn((float)(cx - (double)Q.a.x), vx), dy = __fadd_rn((float)(cy - (double)Q.a.y), vy),
+                        dz = __fadd_rn((float)(cz - (double)Q.a.z), vz);
+            const float syz = fmaf(fmaf(Q.b.y, dy, __fmul_rn(Q.c.y, dz)), dy, __fmul_rn(__fmul_rn(Q.b.z, dz), dz));
+            const float bx = fmaf(Q.b.w, dy, __fmul_rn(Q.c.x, dz));
+            s_q[2 * threadIdx.x] = Q.a.w;
+            s_q[2 * threadIdx.x + 1] = dev::ex2_approx(fmaf(fmaf(Q.b.x, dx, bx), dx, syz));
+          }
+          __syncthreads();
+          if (threadIdx.x == o) {
+            const int m = (int)min((uint32_t)NT, b1 - c0);
+#pragma unroll 8
+            for (int k = 0; k < m; ++k) sum = fmaf(s_q[2 * k], s_q[2 * k + 1], sum);
+          }
+          __syncthreads();
+        }
+        if (threadIdx.x == o) {
+#pragma unroll
+          for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int j = 0; j < B; ++j)
+              if (r * B + j == bit) d[r][j] = sum;
+        }
+      }
+    }
+  }
+  if (owner) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int gz = tz * B + z + r * (B / 2);
+      if (gz >= g.dims[2]) break;
+      float* dst = out + ((int64_t)gz * g.dims[1] + gy) * g.dims[0];
+#pragma unroll
+      for (int i = 0; i < B; ++i)
+        if (gx + i < g.dims[0]) dst[gx + i] = d[r][i];
+    }
+  }
+}
+
+template <int B, int S>
+void launch_density(int64_t n_tiles, const GaussParams* params, const uint32_t* cand, const uint32_t* begin,
+                    const uint32_t* end, const GridArgs& g, float theta, float* out, cudaStream_t s) {
+  k_density<B, S><<<(unsigned)n_tiles, 32 * S, 0, s>>>(params, cand, begin, end, g, theta, out);
 }
 
 // eqs. V_occ, Int, Surf: x over blockIdx.x, rows (y, z) strided over
@@ -518,12 +700,16 @@ extern "C" fgl_status fgl_gaussian_density(const fgl_gaussians* gs, const fgl_gr
     ++launches;
     DCUDA(cudaGetLastError());
     if (timing) DCUDA(cudaEventRecord(S.ev[1], s));
-    if (B == 8)
-      k_density<8><<<(unsigned)n_tiles, DensityCfg<8>::THREADS, 0, s>>>(
-          (const GaussParams*)S.params, v0, begin, end, g, out_density);
-    else
-      k_density<4><<<(unsigned)n_tiles, DensityCfg<4>::THREADS, 0, s>>>(
-          (const GaussParams*)S.params, v0, begin, end, g, out_density);
+    // Warps a tile: four of 32 candidates each even out tiles of unequal counts
+    // (2.25 ms for the pass at 10,304 tiles, 2.53 with two, 2.99 with one); a
+    // grid of fewer than 16 tiles an SM takes eight, or its few tiles would
+    // leave most of the chip idle.
+    const GaussParams* params = (const GaussParams*)S.params;
+    const bool few = n_tiles < 152 * 16;
+    if (B == 8 && few) launch_density<8, 8>(n_tiles, params, v0, begin, end, g, theta, out_density, s);
+    else if (B == 8) launch_density<8, 4>(n_tiles, params, v0, begin, end, g, theta, out_density, s);
+    else if (few) launch_density<4, 4>(n_tiles, params, v0, begin, end, g, theta, out_density, s);
+    else launch_density<4, 1>(n_tiles, params, v0, begin, end, g, theta, out_density, s);
     ++launches;
     DCUDA(cudaGetLastError());
     if (timing) DCUDA(cudaEventRecord(S.ev[2], s));
