@@ -13,8 +13,6 @@ size_t scan_tmp_elems(int64_t n);
 
 // Exclusive prefix sums in place on `stream`; `tmp` holds scan_tmp_elems(n)
 // elements.  `launches` counts the kernels launched.
-cudaError_t scan_exclusive_u32(uint32_t* x, int64_t n, uint32_t* tmp, size_t tmp_elems,
-                               cudaStream_t s, int* launches);
 cudaError_t scan_exclusive_u64(unsigned long long* x, int64_t n, unsigned long long* tmp,
                                size_t tmp_elems, cudaStream_t s, int* launches);
 
