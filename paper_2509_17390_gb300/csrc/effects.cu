@@ -11,7 +11,7 @@
 //   - noise: a kept hit at range t becomes t + (sigma0 + sigma1 t) n,
 //     n = sqrt(-2 ln u1) cos(2 pi u2) (Box-Muller), u1 = ((x1 >> 8) + 1) 2^-24,
 //     u2 = (x2 >> 8) 2^-24, clamped to [0, max_range]; float32 arithmetic.
-// Misses are left as they are.  One thread per return, grid-stride.
+// Misses are left as they are.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -26,17 +26,19 @@ void record_error(int status, const char* msg);  // api.cu
 
 namespace {
 
+// The ten round keys, the key schedule of (seed low, seed high): made once on
+// the host, they reach the rounds as constants.
+struct RoundKeys {
+  uint32_t k0[10], k1[10];
+};
+
 __device__ __forceinline__ void philox4x32_10(uint32_t& c0, uint32_t& c1, uint32_t& c2, uint32_t& c3,
-                                              uint32_t k0, uint32_t k1) {
+                                              const RoundKeys& k) {
 #pragma unroll
   for (int r = 0; r < 10; ++r) {
-    if (r > 0) {
-      k0 += 0x9E3779B9u;
-      k1 += 0xBB67AE85u;
-    }
-    const uint32_t lo0 = 0xD2511F53u * c0, hi0 = __umulhi(0xD2511F53u, c0);
-    const uint32_t lo1 = 0xCD9E8D57u * c2, hi1 = __umulhi(0xCD9E8D57u, c2);
-    const uint32_t n0 = hi1 ^ c1 ^ k0, n2 = hi0 ^ c3 ^ k1;
+    const uint64_t p0 = (uint64_t)0xD2511F53u * c0, p1 = (uint64_t)0xCD9E8D57u * c2;
+    const uint32_t lo0 = (uint32_t)p0, hi0 = (uint32_t)(p0 >> 32), lo1 = (uint32_t)p1, hi1 = (uint32_t)(p1 >> 32);
+    const uint32_t n0 = hi1 ^ c1 ^ k.k0[r], n2 = hi0 ^ c3 ^ k.k1[r];
     c0 = n0;
     c1 = lo1;
     c2 = n2;
@@ -44,27 +46,97 @@ __device__ __forceinline__ void philox4x32_10(uint32_t& c0, uint32_t& c1, uint32
   }
 }
 
-__global__ void k_effects(float* __restrict__ range, int32_t* __restrict__ tri, int64_t n, int n_rays,
-                          int env_offset, uint32_t step, uint32_t k0, uint32_t k1, float drop_prob,
-                          float sigma0, float sigma1, float max_range) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-    if (tri[i] < 0) continue;
-    const int64_t e = i / n_rays;
-    uint32_t x0 = (uint32_t)(i - e * n_rays), x1 = (uint32_t)(env_offset + e), x2 = step, x3 = 0u;
-    philox4x32_10(x0, x1, x2, x3, k0, k1);
-    const float inv24 = 5.9604644775390625e-8f;  // 2^-24
-    if ((float)(x0 >> 8) * inv24 < drop_prob) {
-      range[i] = max_range;
-      tri[i] = -1;
-      continue;
+// One return: true when it changed its range; *drop when it became a miss.
+struct Effects {
+  RoundKeys key;
+  uint32_t step;
+  int32_t env_offset;
+  float drop_prob, sigma0, sigma1, max_range;
+};
+
+__device__ __forceinline__ bool apply(const Effects& fx, uint32_t ray, uint32_t env, float& t, int32_t& tri) {
+  if (tri < 0) return false;
+  uint32_t x0 = ray, x1 = env, x2 = fx.step, x3 = 0u;
+  philox4x32_10(x0, x1, x2, x3, fx.key);
+  const float inv24 = 5.9604644775390625e-8f;  // 2^-24
+  if ((float)(x0 >> 8) * inv24 < fx.drop_prob) {
+    t = fx.max_range;
+    tri = -1;
+    return true;
+  }
+  if (fx.sigma0 == 0.f && fx.sigma1 == 0.f) return false;
+  const float u1 = (float)((x1 >> 8) + 1u) * inv24, u2 = (float)(x2 >> 8) * inv24;
+  const float nrm = sqrtf(-2.f * logf(u1)) * cospif(2.f * u2);
+  t = fminf(fmaxf(t + (fx.sigma0 + fx.sigma1 * t) * nrm, 0.f), fx.max_range);
+  return true;
+}
+
+constexpr int kFxThreads = 256, kFxItems = 4, kFxBlock = kFxThreads * kFxItems;
+
+// A block takes kFxBlock consecutive returns.  One thread finds the block's
+// first (environment, ray) with the 64-bit division; from there a return's
+// environment is a 32-bit division of its offset.  VEC: four consecutive
+// returns a thread in 16-byte accesses (both arrays 16-byte aligned).
+template <bool VEC>
+__global__ void __launch_bounds__(kFxThreads) k_effects(float* __restrict__ range, int32_t* __restrict__ tri,
+                                                        int64_t n, uint32_t n_rays, const Effects fx) {
+  __shared__ uint32_t s_env, s_ray;
+  const int64_t base = (int64_t)blockIdx.x * kFxBlock;
+  if (threadIdx.x == 0) {
+    const int64_t e = base / n_rays;
+    s_env = (uint32_t)fx.env_offset + (uint32_t)e;
+    s_ray = (uint32_t)(base - e * n_rays);
+  }
+  __syncthreads();
+  const uint32_t env0 = s_env, ray0 = s_ray;  // ray0 + kFxBlock < 2^32
+  const uint32_t left = n - base < kFxBlock ? (uint32_t)(n - base) : (uint32_t)kFxBlock;
+  uint32_t ray, env;  // of the return at hand
+  auto at = [&](uint32_t off) {
+    const uint32_t r = ray0 + off, de = r / n_rays;
+    ray = r - de * n_rays;
+    env = env0 + de;
+  };
+  auto next = [&](float& t, int32_t& id) {
+    const bool changed = apply(fx, ray, env, t, id);
+    if (++ray == n_rays) {
+      ray = 0;
+      ++env;
     }
-    if (sigma0 == 0.f && sigma1 == 0.f) continue;
-    const float u1 = (float)((x1 >> 8) + 1u) * inv24, u2 = (float)(x2 >> 8) * inv24;
-    const float nrm = sqrtf(-2.f * logf(u1)) * cospif(2.f * u2);
-    const float t = range[i];
-    const float tn = t + (sigma0 + sigma1 * t) * nrm;
-    range[i] = fminf(fmaxf(tn, 0.f), max_range);
+    return changed;
+  };
+  if (VEC) {
+    const uint32_t off = threadIdx.x * kFxItems;
+    if (off + kFxItems <= left) {
+      float4 t = *reinterpret_cast<const float4*>(range + base + off);
+      int4 id = *reinterpret_cast<const int4*>(tri + base + off);
+      const int4 id0 = id;
+      at(off);
+      const bool c0 = next(t.x, id.x), c1 = next(t.y, id.y), c2 = next(t.z, id.z), c3 = next(t.w, id.w);
+      if (c0 | c1 | c2 | c3) *reinterpret_cast<float4*>(range + base + off) = t;
+      if ((id.x ^ id0.x) | (id.y ^ id0.y) | (id.z ^ id0.z) | (id.w ^ id0.w))
+        *reinterpret_cast<int4*>(tri + base + off) = id;
+      return;
+    }
+    for (uint32_t o = off; o < left; ++o) {  // the last, partial four
+      float t = range[base + o];
+      int32_t id = tri[base + o];
+      const int32_t id0 = id;
+      at(o);
+      if (next(t, id)) range[base + o] = t;
+      if (id != id0) tri[base + o] = id;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < kFxItems; ++k) {
+      const uint32_t o = threadIdx.x + k * kFxThreads;
+      if (o >= left) break;
+      float t = range[base + o];
+      int32_t id = tri[base + o];
+      const int32_t id0 = id;
+      at(o);
+      if (next(t, id)) range[base + o] = t;
+      if (id != id0) tri[base + o] = id;
+    }
   }
 }
 
@@ -93,16 +165,16 @@ extern "C" fgl_status fgl_apply_sensor_effects(const fgl_sensor_effects* fx, flo
   const int64_t n = (int64_t)n_env * n_rays;
   if (n == 0) return FGL_OK;
   if (!range || !tri) return err(FGL_ERR_INVALID, "null range or tri");
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return err(FGL_ERR_CUDA, "cannot query the device");
-  const int64_t want = (n + 255) / 256;
-  const int grid = (int)(want < (int64_t)sms * 16 ? want : (int64_t)sms * 16);
-  k_effects<<<grid, 256, 0, (cudaStream_t)stream>>>(range, tri, n, n_rays, fx->env_offset, fx->step,
-                                                     (uint32_t)fx->seed, (uint32_t)(fx->seed >> 32),
-                                                     fx->drop_prob, fx->noise_sigma0, fx->noise_sigma1,
-                                                     fx->max_range);
+  const int64_t blocks = (n + kFxBlock - 1) / kFxBlock;
+  if (blocks > 0x7FFFFFFF) return err(FGL_ERR_INVALID, "too many returns (more than 2^41)");
+  Effects p{{}, fx->step, fx->env_offset, fx->drop_prob, fx->noise_sigma0, fx->noise_sigma1, fx->max_range};
+  for (uint32_t r = 0; r < 10; ++r) {
+    p.key.k0[r] = (uint32_t)fx->seed + r * 0x9E3779B9u;
+    p.key.k1[r] = (uint32_t)(fx->seed >> 32) + r * 0xBB67AE85u;
+  }
+  const bool vec = (((uintptr_t)range | (uintptr_t)tri) & 15u) == 0;
+  if (vec) k_effects<true><<<(unsigned)blocks, kFxThreads, 0, (cudaStream_t)stream>>>(range, tri, n, (uint32_t)n_rays, p);
+  else k_effects<false><<<(unsigned)blocks, kFxThreads, 0, (cudaStream_t)stream>>>(range, tri, n, (uint32_t)n_rays, p);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return err(FGL_ERR_CUDA, cudaGetErrorString(e));
   return FGL_OK;
