@@ -206,7 +206,9 @@ typedef struct {
                              read with fgl_work_counters */
   int32_t tri_mode;       /* leaf triangle tests: 0 = pooled across the warp
                              (default), 1 = each lane tests its own, postponing
-                             per postpone_pct */
+                             per postpone_pct.  Mode 0 with refill_min 32 also
+                             lets a warp walk the upper tree with 32 neighbouring
+                             rays together where the sensor's are close */
 } fgl_batch_opts;
 
 /* fgl_cast with explicit launch options: block_threads, stack_smem,
@@ -295,7 +297,8 @@ fgl_status fgl_work_counters(uint64_t* rays, uint64_t* node_visits, uint64_t* tr
  * iterations of the persistent kernel's main loop, [4] active lanes summed
  * over those iterations, [5] pooled leaf-test rounds (32 tests each at
  * most), [6] stack entries popped after the leaf tests, [7] ray packets
- * drawn by warps. */
+ * drawn by warps.  A node or triangle that a whole packet of rays visits
+ * together counts once for each of its rays (and one warp iteration or round). */
 fgl_status fgl_work_phase_counters(uint64_t* out, int32_t n);
 
 /* Optional sensor effects on cast returns, applied in place after a cast

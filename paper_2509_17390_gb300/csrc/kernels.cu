@@ -8,6 +8,10 @@
 //                  hands fresh rays to lanes whose ray has finished once
 //                  enough lanes are idle, so warps stay full while the
 //                  per-ray work (eq. cost(r_j)) varies.
+//   k_plain_packets, k_packets : the same two for sensors of narrow packets
+//                  (32 neighbouring rays of one environment): a warp walks
+//                  the upper tree with all its rays together (packet_phase in
+//                  trace.cuh) and only what is left ray by ray.
 //   k_world_rays : debug export of the float32 rays of eq. r_j.
 //   k_l2_read    : bandwidth probe, 16-byte L2 reads of a resident buffer.
 #include <cuda_runtime.h>
@@ -297,6 +301,144 @@ __global__ void __maxnreg__(TMIN ? 72 : 64) k_persistent(BatchHeader* __restrict
   }
 }
 
+// Shared memory of the packet kernels: that of the traversal, then one list
+// slot (8 B) and one pending word a thread.
+__device__ __forceinline__ dev::PacketList packet_smem(int W, int sdepth) {
+  extern __shared__ __align__(16) unsigned long long smem_u64[];
+  uint2* list = reinterpret_cast<uint2*>(reinterpret_cast<char*>(smem_u64) +
+                                         (size_t)blockDim.x * (8 + (size_t)sdepth * (8 + 2 * W)));
+  return dev::PacketList{list + (threadIdx.x & ~31u), reinterpret_cast<uint32_t*>(list + blockDim.x) + threadIdx.x};
+}
+
+// One packet: up to 32 consecutive rays (tile order) of one environment of an
+// item, by one warp.  The packet phase walks the tree for all of them; the
+// per-ray traversal takes what it leaves.
+template <int W, bool COUNT, bool TMIN>
+__device__ __forceinline__ void trace_packet(const ItemDesc& it, int env, int first, int n, const Smem<W>& sm,
+                                             const dev::PacketList& pl,
+                                             const dev::StackRefs<typename dev::KeyWords<W>::T>& st,
+                                             uint32_t (&c)[kWorkCounters]) {
+  const unsigned FULL = 0xFFFFFFFFu;
+  const int lane = threadIdx.x & 31;
+  const bool live = lane < n;  // a lane past the end copies the first ray (and neither traces alone nor stores)
+  const float4 ds = __ldg((const float4*)it.dirs + first + (live ? lane : 0));
+  const int64_t o = (int64_t)env * it.n_rays + __float_as_int(ds.w);
+  dev::Tracer<W, COUNT, TMIN> tr;
+  dev::PacketEnd end;
+  {
+    float ox, oy, oz, dx, dy, dz;
+    dev::world_ray(it.poses + 12 * (int64_t)env, ds, ox, oy, oz, dx, dy, dz);
+    dev::setup_ray(tr.r, ox, oy, oz, dx, dy, dz);
+    tr.start(it.nodes, it.tris, it.min_range, it.max_range, it.n_nodes, it.n_tris);
+    if (COUNT) tr.n_rounds = tr.n_pops = 0;
+    end = dev::packet_phase(tr, dx, dy, dz, pl, lane, live, &g_status, c[3], c[4]);
+  }
+  if (end != dev::kPacketDone) {
+    bool active = live && (end == dev::kPacketNone || tr.next_entry(pl));
+    while (__any_sync(FULL, active)) {
+      if (COUNT) {
+        c[3] += lane == 0 ? 1u : 0u;
+        c[4] += active ? 1u : 0u;
+      }
+      bool ok = true;
+      if (active) ok = tr.descend(st);
+      dev::tri_phase_warp(tr, sm.keys, lane, &g_status);
+      if (active) {
+        if (!ok) {
+          atomicOr(&g_status, tr.fail_bits());
+          active = false;
+        } else {
+          active = !tr.template finish_pooled<true>(st, pl);
+        }
+      }
+    }
+  }
+  if (live) {
+    float rg;
+    int32_t id;
+    tr.result(rg, id);
+    __stcs(it.out_range + o, rg);  // evict-first: the results do not push the BVH out of L2
+    __stcs(it.out_tri + o, id);
+  }
+  if (COUNT) {
+    c[0] += live ? 1u : 0u;
+    c[1] += tr.n_nodes;
+    c[2] += tr.n_tris;
+    c[5] += tr.n_rounds;
+    c[6] += tr.n_pops;
+  }
+}
+
+// k_plain with packet phases: warp w of the grid takes packet w of the item.
+template <int W, bool COUNT>
+__global__ void __maxnreg__(72) k_plain_packets(const ItemDesc it, int sdepth) {
+  using Keys = typename dev::KeyWords<W>::T;
+  if (it.width != W) {  // never read nodes laid out for another width
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&g_status, 2u);
+    return;
+  }
+  const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int env = (p >> 32) ? (int)(p / it.pk_per_env) : (int)((uint32_t)p / (uint32_t)it.pk_per_env);
+  if (env >= it.n_env) return;
+  const int first = (int)(p - (int64_t)env * it.pk_per_env) * 32;
+  const Smem<W> sm = smem_layout<W>(sdepth);
+  uint2 ls[kStackLocal];
+  Keys lq[kStackLocal];
+  const dev::StackRefs<Keys> st{sm.ss, sm.sq, ls, lq, (int)blockDim.x, sdepth};
+  uint32_t c[kWorkCounters] = {};
+  trace_packet<W, COUNT, false>(it, env, first, min(32, it.n_rays - first), sm, packet_smem(W, sdepth), st, c);
+  flush_counters<COUNT>(c);
+}
+
+// k_persistent with packet phases: a warp draws packets of the queue and takes
+// the rays of each 32 at a time.  Bound, like k_persistent, by instruction
+// issue (0.70-0.73 of it), but with 148 instead of 224 warp instructions a ray:
+// 4096 x 5760 rays on 1 M triangles of a cluttered room 4.91 -> 3.65 ms, a fleet
+// of dense sensors on 3 cm triangles 1.86 -> 1.68 ms, one 57,600-ray scan 54 ->
+// 45 us.  Under the 72-register cap 88 bytes a thread spill; 64 (more spills)
+// and 80 (fewer warps) are 1-4% slower, and sharing the loop with k_persistent's
+// refill of partly idle warps keeps so much alive that most of the gain is lost.
+template <int W, bool COUNT, bool TMIN>
+__global__ void __maxnreg__(72) k_packets(BatchHeader* __restrict__ hdr, const ItemDesc* __restrict__ items,
+                                           int sdepth) {
+  using Keys = typename dev::KeyWords<W>::T;
+  const unsigned FULL = 0xFFFFFFFFu;
+  const int lane = threadIdx.x & 31;
+  const Smem<W> sm = smem_layout<W>(sdepth);
+  const dev::PacketList pl = packet_smem(W, sdepth);
+  uint2 ls[kStackLocal];
+  Keys lq[kStackLocal];
+  const dev::StackRefs<Keys> st{sm.ss, sm.sq, ls, lq, (int)blockDim.x, sdepth};
+  uint32_t c[kWorkCounters] = {};
+  for (;;) {
+    unsigned long long p = 0;
+    if (lane == 0) p = atomicAdd(&hdr->head, 1ull);
+    p = __shfl_sync(FULL, p, 0);
+    if ((int64_t)p >= hdr->n_packets) break;
+    int lo = 0, hi = hdr->n_items - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (items[mid].pk_begin <= (int64_t)p) lo = mid;
+      else hi = mid - 1;
+    }
+    const ItemDesc& it = items[lo];
+    if (COUNT && lane == 0) ++c[7];
+    if (it.width != W) {  // never read nodes laid out for another width
+      if (lane == 0) atomicOr(&g_status, 2u);
+      continue;
+    }
+    const int64_t local = (int64_t)p - it.pk_begin;
+    const int ppe = it.pk_per_env;
+    const int env = (local >> 32) ? (int)(local / ppe) : (int)((uint32_t)local / (uint32_t)ppe);
+    const int P = hdr->packet_rays;
+    int first = (int)(local - (int64_t)env * ppe) * P;
+    const int end = min(first + P, it.n_rays);
+    for (; first < end; first += 32)
+      trace_packet<W, COUNT, TMIN>(it, env, first, min(32, end - first), sm, pl, st, c);
+  }
+  flush_counters<COUNT>(c);
+}
+
 // Second pass over one item for instance k: every ray, moved into the
 // instance's frame by the inverse of its rigid pose (the float32 sequence of
 // fgl.h), is cast against the instance's BVH, pruned by the return found so
@@ -541,6 +683,19 @@ __global__ void k_world_rays(const float4* __restrict__ dirs, const float* __res
   out_d[o + 2] = dz;
 }
 
+template <int W, bool COUNT, bool TMIN>
+void* packets_fn() {
+  return (void*)k_packets<W, COUNT, TMIN>;
+}
+template <int W>
+void* pick_packets_w(bool count, bool tmin) {
+  if (tmin) return count ? packets_fn<W, true, true>() : packets_fn<W, false, true>();
+  return count ? packets_fn<W, true, false>() : packets_fn<W, false, false>();
+}
+void* pick_packets(int W, bool count, bool tmin) {
+  return W == 8 ? pick_packets_w<8>(count, tmin) : pick_packets_w<4>(count, tmin);
+}
+
 template <int W, bool COUNT>
 void* plain_fn() {
   return (void*)k_plain<W, COUNT>;
@@ -570,40 +725,65 @@ size_t stack_smem_bytes(int W, int block, int sdepth) {
          (size_t)block * (size_t)sdepth * (sizeof(uint2) + 2 * (size_t)W);
 }
 
-cudaError_t launch_plain(int W, bool count, const ItemDesc& it, int block, int sdepth,
+static size_t packets_smem_bytes(int W, int block, int sdepth) {
+  return stack_smem_bytes(W, block, sdepth) + (size_t)block * (sizeof(uint2) + sizeof(uint32_t));
+}
+
+bool packets_fit(int W, int block, int sdepth) {
+  int dev = 0, optin = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+    return false;
+  return packets_smem_bytes(W, block, sdepth) <= (size_t)optin;
+}
+
+static cudaError_t allow_smem(void* fn, size_t smem) {
+  if (smem <= 48 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
+cudaError_t launch_plain(int W, bool count, bool packets, const ItemDesc& it, int block, int sdepth,
                          int tri_mode, int postpone_pct, cudaStream_t s) {
   const int64_t total = (int64_t)it.n_env * it.n_rays;
   if (total == 0) return cudaSuccess;
+  ItemDesc arg = it;
+  if (packets) {
+    arg.pk_per_env = (it.n_rays + 31) / 32;
+    const int64_t warps = (int64_t)it.n_env * arg.pk_per_env;
+    const int64_t grid = (warps * 32 + block - 1) / block;
+    const size_t smem = packets_smem_bytes(W, block, sdepth);
+    void* fn = W == 8 ? (count ? (void*)k_plain_packets<8, true> : (void*)k_plain_packets<8, false>)
+                      : (count ? (void*)k_plain_packets<4, true> : (void*)k_plain_packets<4, false>);
+    const cudaError_t e = allow_smem(fn, smem);
+    if (e != cudaSuccess) return e;
+    void* args[] = {&arg, &sdepth};
+    return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(block), args, smem, s);
+  }
   const int64_t grid = (total + block - 1) / block;
   const size_t smem = stack_smem_bytes(W, block, sdepth);
   void* fn = pick_plain(W, count);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  ItemDesc arg = it;
+  const cudaError_t e = allow_smem(fn, smem);
+  if (e != cudaSuccess) return e;
   void* args[] = {&arg, &sdepth, &tri_mode, &postpone_pct};
   return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(block), args, smem, s);
 }
 
-int persistent_blocks_per_sm(int W, bool count, bool tmin, int block, int sdepth) {
-  void* fn = pick_persistent(W, count, tmin);
-  const size_t smem = stack_smem_bytes(W, block, sdepth);
-  if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+int persistent_blocks_per_sm(int W, bool count, bool tmin, bool packets, int block, int sdepth) {
+  void* fn = packets ? pick_packets(W, count, tmin) : pick_persistent(W, count, tmin);
+  const size_t smem = packets ? packets_smem_bytes(W, block, sdepth) : stack_smem_bytes(W, block, sdepth);
+  allow_smem(fn, smem);
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, block, smem) != cudaSuccess) return 1;
   return n > 0 ? n : 1;
 }
 
-cudaError_t launch_persistent(int W, bool count, bool tmin, void* scratch, int grid, int block,
+cudaError_t launch_persistent(int W, bool count, bool tmin, bool packets, void* scratch, int grid, int block,
                               int sdepth, int refill_min, int tri_mode, int postpone_pct,
                               cudaStream_t s) {
-  void* fn = pick_persistent(W, count, tmin);
-  const size_t smem = stack_smem_bytes(W, block, sdepth);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  void* fn = packets ? pick_packets(W, count, tmin) : pick_persistent(W, count, tmin);
+  const size_t smem = packets ? packets_smem_bytes(W, block, sdepth) : stack_smem_bytes(W, block, sdepth);
+  const cudaError_t e = allow_smem(fn, smem);
+  if (e != cudaSuccess) return e;
   BatchHeader* hdr = (BatchHeader*)scratch;
   const ItemDesc* items = (const ItemDesc*)((char*)scratch + sizeof(BatchHeader));
   void* args[] = {&hdr, &items, &sdepth, &refill_min, &tri_mode, &postpone_pct};

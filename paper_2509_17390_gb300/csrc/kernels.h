@@ -14,17 +14,25 @@ size_t stack_smem_bytes(int W, int block, int sdepth);
 
 // One thread per ray of one item (grid = ceil(n_env * n_rays / block)).
 // tri_mode 0: warp-pooled leaf tests; 1: lane-serial with postponing.
-cudaError_t launch_plain(int W, bool count, const ItemDesc& it, int block, int sdepth,
+// packets: one packet of 32 rays of an environment a warp, walked together
+// before the per-ray traversal (needs tri_mode 0; see packets_fit).
+cudaError_t launch_plain(int W, bool count, bool packets, const ItemDesc& it, int block, int sdepth,
                          int tri_mode, int postpone_pct, cudaStream_t s);
 
+// Whether a block of this shape has room for the packet lists beside its
+// stacks (large blocks with deep shared stacks do not).
+bool packets_fit(int W, int block, int sdepth);
+
 // Resident blocks per SM of the persistent kernel for this configuration.
-int persistent_blocks_per_sm(int W, bool count, bool tmin, int block, int sdepth);
+int persistent_blocks_per_sm(int W, bool count, bool tmin, bool packets, int block, int sdepth);
 
 // Persistent kernel over the work queue in `scratch`: a BatchHeader
 // followed by n_items ItemDesc records (device memory).  tmin selects the
 // instantiation that honours ItemDesc::min_range (needed when any item of
-// the group has min_range > 0; otherwise min_range is taken as 0).
-cudaError_t launch_persistent(int W, bool count, bool tmin, void* scratch, int grid, int block,
+// the group has min_range > 0; otherwise min_range is taken as 0).  packets
+// selects the kernel whose warps walk whole packets together (the group's
+// sensors have narrow packets, tri_mode 0, refill 32).
+cudaError_t launch_persistent(int W, bool count, bool tmin, bool packets, void* scratch, int grid, int block,
                               int sdepth, int refill_min, int tri_mode, int postpone_pct,
                               cudaStream_t s);
 

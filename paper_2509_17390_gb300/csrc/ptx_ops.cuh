@@ -63,6 +63,19 @@ __device__ __forceinline__ uint32_t prmt_sign(uint32_t x, uint32_t sel) {
   return r;
 }
 
+// Minimum / maximum of a float over the 32 lanes of a full warp (NaN lanes are
+// passed over).
+__device__ __forceinline__ float redux_minf(float x) {
+  float r;
+  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float redux_maxf(float x) {
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // Packed pair of floats (lo, hi) in one 64-bit register pair.
 __device__ __forceinline__ uint64_t pack2f(float lo, float hi) {
   uint64_t r;

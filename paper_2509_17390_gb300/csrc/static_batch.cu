@@ -28,7 +28,7 @@
 namespace fgl {
 // Allocation-free item check + descriptor fill, and launch-option defaults and
 // checks (api.cu); both return a constant message, or nullptr when valid.
-const char* static_item_desc(const fgl_cast_item& it, ItemDesc* d, int* width);
+const char* static_item_desc(const fgl_cast_item& it, ItemDesc* d, int* width, bool* narrow);
 const char* launch_opts(const fgl_batch_opts* o, int* packet, int* block, int* sdepth, int* bpsm,
                         int* graph, int* refill, int* postpone, int* count, int* tri_mode);
 }  // namespace fgl
@@ -118,18 +118,20 @@ extern "C" fgl_status fgl_cast_batched_static(const fgl_cast_item* items, int32_
   // into the image
   ItemDesc descs[kStaticMaxItems];
   int widths[kStaticMaxItems];
+  bool narrow[kStaticMaxItems];
   for (int i = 0; i < n_items; ++i) {
-    const char* msg = static_item_desc(items[i], &descs[i], &widths[i]);
+    const char* msg = static_item_desc(items[i], &descs[i], &widths[i], &narrow[i]);
     if (msg) return err(FGL_ERR_INVALID, msg);
   }
   StaticImage img;
   img.n_words = 0;
-  size_t group_off[kMaxGroups] = {0, 0};
-  int group_w[kMaxGroups] = {0, 0};
-  bool group_tmin[kMaxGroups] = {false, false};
+  size_t group_off[kMaxGroups] = {};
+  int group_w[kMaxGroups] = {};
+  bool group_tmin[kMaxGroups] = {}, group_packets[kMaxGroups] = {};
   int n_groups = 0;
   size_t used = 0;
   for (int W : {8, 4}) {
+    int64_t together = 0;  // packets of narrow sensors less those of the others, as for fgl_cast_batched
     BatchHeader h;
     std::memset(&h, 0, sizeof(h));
     const size_t hdr_off = used;
@@ -140,6 +142,8 @@ extern "C" fgl_status fgl_cast_batched_static(const fgl_cast_item* items, int32_
     for (int i = 0; i < n_items; ++i) {
       ItemDesc d = descs[i];
       if (widths[i] != W || d.n_env == 0) continue;
+      const int64_t warps = (int64_t)d.n_env * ((d.n_rays + 31) / 32);
+      together += narrow[i] ? warps : -warps;
       d.pk_per_env = (d.n_rays + packet - 1) / packet;
       d.pk_begin = packets;
       packets += (int64_t)d.pk_per_env * d.n_env;
@@ -157,6 +161,7 @@ extern "C" fgl_status fgl_cast_batched_static(const fgl_cast_item* items, int32_
     group_off[n_groups] = hdr_off;
     group_w[n_groups] = W;
     group_tmin[n_groups] = tmin;
+    group_packets[n_groups] = together >= 0 && tri_mode == 0 && refill == 32 && packets_fit(W, block, sdepth);
     ++n_groups;
     used = off;
   }
@@ -180,9 +185,9 @@ extern "C" fgl_status fgl_cast_batched_static(const fgl_cast_item* items, int32_
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_err(e);
   for (int g = 0; g < n_groups; ++g) {
     const int per_sm =
-        bpsm ? bpsm : persistent_blocks_per_sm(group_w[g], count != 0, group_tmin[g], block, sdepth);
+        bpsm ? bpsm : persistent_blocks_per_sm(group_w[g], count != 0, group_tmin[g], group_packets[g], block, sdepth);
     const int grid = (sms > 0 ? sms : 1) * (per_sm > 0 ? per_sm : 1);
-    e = launch_persistent(group_w[g], count != 0, group_tmin[g], (char*)scratch + group_off[g], grid, block,
+    e = launch_persistent(group_w[g], count != 0, group_tmin[g], group_packets[g], (char*)scratch + group_off[g], grid, block,
                           sdepth, refill, tri_mode, postpone, s);
     if (e != cudaSuccess) return cuda_err(e);
   }

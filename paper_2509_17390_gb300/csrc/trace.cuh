@@ -91,6 +91,63 @@ __device__ __forceinline__ void setup_ray(Ray& r, float ox, float oy, float oz, 
   r.Sy = __fmul_rn(sel3(dx, dy, dz, ky), r.Sz);
 }
 
+// The three edge functions in float64 (products of two floats are exact
+// there; one rounding per difference).
+static __device__ __noinline__ float3 edges64(float Ax, float Ay, float Bx, float By, float Cx, float Cy) {
+  return make_float3((float)((double)Cx * (double)By - (double)Cy * (double)Bx),
+                     (float)((double)Ax * (double)Cy - (double)Ay * (double)Cx),
+                     (float)((double)Bx * (double)Ay - (double)By * (double)Ax));
+}
+
+// The test from the translated vertices in the ray's axes: (X, Y, Z) of each
+// vertex are its kx, ky, kz coordinates minus the origin's.
+template <bool kAll>
+__device__ __forceinline__ float tri_hit_axes(const Ray& r, float AX, float AY, float Akz, float BX, float BY,
+                                              float Bkz, float CX, float CY, float Ckz, float tbest) {
+  float Ax = __fsub_rn(AX, __fmul_rn(r.Sx, Akz));
+  float Ay = __fsub_rn(AY, __fmul_rn(r.Sy, Akz));
+  float Bx = __fsub_rn(BX, __fmul_rn(r.Sx, Bkz));
+  float By = __fsub_rn(BY, __fmul_rn(r.Sy, Bkz));
+  float Cx = __fsub_rn(CX, __fmul_rn(r.Sx, Ckz));
+  float Cy = __fsub_rn(CY, __fmul_rn(r.Sy, Ckz));
+  float U = __fsub_rn(__fmul_rn(Cx, By), __fmul_rn(Cy, Bx));
+  float V = __fsub_rn(__fmul_rn(Ax, Cy), __fmul_rn(Ay, Cx));
+  float W = __fsub_rn(__fmul_rn(Bx, Ay), __fmul_rn(By, Ax));
+  const bool zero = U == 0.f || V == 0.f || W == 0.f;
+  if (kAll) {
+    // In a loop that all lanes run together the compiler turns the rare
+    // float64 fallback into predicated work of every test (it kept this chip's
+    // small float64 pipe 86% busy); behind a call it stays a branch.
+    if (__any_sync(0xFFFFFFFFu, zero)) {
+      const float3 e = edges64(Ax, Ay, Bx, By, Cx, Cy);
+      if (zero) {
+        U = e.x;
+        V = e.y;
+        W = e.z;
+      }
+    }
+  } else if (zero) {
+    // products of two floats are exact in double; one rounding per difference
+    double u = (double)Cx * (double)By - (double)Cy * (double)Bx;
+    double v = (double)Ax * (double)Cy - (double)Ay * (double)Cx;
+    double w = (double)Bx * (double)Ay - (double)By * (double)Ax;
+    U = (float)u;
+    V = (float)v;
+    W = (float)w;
+  }
+  const bool miss = (U < 0.f || V < 0.f || W < 0.f) && (U > 0.f || V > 0.f || W > 0.f);
+  if (kAll ? __all_sync(0xFFFFFFFFu, miss) : miss) return -1.f;
+  float det = __fadd_rn(__fadd_rn(U, V), W);
+  float Az = __fmul_rn(r.Sz, Akz), Bz = __fmul_rn(r.Sz, Bkz), Cz = __fmul_rn(r.Sz, Ckz);
+  float T = __fadd_rn(__fadd_rn(__fmul_rn(U, Az), __fmul_rn(V, Bz)), __fmul_rn(W, Cz));
+  // t = T/det must be > 0: same sign, T != 0; certainly beyond tbest:
+  // |T| > tbest*|det|*(1+2^-20) implies fl(T/det) > tbest
+  const bool off = miss || det == 0.f || ((__float_as_uint(T) ^ __float_as_uint(det)) >> 31) || T == 0.f ||
+                   fabsf(T) > __fmul_rn(__fmul_rn(tbest, fabsf(det)), 1.00000095367431640625f);
+  if (off) return -1.f;
+  return __fdiv_rn(T, det);
+}
+
 // Watertight float32 ray/triangle test (Woop, Benthin & Wald 2013, JCGT 2(1)):
 // translate the vertices to the ray origin, shear so the ray is the +z axis
 // of the (kx, ky, kz) frame, and take the signs of the three 2D edge
@@ -102,35 +159,9 @@ __device__ __forceinline__ float tri_hit(const Ray& r, float4 a, float4 b, float
   float A0 = __fsub_rn(a.x, r.ox), A1 = __fsub_rn(a.y, r.oy), A2 = __fsub_rn(a.z, r.oz);
   float B0 = __fsub_rn(b.x, r.ox), B1 = __fsub_rn(b.y, r.oy), B2 = __fsub_rn(b.z, r.oz);
   float C0 = __fsub_rn(c.x, r.ox), C1 = __fsub_rn(c.y, r.oy), C2 = __fsub_rn(c.z, r.oz);
-  float Akz = sel3(A0, A1, A2, kz), Bkz = sel3(B0, B1, B2, kz), Ckz = sel3(C0, C1, C2, kz);
-  float Ax = __fsub_rn(sel3(A0, A1, A2, kx), __fmul_rn(r.Sx, Akz));
-  float Ay = __fsub_rn(sel3(A0, A1, A2, ky), __fmul_rn(r.Sy, Akz));
-  float Bx = __fsub_rn(sel3(B0, B1, B2, kx), __fmul_rn(r.Sx, Bkz));
-  float By = __fsub_rn(sel3(B0, B1, B2, ky), __fmul_rn(r.Sy, Bkz));
-  float Cx = __fsub_rn(sel3(C0, C1, C2, kx), __fmul_rn(r.Sx, Ckz));
-  float Cy = __fsub_rn(sel3(C0, C1, C2, ky), __fmul_rn(r.Sy, Ckz));
-  float U = __fsub_rn(__fmul_rn(Cx, By), __fmul_rn(Cy, Bx));
-  float V = __fsub_rn(__fmul_rn(Ax, Cy), __fmul_rn(Ay, Cx));
-  float W = __fsub_rn(__fmul_rn(Bx, Ay), __fmul_rn(By, Ax));
-  if (U == 0.f || V == 0.f || W == 0.f) {
-    // products of two floats are exact in double; one rounding per difference
-    double u = (double)Cx * (double)By - (double)Cy * (double)Bx;
-    double v = (double)Ax * (double)Cy - (double)Ay * (double)Cx;
-    double w = (double)Bx * (double)Ay - (double)By * (double)Ax;
-    U = (float)u;
-    V = (float)v;
-    W = (float)w;
-  }
-  if ((U < 0.f || V < 0.f || W < 0.f) && (U > 0.f || V > 0.f || W > 0.f)) return -1.f;
-  float det = __fadd_rn(__fadd_rn(U, V), W);
-  if (det == 0.f) return -1.f;
-  float Az = __fmul_rn(r.Sz, Akz), Bz = __fmul_rn(r.Sz, Bkz), Cz = __fmul_rn(r.Sz, Ckz);
-  float T = __fadd_rn(__fadd_rn(__fmul_rn(U, Az), __fmul_rn(V, Bz)), __fmul_rn(W, Cz));
-  // t = T/det must be > 0: same sign, T != 0
-  if (((__float_as_uint(T) ^ __float_as_uint(det)) >> 31) || T == 0.f) return -1.f;
-  // certainly beyond tbest: |T| > tbest*|det|*(1+2^-20) implies fl(T/det) > tbest
-  if (fabsf(T) > __fmul_rn(__fmul_rn(tbest, fabsf(det)), 1.00000095367431640625f)) return -1.f;
-  return __fdiv_rn(T, det);
+  return tri_hit_axes<false>(r, sel3(A0, A1, A2, kx), sel3(A0, A1, A2, ky), sel3(A0, A1, A2, kz), sel3(B0, B1, B2, kx),
+                      sel3(B0, B1, B2, ky), sel3(B0, B1, B2, kz), sel3(C0, C1, C2, kx), sel3(C0, C1, C2, ky),
+                      sel3(C0, C1, C2, kz), tbest);
 }
 
 // Child keys of a node group: one 16-bit key per child slot, two per 32-bit
@@ -290,6 +321,14 @@ struct StackRefs {
   int sdepth;
 };
 
+// The subtrees a packet phase (below) left to its rays: `entry` points at the
+// warp's 32 shared-memory slots (entry distance bits, node), ascending, and
+// `pend` at the lane's own word of slots its ray still has to visit.
+struct PacketList {
+  uint2* entry;
+  uint32_t* pend;
+};
+
 // TMIN: the rays may have a minimum range t_min > 0 (eq. t_j*: hits nearer
 // than it are discarded); without it t_min is the constant 0 and costs no
 // register.
@@ -441,15 +480,34 @@ struct Tracer {
 
   // finish() for the pooled leaf tests, where the stack holds node groups
   // only (no postponed triangle groups), so a popped group needs no type test.
-  __device__ __forceinline__ bool finish_pooled(const StackRefs<Keys>& st) {
+  // LIST: an empty stack moves on to the next subtree the packet phase left.
+  template <bool LIST = false>
+  __device__ __forceinline__ bool finish_pooled(const StackRefs<Keys>& st, const PacketList& pl = PacketList{}) {
     if (ng.y & kGroupPending) return false;
     const uint32_t hb = half_rp(best_t);
     for (;;) {
-      if (sp == 0) return true;
+      if (sp == 0) return LIST ? !next_entry(pl) : true;
       pop(st);
       if (COUNT) ++n_pops;
       if ((key_min(kq) & (0xFFFFu ^ (W - 1))) <= hb) return false;
     }
+  }
+
+  // Make the lane's next subtree of the packet list the current node group;
+  // false when none is left that could hold a nearer hit.  The list ascends
+  // in entry distance, so the first entry beyond the best hit ends it.
+  __device__ __forceinline__ bool next_entry(const PacketList& pl) {
+    const uint32_t pend = *pl.pend;
+    if (pend == 0u) return false;
+    const uint2 e = pl.entry[__ffs(pend) - 1];
+    if (__uint_as_float(e.x) > best_t) return false;
+    *pl.pend = pend & (pend - 1u);
+    ng = make_uint2(e.y, kGroupPending | 1u);
+    tg = make_uint2(0u, 0u);
+    kq.x = 0xFFFF0000u;
+    kq.y = 0xFFFFFFFFu;
+    if constexpr (W == 8) kq.z = kq.w = 0xFFFFFFFFu;
+    return true;
   }
 
   // After the leaf tests: once the current node group has no pending child,
@@ -596,6 +654,236 @@ __device__ __forceinline__ void tri_phase_warp(Tracer<W, COUNT, TMIN>& tr, unsig
     tr.best_id = (int32_t)(uint32_t)k;
   }
   tr.tg.y = 0;
+}
+
+// ---------------------------------------------------------------------------
+// packet phase: the rays of one warp share their origin (one environment), so
+// the upper part of the tree is walked once for all of them
+// ---------------------------------------------------------------------------
+constexpr uint32_t kNoEntry = 0xFFFFFFFFu;
+constexpr uint32_t kSmallNode = 0x80000000u;  // node indexes stay below 2^31 (node arrays below 512 GB)
+
+// A packet whose rays spread over more than this tangent (about 35 degrees)
+// is left to the per-ray traversal: a 4 x 8 tile of 2 x 1 degree beams spreads
+// over 0.12, consecutive rays of a rosette over 1.3, where the phase costs 3-7%
+// and finishes nothing.
+constexpr float kPacketMaxSpread = 0.7f;
+// A node goes to the per-ray traversal once its box is narrower than this
+// many widths of the packet at the box's distance: few of the rays meet it then.
+// (1.0 / 1.5 / 2.5 / 4: a 4096 x 5760 step 2.01 / 1.95 / 1.94 / 1.99 ms for half
+// of it, a 57,600-ray scan 60 / 52 / 46 / 46 us.)
+constexpr float kPacketWidths = 2.5f;
+
+enum PacketEnd { kPacketNone = 0, kPacketDone = 1, kPacketEntries = 2 };
+
+// Walks the tree best first with the packet's frustum and tests every leaf
+// triangle it meets against all 32 rays.  The frustum is a rectangle in the
+// plane z = 1 of the dominant axis: a0 <= x / z <= a1, b0 <= y / z <= b1 over
+// all rays (widened far beyond float32 rounding), so a box needs four
+// compares against two scaled coordinates each.  The two nearest nodes are
+// opened together: lane W g + c tests child c of node g.  The boxes still to
+// visit sit one a lane (distance bits with the slot in the low 3, node,
+// parent), and a warp minimum picks the nearest.
+//
+// Every box test here is conservative for each ray of the packet, the
+// triangle test and the (t, id) rule are the per-ray ones, and what is left
+// goes to the per-ray traversal, so results do not depend on the phase.
+//
+// Ends with every ray finished (kPacketDone), or -- at the first node that is
+// small against the packet, or when the lanes run out of room -- with the
+// boxes left in the list in ascending distance and each lane's word of the
+// ones its own ray meets (kPacketEntries), or without having started because
+// the rays spread too far (kPacketNone).  All 32 lanes call it; a lane
+// without a ray of its own carries a copy of another lane's (live = false).
+template <int W, bool COUNT, bool TMIN>
+__device__ __forceinline__ PacketEnd packet_phase(Tracer<W, COUNT, TMIN>& tr, float dx, float dy, float dz,
+                                                  const PacketList& pl, int lane, bool live, unsigned* status,
+                                                  uint32_t& c_iters, uint32_t& c_lane_iters) {
+  const unsigned FULL = 0xFFFFFFFFu;
+  uint32_t* parents = pl.pend - lane;  // the pending words carry parents until the end
+  *pl.pend = 0u;
+  // dominant axis of a ray in the middle of the packet
+  const float mx = fabsf(__shfl_sync(FULL, dx, 12)), my = fabsf(__shfl_sync(FULL, dy, 12)),
+              mz = fabsf(__shfl_sync(FULL, dz, 12));
+  const uint32_t kz = mx >= my ? (mx >= mz ? 0u : 2u) : (my >= mz ? 1u : 2u);
+  const uint32_t kx = kz == 2u ? 0u : kz + 1u, ky = kx == 2u ? 0u : kx + 1u;
+  const float dzk = sel3(dx, dy, dz, kz);
+  const float sg = __shfl_sync(FULL, dzk, 12) < 0.f ? -1.f : 1.f;
+  const float w = dzk * sg, u = sel3(dx, dy, dz, kx), v = sel3(dx, dy, dz, ky);
+  if (!__all_sync(FULL, w > 0.05f)) return kPacketNone;
+  const float rw = 1.f / w;
+  float a0 = redux_minf(u * rw), a1 = redux_maxf(u * rw), b0 = redux_minf(v * rw), b1 = redux_maxf(v * rw);
+  const float spread = fmaxf(a1 - a0, b1 - b0);
+  if (!(spread <= kPacketMaxSpread)) return kPacketNone;
+  constexpr float kSlack = 2e-5f;
+  a0 -= kSlack * (1.f + fabsf(a0));
+  a1 += kSlack * (1.f + fabsf(a1));
+  b0 -= kSlack * (1.f + fabsf(b0));
+  b1 += kSlack * (1.f + fabsf(b1));
+  const float narrow = kPacketWidths * spread;
+  // t >= z / max w, and along x (y): t >= X0 / max u for a box in front,
+  // t >= -X1 / max(-u) for one behind; 0 where no ray goes that way
+  constexpr float kUnder = 0.99999f;
+  auto under = [&](float m) { return m > 1e-20f ? kUnder * rcp_approx(m) : 0.f; };
+  const float iz = under(redux_maxf(w)), ixp = under(redux_maxf(u)), ixn = -under(redux_maxf(-u)),
+              iyp = under(redux_maxf(v)), iyn = -under(redux_maxf(-v));
+  const float oX = sel3(tr.r.ox, tr.r.oy, tr.r.oz, kx), oY = sel3(tr.r.ox, tr.r.oy, tr.r.oz, ky),
+              oZ = sel3(tr.r.ox, tr.r.oy, tr.r.oz, kz);
+  const int c = lane & (W - 1);
+  // this lane's plane words of a node record (in floats): x, y, near and far z
+  const uint32_t fx = 8 + W * kx + c, fy = 8 + W * ky + c, fz = 8 + W * kz + c;
+  const uint32_t fzn = fz + (sg > 0.f ? 0 : 3 * W), fzf = fz + (sg > 0.f ? 3 * W : 0);
+  const unsigned lt = (1u << lane) - 1u;
+  // the triangle test's own axes of this lane's ray
+  const uint32_t tkx = tr.r.k & 3u, tky = (tr.r.k >> 2) & 3u, tkz = (tr.r.k >> 4) & 3u;
+  const float toX = sel3(tr.r.ox, tr.r.oy, tr.r.oz, tkx), toY = sel3(tr.r.ox, tr.r.oy, tr.r.oz, tky),
+              toZ = sel3(tr.r.ox, tr.r.oy, tr.r.oz, tkz);
+
+  uint32_t tkey = __float_as_uint(tr.best_t) | 7u;  // the farthest best hit of the packet, as a key
+  uint32_t fkey = lane == 0 ? 0u : kNoEntry, fnode = 0u, fpar = 0u;
+  int live_n = 1;  // boxes waiting
+  for (;;) {
+    const uint32_t m0 = __reduce_min_sync(FULL, fkey);
+    if (m0 > tkey) return kPacketDone;
+    const unsigned own0 = __ballot_sync(FULL, fkey == m0);
+    int src = __ffs(own0) - 1;
+    const bool last = live_n > 32 - W || (__shfl_sync(FULL, fnode, src) & kSmallNode);
+    if (last) break;
+    if (lane == src) fkey = kNoEntry;
+    --live_n;
+    bool use = lane < W;
+    if (live_n <= 32 - 2 * W) {  // room for the children of two nodes
+      const uint32_t m1 = __reduce_min_sync(FULL, fkey);
+      if (m1 <= tkey) {
+        const int s1 = __ffs(__ballot_sync(FULL, fkey == m1)) - 1;
+        if (!(__shfl_sync(FULL, fnode, s1) & kSmallNode)) {
+          if (lane == s1) fkey = kNoEntry;
+          --live_n;
+          if (lane >= W) src = s1;
+          use = lane < 2 * W;
+        }
+      }
+    }
+    const uint32_t node = __shfl_sync(FULL, fnode, src);
+#ifdef FGL_CHECKED
+    if (__any_sync(FULL, node >= tr.lim_nodes)) {
+      if (lane == 0) atomicOr(status, 4u);
+      return kPacketDone;
+    }
+#endif
+    const float* nd = (const float*)tr.nodes + (size_t)node * (node_stride(W) / 4);
+    const float x0r = __ldg(nd + fx), x1r = __ldg(nd + fx + 3 * W), y0r = __ldg(nd + fy), y1r = __ldg(nd + fy + 3 * W);
+    const float znr = __ldg(nd + fzn), zfr = __ldg(nd + fzf);
+    const uint32_t hb = __ldg((const uint32_t*)nd + 8 + 6 * W + c);
+    const uint4 h0 = __ldg((const uint4*)nd);
+    const uint2 base = __ldg((const uint2*)(nd + 4));  // child_base, tri_base
+    const float rx = sel3(__uint_as_float(h0.x), __uint_as_float(h0.y), __uint_as_float(h0.z), kx) - oX;
+    const float ry = sel3(__uint_as_float(h0.x), __uint_as_float(h0.y), __uint_as_float(h0.z), ky) - oY;
+    const float rz = (sel3(__uint_as_float(h0.x), __uint_as_float(h0.y), __uint_as_float(h0.z), kz) - oZ) * sg;
+    const float X0 = x0r + rx, X1 = x1r + rx, Y0 = y0r + ry, Y1 = y1r + ry;
+    const float zn = fmaf(znr, sg, rz), zf = fmaf(zfr, sg, rz), zc = fmaxf(zn, 0.f);
+    const float tn = max3f(max3f(zc * iz, X0 * ixp, X1 * ixn), Y0 * iyp, Y1 * iyn);
+    // inside: every one of these differences is non-negative
+    const float in = min3f(min3f(X1 - fminf(a0 * zc, a0 * zf), fmaxf(a1 * zc, a1 * zf) - X0, zf),
+                           Y1 - fminf(b0 * zc, b0 * zf), fmaxf(b1 * zc, b1 * zf) - Y0);
+    const bool hit = use & (in >= 0.f) & (__float_as_uint(tn) <= tkey);
+    const uint32_t got = hit ? hb : 0u;  // 0 for an empty slot
+    if (COUNT) {
+      const uint32_t nodes_now = __popc(__ballot_sync(FULL, use)) / W;
+      c_iters += lane == 0 ? nodes_now : 0u;
+      c_lane_iters += live ? nodes_now : 0u;
+      tr.n_nodes += live ? nodes_now : 0u;
+    }
+    const unsigned bi = __ballot_sync(FULL, got >> 24);
+    if (bi) {
+      if (got >> 24) {
+        const uint32_t child = base.x + __popc(h0.w & ((1u << c) - 1u));
+        const bool small = max3f(X1 - X0, Y1 - Y0, zf - zn) < narrow * zc;
+        const int at = __popc(bi & lt);
+        pl.entry[at] = make_uint2((__float_as_uint(tn) & ~7u) | (uint32_t)c, small ? child | kSmallNode : child);
+        parents[at] = node;
+      }
+      __syncwarp();
+      const int n_in = __popc(bi);
+      const int rank = __popc(__ballot_sync(FULL, fkey == kNoEntry) & lt);
+      if (fkey == kNoEntry && rank < n_in) {
+        const uint2 e = pl.entry[rank];
+        fkey = e.x;
+        fnode = e.y;
+        fpar = parents[rank];
+      }
+      live_n += n_in;
+      __syncwarp();
+    }
+    if (__any_sync(FULL, got & 0x00FFFFFFu)) {
+#pragma unroll 1
+      for (int g = 0; g < 2; ++g) {
+        uint32_t bits = __reduce_or_sync(FULL, lane / W == g ? got & 0x00FFFFFFu : 0u);
+        const uint32_t tb = __shfl_sync(FULL, base.y, g * W);
+        while (bits) {
+          const uint32_t pos = __ffs(bits) - 1;
+          bits &= bits - 1;
+#ifdef FGL_CHECKED
+          if ((size_t)tb + pos >= tr.lim_tris) {
+            if (lane == 0) atomicOr(status, 4u);
+            return kPacketDone;
+          }
+#else
+          (void)status;
+#endif
+          if (COUNT) {
+            tr.n_tris += live ? 1u : 0u;
+            tr.n_rounds += lane == 0 ? 1u : 0u;
+          }
+          const float* tp = (const float*)tr.tris + 12 * ((size_t)tb + pos);
+          const float* px = tp + tkx;
+          const float* py = tp + tky;
+          const float* pz = tp + tkz;
+          const int32_t id = __ldg((const int32_t*)tp + 3);
+          tr.consider(tri_hit_axes<true>(tr.r, __ldg(px) - toX, __ldg(py) - toY, __ldg(pz) - toZ, __ldg(px + 4) - toX,
+                                   __ldg(py + 4) - toY, __ldg(pz + 4) - toZ, __ldg(px + 8) - toX, __ldg(py + 8) - toY,
+                                   __ldg(pz + 8) - toZ, tr.best_t),
+                      id);
+        }
+      }
+      tkey = __float_as_uint(redux_maxf(tr.best_t)) | 7u;
+    }
+  }
+  // the boxes left, nearest first: each lane keeps the ones its ray meets
+  float e0 = 0.f, e1 = 0.f, e2 = 0.f, e3 = 0.f, e4 = 0.f, e5 = 0.f;
+  uint32_t key = kNoEntry;
+  if (fkey <= tkey) {
+    const float* nd = (const float*)tr.nodes + (size_t)fpar * (node_stride(W) / 4);
+    const float* q = nd + 8 + (fkey & 7u);
+    const float rx = __ldg(nd) - tr.r.ox, ry = __ldg(nd + 1) - tr.r.oy, rz = __ldg(nd + 2) - tr.r.oz;
+    e0 = __ldg(q) + rx;
+    e1 = __ldg(q + W) + ry;
+    e2 = __ldg(q + 2 * W) + rz;
+    e3 = __ldg(q + 3 * W) + rx;
+    e4 = __ldg(q + 4 * W) + ry;
+    e5 = __ldg(q + 5 * W) + rz;
+    key = fkey;
+  }
+  __syncwarp();
+  uint32_t mine = 0u;
+  for (uint32_t slot = 1u, k = 0u;; slot <<= 1, ++k) {
+    const uint32_t m = __reduce_min_sync(FULL, key);
+    if (m == kNoEntry) break;
+    const int own = __ffs(__ballot_sync(FULL, key == m)) - 1;
+    if (lane == own) {
+      pl.entry[k] = make_uint2(fkey & ~7u, fnode & ~kSmallNode);
+      key = kNoEntry;
+    }
+    const float x0 = __shfl_sync(FULL, e0, own) * tr.r.ix, x1 = __shfl_sync(FULL, e3, own) * tr.r.ix;
+    const float y0 = __shfl_sync(FULL, e1, own) * tr.r.iy, y1 = __shfl_sync(FULL, e4, own) * tr.r.iy;
+    const float z0 = __shfl_sync(FULL, e2, own) * tr.r.iz, z1 = __shfl_sync(FULL, e5, own) * tr.r.iz;
+    const float tn = max3f(fminf(x0, x1), fminf(y0, y1), fmaxf(fminf(z0, z1), tr.tmin()));
+    const float tf = min3f(fmaxf(x0, x1), fmaxf(y0, y1), fminf(fmaxf(z0, z1), tr.best_t));
+    if (tn <= tf) mine |= slot;
+  }
+  *pl.pend = mine;
+  __syncwarp();
+  return kPacketEntries;
 }
 
 }  // namespace dev
