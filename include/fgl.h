@@ -349,8 +349,7 @@ fgl_status fgl_world_rays(fgl_sensor sensor, const float* poses, int32_t n_env, 
 
 /* ------------------------------------------------------------------------ */
 /* Triangle LBVH built on the GPU (paper Sec. IV-C with the LBVH routine of  */
-/* Sec. IV-A): for meshes that change every frame, and the paper's one-      */
-/* thread-per-beam traversal                                                 */
+/* Sec. IV-A): for meshes that change every frame                            */
 /* ------------------------------------------------------------------------ */
 
 typedef struct fgl_lbvh_s* fgl_lbvh;
@@ -373,19 +372,22 @@ typedef struct {
  * Morton codes (eqs. u_i, m_i: 10 bits per axis of the centroid in the box of
  * all centroids), a stable radix sort, the hierarchy from longest common
  * prefixes (eq. LCP; equal codes ordered by position), then node boxes bottom
- * up; leaf boxes are grown by 2^-17 max(1, max |coord|).  Synchronises
+ * up; leaf boxes are grown by 2^-17 max(1, max |coord|).  The binary tree is
+ * then opened into the 8-wide nodes that the casts walk (91 B a triangle, plus
+ * 48 B for the triangles in their order; the build's scratch, about 140 B a
+ * triangle, stays with the LBVH for the next rebuild).  Synchronises
  * `stream` at the end.  Errors: FGL_ERR_INVALID (empty mesh, nt >= 2^30, a
  * vertex id out of range or a non-finite vertex), FGL_ERR_OOM, FGL_ERR_CUDA. */
 fgl_status fgl_lbvh_build(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
                           fgl_stream stream, fgl_lbvh* out);
 fgl_status fgl_lbvh_destroy(fgl_lbvh lbvh);
 fgl_status fgl_lbvh_get_stats(fgl_lbvh lbvh, fgl_lbvh_stats* out);
-/* Host copies of the nodes (64 B each: both child boxes as floats, then int32
+/* Host copies of the binary nodes (64 B each: both child boxes as floats, then int32
  * left, right, parent, 0; a reference < 0 is ~leaf) and the triangles in
  * Morton order (48 B each, as the wide BVH's leaf records). */
 fgl_status fgl_lbvh_export(fgl_lbvh lbvh, void* nodes, int64_t node_bytes, void* tris,
                            int64_t tri_bytes);
-/* eq. t_j* over an LBVH, one thread per beam (the paper's form): the same
+/* eq. t_j* over an LBVH, with fgl_cast's kernels on its 8-wide nodes: the same
  * returns, bit for bit, as fgl_cast on a wide BVH of the same mesh (same
  * triangle test and (t, id) rule), t in [min_range, max_range]. */
 fgl_status fgl_cast_lbvh(fgl_lbvh lbvh, fgl_sensor sensor, const float* poses, int32_t n_env,

@@ -482,7 +482,7 @@ class Lbvh:
 
     def cast(self, sensor: "Sensor", poses, max_range: float, min_range: float = 0.0,
              out_range=None, out_tri=None, stream=None):
-        """eq. t_j* over the LBVH, one thread per beam (fgl_cast_lbvh)."""
+        """eq. t_j* over the LBVH (fgl_cast_lbvh)."""
         n_env = poses.shape[0] if poses.dim() == 3 else poses.numel() // 12
         n = n_env * sensor.n_rays
         out_range, out_tri = _outputs(n, poses.device, out_range, out_tri)

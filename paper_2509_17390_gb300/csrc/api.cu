@@ -801,8 +801,8 @@ fgl_status fgl_cast(fgl_scene scene, fgl_sensor sensor, const float* poses, int3
   Opts o;
   ItemDesc d = make_desc(it);
   const bool packets = sensor->narrow && packet_opts(scene->bvh.width, o);
-  FGL_CUDA(launch_plain(scene->bvh.width, false, packets, d, o.block, o.sdepth, o.tri_mode, o.postpone,
-                        (cudaStream_t)stream));
+  FGL_CUDA(launch_plain(scene->bvh.width, false, packets, false, d, nullptr, o.block, o.sdepth, o.tri_mode,
+                        o.postpone, (cudaStream_t)stream));
   return FGL_OK;
 }
 
@@ -820,8 +820,8 @@ fgl_status fgl_cast_opts(fgl_scene scene, fgl_sensor sensor, const float* poses,
   // the refill threshold has no meaning here
   const bool packets =
       sensor->narrow && o.tri_mode == 0 && packets_fit(scene->bvh.width, o.block, o.sdepth);
-  FGL_CUDA(launch_plain(scene->bvh.width, o.count != 0, packets, d, o.block, o.sdepth, o.tri_mode, o.postpone,
-                        (cudaStream_t)stream));
+  FGL_CUDA(launch_plain(scene->bvh.width, o.count != 0, packets, false, d, nullptr, o.block, o.sdepth, o.tri_mode,
+                        o.postpone, (cudaStream_t)stream));
   return FGL_OK;
 }
 
@@ -837,8 +837,18 @@ fgl_status fgl_cast_lbvh(fgl_lbvh lbvh, fgl_sensor sensor, const float* poses, i
   if (n_env > 0 && (!poses || !out_range || !out_tri))
     return fail(FGL_ERR_INVALID, "null poses or output pointer");
   if (n_env == 0) return FGL_OK;
-  FGL_CUDA(launch_lbvh_cast(lbvh, sensor->d_dirs, poses, n_env, sensor->n_rays, min_range, max_range,
-                            out_range, out_tri, (cudaStream_t)stream));
+  ItemDesc d = lbvh_item(lbvh);
+  d.dirs = sensor->d_dirs;
+  d.poses = poses;
+  d.out_range = out_range;
+  d.out_tri = out_tri;
+  d.n_env = n_env;
+  d.n_rays = sensor->n_rays;
+  d.max_range = max_range;
+  d.min_range = min_range;
+  const Opts o;
+  FGL_CUDA(launch_plain(8, false, sensor->narrow && packet_opts(8, o), min_range > 0.f, d, lbvh_status(lbvh),
+                        o.block, o.sdepth, o.tri_mode, o.postpone, (cudaStream_t)stream));
   return FGL_OK;
 }
 

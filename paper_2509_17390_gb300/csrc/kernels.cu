@@ -67,15 +67,16 @@ __device__ __forceinline__ Smem<W> smem_layout(int sdepth) {
   return m;
 }
 
-template <int W, bool COUNT>
-__global__ void __maxnreg__(72) k_plain(const ItemDesc it, int sdepth, int tri_mode,
-                                               int postpone_pct) {
+template <int W, bool COUNT, bool TMIN>
+__global__ void __maxnreg__(72) k_plain(const ItemDesc it, int sdepth, int tri_mode, int postpone_pct,
+                                        unsigned* status) {
   using Keys = typename dev::KeyWords<W>::T;
   const unsigned FULL = 0xFFFFFFFFu;
   const Smem<W> sm = smem_layout<W>(sdepth);
   const int lane = threadIdx.x & 31;
+  if (status == nullptr) status = &g_status;
   if (it.width != W) {  // never read nodes laid out for another width
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&g_status, 2u);
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(status, 2u);
     return;
   }
   const int64_t total = (int64_t)it.n_env * it.n_rays;
@@ -83,7 +84,7 @@ __global__ void __maxnreg__(72) k_plain(const ItemDesc it, int sdepth, int tri_m
   bool done = gid >= total;
   int env = 0;
   float4 ds = make_float4(0.f, 0.f, 0.f, 0.f);
-  dev::Tracer<W, COUNT> tr;
+  dev::Tracer<W, COUNT, TMIN> tr;
   tr.tg = make_uint2(0u, 0u);
   tr.ng = make_uint2(0u, 0u);
   if (COUNT) tr.n_nodes = tr.n_tris = tr.n_rounds = tr.n_pops = 0;
@@ -103,10 +104,10 @@ __global__ void __maxnreg__(72) k_plain(const ItemDesc it, int sdepth, int tri_m
     while (__any_sync(FULL, !done)) {
       bool ok = true;
       if (!done) ok = tr.descend(st);
-      dev::tri_phase_warp(tr, sm.keys, lane, &g_status);
+      dev::tri_phase_warp(tr, sm.keys, lane, status);
       if (!done) {
         if (!ok) {
-          atomicOr(&g_status, tr.fail_bits());
+          atomicOr(status, tr.fail_bits());
           done = true;
         } else {
           done = tr.finish_pooled(st);
@@ -116,7 +117,7 @@ __global__ void __maxnreg__(72) k_plain(const ItemDesc it, int sdepth, int tri_m
   } else if (!done) {
     for (;;) {
       const int pl = postpone_threshold(postpone_pct);
-      if (tr.step(st, pl, &g_status)) break;
+      if (tr.step(st, pl, status)) break;
     }
   }
   if (gid < total) {
@@ -317,7 +318,7 @@ template <int W, bool COUNT, bool TMIN>
 __device__ __forceinline__ void trace_packet(const ItemDesc& it, int env, int first, int n, const Smem<W>& sm,
                                              const dev::PacketList& pl,
                                              const dev::StackRefs<typename dev::KeyWords<W>::T>& st,
-                                             uint32_t (&c)[kWorkCounters]) {
+                                             unsigned* status, uint32_t (&c)[kWorkCounters]) {
   const unsigned FULL = 0xFFFFFFFFu;
   const int lane = threadIdx.x & 31;
   const bool live = lane < n;  // a lane past the end copies the first ray (and neither traces alone nor stores)
@@ -331,7 +332,7 @@ __device__ __forceinline__ void trace_packet(const ItemDesc& it, int env, int fi
     dev::setup_ray(tr.r, ox, oy, oz, dx, dy, dz);
     tr.start(it.nodes, it.tris, it.min_range, it.max_range, it.n_nodes, it.n_tris);
     if (COUNT) tr.n_rounds = tr.n_pops = 0;
-    end = dev::packet_phase(tr, dx, dy, dz, pl, lane, live, &g_status, c[3], c[4]);
+    end = dev::packet_phase(tr, dx, dy, dz, pl, lane, live, status, c[3], c[4]);
   }
   if (end != dev::kPacketDone) {
     bool active = live && (end == dev::kPacketNone || tr.next_entry(pl));
@@ -342,10 +343,10 @@ __device__ __forceinline__ void trace_packet(const ItemDesc& it, int env, int fi
       }
       bool ok = true;
       if (active) ok = tr.descend(st);
-      dev::tri_phase_warp(tr, sm.keys, lane, &g_status);
+      dev::tri_phase_warp(tr, sm.keys, lane, status);
       if (active) {
         if (!ok) {
-          atomicOr(&g_status, tr.fail_bits());
+          atomicOr(status, tr.fail_bits());
           active = false;
         } else {
           active = !tr.template finish_pooled<true>(st, pl);
@@ -370,23 +371,24 @@ __device__ __forceinline__ void trace_packet(const ItemDesc& it, int env, int fi
 }
 
 // k_plain with packet phases: warp w of the grid takes packet w of the item.
-template <int W, bool COUNT>
-__global__ void __maxnreg__(72) k_plain_packets(const ItemDesc it, int sdepth) {
+template <int W, bool COUNT, bool TMIN>
+__global__ void __maxnreg__(72) k_plain_packets(const ItemDesc it, int sdepth, unsigned* status) {
   using Keys = typename dev::KeyWords<W>::T;
+  if (status == nullptr) status = &g_status;
   if (it.width != W) {  // never read nodes laid out for another width
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&g_status, 2u);
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(status, 2u);
     return;
   }
   const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int env = (p >> 32) ? (int)(p / it.pk_per_env) : (int)((uint32_t)p / (uint32_t)it.pk_per_env);
+  const int64_t env = (p >> 32) ? p / it.pk_per_env : (int64_t)((uint32_t)p / (uint32_t)it.pk_per_env);
   if (env >= it.n_env) return;
-  const int first = (int)(p - (int64_t)env * it.pk_per_env) * 32;
+  const int first = (int)(p - env * it.pk_per_env) * 32;
   const Smem<W> sm = smem_layout<W>(sdepth);
   uint2 ls[kStackLocal];
   Keys lq[kStackLocal];
   const dev::StackRefs<Keys> st{sm.ss, sm.sq, ls, lq, (int)blockDim.x, sdepth};
   uint32_t c[kWorkCounters] = {};
-  trace_packet<W, COUNT, false>(it, env, first, min(32, it.n_rays - first), sm, packet_smem(W, sdepth), st, c);
+  trace_packet<W, COUNT, TMIN>(it, (int)env, first, min(32, it.n_rays - first), sm, packet_smem(W, sdepth), st, status, c);
   flush_counters<COUNT>(c);
 }
 
@@ -434,7 +436,7 @@ __global__ void __maxnreg__(72) k_packets(BatchHeader* __restrict__ hdr, const I
     int first = (int)(local - (int64_t)env * ppe) * P;
     const int end = min(first + P, it.n_rays);
     for (; first < end; first += 32)
-      trace_packet<W, COUNT, TMIN>(it, env, first, min(32, end - first), sm, pl, st, c);
+      trace_packet<W, COUNT, TMIN>(it, env, first, min(32, end - first), sm, pl, st, &g_status, c);
   }
   flush_counters<COUNT>(c);
 }
@@ -696,18 +698,21 @@ void* pick_packets(int W, bool count, bool tmin) {
   return W == 8 ? pick_packets_w<8>(count, tmin) : pick_packets_w<4>(count, tmin);
 }
 
-template <int W, bool COUNT>
-void* plain_fn() {
-  return (void*)k_plain<W, COUNT>;
-}
 template <int W, bool COUNT, bool TMIN>
 void* persistent_fn() {
   return (void*)k_persistent<W, COUNT, TMIN>;
 }
 
-void* pick_plain(int W, bool count) {
-  if (W == 8) return count ? plain_fn<8, true>() : plain_fn<8, false>();
-  return count ? plain_fn<4, true>() : plain_fn<4, false>();
+// A minimum range comes with a GPU-built hierarchy only (8-wide, not counted).
+void* pick_plain(int W, bool count, bool tmin) {
+  if (W == 8 && tmin) return (void*)k_plain<8, false, true>;
+  if (W == 8) return count ? (void*)k_plain<8, true, false> : (void*)k_plain<8, false, false>;
+  return count ? (void*)k_plain<4, true, false> : (void*)k_plain<4, false, false>;
+}
+void* pick_plain_packets(int W, bool count, bool tmin) {
+  if (W == 8 && tmin) return (void*)k_plain_packets<8, false, true>;
+  if (W == 8) return count ? (void*)k_plain_packets<8, true, false> : (void*)k_plain_packets<8, false, false>;
+  return count ? (void*)k_plain_packets<4, true, false> : (void*)k_plain_packets<4, false, false>;
 }
 template <int W>
 void* pick_persistent_w(bool count, bool tmin) {
@@ -742,30 +747,22 @@ static cudaError_t allow_smem(void* fn, size_t smem) {
   return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
-cudaError_t launch_plain(int W, bool count, bool packets, const ItemDesc& it, int block, int sdepth,
-                         int tri_mode, int postpone_pct, cudaStream_t s) {
+cudaError_t launch_plain(int W, bool count, bool packets, bool tmin, const ItemDesc& it, unsigned* status, int block,
+                         int sdepth, int tri_mode, int postpone_pct, cudaStream_t s) {
   const int64_t total = (int64_t)it.n_env * it.n_rays;
   if (total == 0) return cudaSuccess;
+  if (tmin && (W != 8 || count)) return cudaErrorInvalidValue;  // no such form
   ItemDesc arg = it;
-  if (packets) {
-    arg.pk_per_env = (it.n_rays + 31) / 32;
-    const int64_t warps = (int64_t)it.n_env * arg.pk_per_env;
-    const int64_t grid = (warps * 32 + block - 1) / block;
-    const size_t smem = packets_smem_bytes(W, block, sdepth);
-    void* fn = W == 8 ? (count ? (void*)k_plain_packets<8, true> : (void*)k_plain_packets<8, false>)
-                      : (count ? (void*)k_plain_packets<4, true> : (void*)k_plain_packets<4, false>);
-    const cudaError_t e = allow_smem(fn, smem);
-    if (e != cudaSuccess) return e;
-    void* args[] = {&arg, &sdepth};
-    return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(block), args, smem, s);
-  }
-  const int64_t grid = (total + block - 1) / block;
-  const size_t smem = stack_smem_bytes(W, block, sdepth);
-  void* fn = pick_plain(W, count);
+  arg.pk_per_env = (it.n_rays + 31) / 32;
+  const int64_t threads = packets ? (int64_t)it.n_env * arg.pk_per_env * 32 : total;
+  const int64_t grid = (threads + block - 1) / block;
+  const size_t smem = packets ? packets_smem_bytes(W, block, sdepth) : stack_smem_bytes(W, block, sdepth);
+  void* fn = packets ? pick_plain_packets(W, count, tmin) : pick_plain(W, count, tmin);
   const cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
-  void* args[] = {&arg, &sdepth, &tri_mode, &postpone_pct};
-  return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(block), args, smem, s);
+  void* plain_args[] = {&arg, &sdepth, &tri_mode, &postpone_pct, &status};
+  void* packet_args[] = {&arg, &sdepth, &status};
+  return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(block), packets ? packet_args : plain_args, smem, s);
 }
 
 int persistent_blocks_per_sm(int W, bool count, bool tmin, bool packets, int block, int sdepth) {

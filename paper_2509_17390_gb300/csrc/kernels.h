@@ -16,8 +16,10 @@ size_t stack_smem_bytes(int W, int block, int sdepth);
 // tri_mode 0: warp-pooled leaf tests; 1: lane-serial with postponing.
 // packets: one packet of 32 rays of an environment a warp, walked together
 // before the per-ray traversal (needs tri_mode 0; see packets_fit).
-cudaError_t launch_plain(int W, bool count, bool packets, const ItemDesc& it, int block, int sdepth,
-                         int tri_mode, int postpone_pct, cudaStream_t s);
+// tmin honours it.min_range (8-wide nodes, not counted); status: the word that
+// takes traversal errors (null: the shared one).
+cudaError_t launch_plain(int W, bool count, bool packets, bool tmin, const ItemDesc& it, unsigned* status, int block,
+                         int sdepth, int tri_mode, int postpone_pct, cudaStream_t s);
 
 // Whether a block of this shape has room for the packet lists beside its
 // stacks (large blocks with deep shared stacks do not).
@@ -47,10 +49,10 @@ cudaError_t launch_instance_pass(const InstancePass& a, bool tmin, int block, in
 // World-frame return points of one item, after its scene and instance passes.
 cudaError_t launch_points(const ItemDesc& it, float* out, cudaStream_t s);
 
-// One-thread-per-ray cast over a GPU-built triangle LBVH (lbvh.cu).
-cudaError_t launch_lbvh_cast(const fgl_lbvh_s* L, const void* dirs, const float* poses, int n_env,
-                             int n_rays, float min_range, float max_range, float* out_range,
-                             int32_t* out_tri, cudaStream_t s);
+// The wide form of a GPU-built triangle LBVH as an item (sensor, poses,
+// ranges and outputs to be filled in) and its own status word (lbvh.cu).
+ItemDesc lbvh_item(const fgl_lbvh_s* L);
+unsigned* lbvh_status(const fgl_lbvh_s* L);
 
 // Debug export of world rays (beam order).
 cudaError_t launch_l2_read(const void* buf, int64_t bytes, int reps, unsigned* sink, int sms,
