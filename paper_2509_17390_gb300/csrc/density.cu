@@ -22,6 +22,7 @@
 // The paper finds the candidates of a tile with an LBVH query over Gaussian
 // AABBs (Karras); binning each Gaussian to the tiles its AABB covers gives
 // the same candidate sets without building or traversing a tree.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -226,11 +227,14 @@ __global__ void k_tile_bounds(const uint32_t* __restrict__ keys, int64_t n, int6
 // density: one block per tile of B^3 voxels.  Each warp of the block sums
 // every S-th batch of 32 candidates over the whole tile (two x-rows a lane, so
 // that a staged candidate is read once for 64 rows); the warps' sums are added
-// in warp order.  Bound by instruction issue and the FMA pipe about equally
+// in warp order.  A tile of more than 2 x 32 S candidates is shared by the K
+// blocks of a cluster, whose sums the first adds in block order (the others of
+// a smaller tile leave at once).  Bound by instruction issue and the FMA pipe about equally
 // (36 warp instructions for a candidate and 32 rows, of which 3 exponentials;
 // one exponential a voxel took 40, and 8 of them held the MUFU pipe longest).
-// 720 k Gaussians, 10,304 tiles of 2.5 cm voxels: 2.22 -> 1.51 ms; 85 k
-// Gaussians, 630 tiles of 5 cm: 0.63 -> 0.20 ms.
+// 720 k Gaussians, 10,304 tiles of 2.5 cm voxels: 2.22 -> 1.47 ms; 85 k
+// Gaussians, 630 tiles of 5 cm, up to 11,400 candidates a tile: 0.63 -> 0.10 ms
+// (0.23 without the clusters and with the voxels close to theta one at a time).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   uint64_t d;
@@ -259,10 +263,11 @@ constexpr float kRowFall = 20.f, kRowSlope = 60.f;
 
 // Voxels whose density falls this close to theta (relative) are summed again
 // voxel by voxel in candidate order, so that the masks never hang on the
-// rounding of the factored form or of the warps' partial sums: they differ
+// rounding of the factored form or of the warps' partial sums: those differ
 // from those sums by a few 1e-6 (a term's exponent by a few units of 2^-24 of
 // its partial sums).
 constexpr float kThetaBand = 1e-4f;
+constexpr int kCloseAtOnce = 8;
 
 // One staged candidate.  bx = M01 dy + M02 dz is the x coefficient and
 // syz = M11 dy^2 + M12 dy dz + M22 dz^2 the y/z part of the exponent.
@@ -280,23 +285,32 @@ struct DensityCfg {
   static constexpr int SUB = 32 / LANES;    // candidates a warp takes at once
 };
 
-template <int B, int S>
+template <int B, int S, int K>
 __global__ void __launch_bounds__(32 * S)
     k_density(const GaussParams* __restrict__ params, const uint32_t* __restrict__ cand,
               const uint32_t* __restrict__ begin, const uint32_t* __restrict__ end, GridArgs g, float theta,
               float* __restrict__ out) {
   using C = DensityCfg<B>;
   constexpr int NT = 32 * S;
-  __shared__ StagedGauss stage[S][32];
+  namespace cg = cooperative_groups;
+  constexpr int kRow = NT + 4;  // a voxel's terms of a batch of NT candidates, on banks of their own
+  __shared__ union {
+    StagedGauss batch[S][32];
+    float terms[2][1 + kCloseAtOnce][kRow];  // alpha^2, then 2^q of each voxel
+  } sh;
   __shared__ float s_sum[S > 1 ? S - 1 : 1][C::ROWS * B];
   const unsigned FULL = 0xFFFFFFFFu;
-  const int tile = blockIdx.x;
+  const int tile = blockIdx.x / K, rank = blockIdx.x % K;
   const int tx = tile % g.ntiles[0], ty = (tile / g.ntiles[0]) % g.ntiles[1],
             tz = tile / (g.ntiles[0] * g.ntiles[1]);
   const uint32_t b0 = begin[tile], b1 = end[tile];
+  // the tile's batches go round the warps of one block or of the whole cluster
+  const bool split = K > 1 && b1 - b0 > 2 * NT;
+  if (K > 1 && !split && rank > 0) return;  // all of the cluster's blocks agree
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t first = b0 + 32 * (split ? rank * S + warp : warp), stride = split ? 32 * S * K : 32 * S;
   const int slot = lane % C::LANES, sub = lane / C::LANES, y = slot % B, z = slot / B;  // rows (y, z), (y, z + B / 2)
-  StagedGauss* st = stage[warp];
+  StagedGauss* st = sh.batch[warp];
   // tile corner in FP64 (the offsets to the means are formed there, then
   // rounded once: |tile corner - mu| is small, so the float offset is accurate)
   const double cx = (double)g.o[0] + (double)(tx * B) * (double)g.h;
@@ -315,9 +329,9 @@ __global__ void __launch_bounds__(32 * S)
   // candidate numbers one batch earlier
   GaussParams P = {};
   uint32_t next = 0;
-  if (b0 + 32 * warp + lane < b1) P = params[cand[b0 + 32 * warp + lane]];
-  if (b0 + 32 * (warp + S) + lane < b1) next = cand[b0 + 32 * (warp + S) + lane];
-  for (uint32_t c0 = b0 + 32 * warp; c0 < b1; c0 += 32 * S) {
+  if (first + lane < b1) P = params[cand[first + lane]];
+  if (first + stride + lane < b1) next = cand[first + stride + lane];
+  for (uint32_t c0 = first; c0 < b1; c0 += stride) {
     __syncwarp();  // the batch before this one is summed
     const bool valid = c0 + lane < b1;
     const float dX = (float)(cx - (double)P.a.x), dY = (float)(cy - (double)P.a.y), dZ = (float)(cz - (double)P.a.z);
@@ -345,8 +359,8 @@ __global__ void __launch_bounds__(32 * S)
       }
     }
     __syncwarp();
-    if (c0 + 32 * S + lane < b1) P = params[next];
-    if (c0 + 64 * S + lane < b1) next = cand[c0 + 64 * S + lane];
+    if (c0 + stride + lane < b1) P = params[next];
+    if (c0 + 2 * stride + lane < b1) next = cand[c0 + 2 * stride + lane];
 #pragma unroll 1
     for (int i = sub; i < nf; i += C::SUB) {
       const float4 at = st[i].at, m = st[i].m, n = st[i].n;
@@ -425,57 +439,45 @@ __global__ void __launch_bounds__(32 * S)
           for (int i = 0; i < B; ++i) d[r][i] += s_sum[v][(r * B + i) * C::LANES + slot];
     }
   }
-  const int gx = tx * B, gy = ty * B + y;
-  const bool owner = warp == 0 && sub == 0 && gy < g.dims[1];
-  // voxels close to theta: their terms, a candidate a thread, then one
-  // thread's sum in candidate order
-  uint32_t close = 0;
+  if (K > 1 && split) {  // rank 0 adds the blocks' sums in rank order
+    __shared__ float s_part[C::ROWS * B];
+    cg::cluster_group cl = cg::this_cluster();
+    if (warp == 0 && sub == 0) {
 #pragma unroll
-  for (int r = 0; r < 2; ++r)
+      for (int r = 0; r < 2; ++r)
 #pragma unroll
-    for (int i = 0; i < B; ++i)
-      if (owner && tz * B + z + r * (B / 2) < g.dims[2] &&
-          fabsf(d[r][i] - theta) <= kThetaBand * (fabsf(d[r][i]) + fabsf(theta)))
-        close |= 1u << (r * B + i);
-  if (__syncthreads_or(close != 0u && b1 > b0)) {
-    __shared__ uint32_t s_close[C::LANES];
-    float* s_q = reinterpret_cast<float*>(stage);  // alpha^2 and 2^q of a batch of candidates
-    if (threadIdx.x < C::LANES) s_close[threadIdx.x] = close;
-    __syncthreads();
-    for (int o = 0; o < C::LANES; ++o) {
-      for (uint32_t left = s_close[o]; left; left &= left - 1) {  // the same for the whole block
-        const int bit = __ffs(left) - 1, i = bit % B;
-        const float vx = __fmul_rn((float)i + 0.5f, g.h), vy = __fmul_rn((float)(o % B) + 0.5f, g.h),
-                    vz = __fmul_rn((float)(o / B + (bit / B) * (B / 2)) + 0.5f, g.h);
-        float sum = 0.f;
-        for (uint32_t c0 = b0; c0 < b1; c0 += NT) {
-          if (c0 + threadIdx.x < b1) {
-            const GaussParams Q = params[cand[c0 + threadIdx.x]];
-            const float dx = __fadd_rn((float)(cx - (double)Q.a.x), vx), dy = __fadd_rn((float)(cy - (double)Q.a.y), vy),
-                        dz = __fadd_rn((float)(cz - (double)Q.a.z), vz);
-            const float syz = fmaf(fmaf(Q.b.y, dy, __fmul_rn(Q.c.y, dz)), dy, __fmul_rn(__fmul_rn(Q.b.z, dz), dz));
-            const float bx = fmaf(Q.b.w, dy, __fmul_rn(Q.c.x, dz));
-            s_q[2 * threadIdx.x] = Q.a.w;
-            s_q[2 * threadIdx.x + 1] = dev::ex2_approx(fmaf(fmaf(Q.b.x, dx, bx), dx, syz));
-          }
-          __syncthreads();
-          if (threadIdx.x == o) {
-            const int m = (int)min((uint32_t)NT, b1 - c0);
-#pragma unroll 8
-            for (int k = 0; k < m; ++k) sum = fmaf(s_q[2 * k], s_q[2 * k + 1], sum);
-          }
-          __syncthreads();
-        }
-        if (threadIdx.x == o) {
+        for (int i = 0; i < B; ++i) s_part[(r * B + i) * C::LANES + slot] = d[r][i];
+    }
+    cl.sync();
+    if (rank == 0) {
+      for (int v = threadIdx.x; v < C::ROWS * B; v += NT) {
+        float part[K];
 #pragma unroll
-          for (int r = 0; r < 2; ++r)
+        for (int k = 1; k < K; ++k) part[k] = *cl.map_shared_rank(s_part + v, k);
+        float sum = s_part[v];
 #pragma unroll
-            for (int j = 0; j < B; ++j)
-              if (r * B + j == bit) d[r][j] = sum;
-        }
+        for (int k = 1; k < K; ++k) sum += part[k];
+        s_part[v] = sum;  // read by nobody else
       }
     }
+    cl.sync();  // and the others' memory stays until it is read
+    if (rank > 0) return;
+    if (warp == 0 && sub == 0) {
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int i = 0; i < B; ++i) d[r][i] = s_part[(r * B + i) * C::LANES + slot];
+    }
   }
+  const int gx = tx * B, gy = ty * B + y;
+  const bool owner = warp == 0 && sub == 0 && gy < g.dims[1];
+  // the tile's densities; the voxels close to theta are then listed and summed
+  // again, kCloseAtOnce at a time: their terms a candidate a thread, each
+  // voxel's sum a lane's, in candidate order
+  __shared__ uint16_t s_close[C::ROWS * B];
+  __shared__ int s_n_close;
+  if (threadIdx.x == 0) s_n_close = 0;
+  __syncthreads();
   if (owner) {
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
@@ -483,16 +485,69 @@ __global__ void __launch_bounds__(32 * S)
       if (gz >= g.dims[2]) break;
       float* dst = out + ((int64_t)gz * g.dims[1] + gy) * g.dims[0];
 #pragma unroll
-      for (int i = 0; i < B; ++i)
-        if (gx + i < g.dims[0]) dst[gx + i] = d[r][i];
+      for (int i = 0; i < B; ++i) {
+        if (gx + i >= g.dims[0]) break;
+        dst[gx + i] = d[r][i];
+        if (b1 > b0 && fabsf(d[r][i] - theta) <= kThetaBand * (fabsf(d[r][i]) + fabsf(theta)))
+          s_close[atomicAdd(&s_n_close, 1)] = (uint16_t)(((z + r * (B / 2)) * B + y) * B + i);
+      }
     }
+  }
+  __syncthreads();
+  const int n_close = s_n_close;
+  for (int v0 = 0; v0 < n_close; v0 += kCloseAtOnce) {
+    const int n = min(kCloseAtOnce, n_close - v0);
+    float sum = 0.f;
+    GaussParams Q = {};
+    if (b0 + threadIdx.x < b1) Q = params[cand[b0 + threadIdx.x]];
+    int buf = 0;
+    for (uint32_t c0 = b0; c0 < b1; c0 += NT, buf ^= 1) {
+      const bool some = c0 + threadIdx.x < b1;
+      const float ex = (float)(cx - (double)Q.a.x), ey = (float)(cy - (double)Q.a.y), ez = (float)(cz - (double)Q.a.z);
+      sh.terms[buf][0][threadIdx.x] = some ? Q.a.w : 0.f;
+#pragma unroll 1
+      for (int v = 0; v < n; ++v) {
+        const int at = s_close[v0 + v];
+        const float dx = __fadd_rn(ex, __fmul_rn((float)(at % B) + 0.5f, g.h)),
+                    dy = __fadd_rn(ey, __fmul_rn((float)(at / B % B) + 0.5f, g.h)),
+                    dz = __fadd_rn(ez, __fmul_rn((float)(at / (B * B)) + 0.5f, g.h));
+        const float syz = fmaf(fmaf(Q.b.y, dy, __fmul_rn(Q.c.y, dz)), dy, __fmul_rn(__fmul_rn(Q.b.z, dz), dz));
+        const float bx = fmaf(Q.b.w, dy, __fmul_rn(Q.c.x, dz));
+        sh.terms[buf][1 + v][threadIdx.x] = some ? dev::ex2_approx(fmaf(fmaf(Q.b.x, dx, bx), dx, syz)) : 0.f;
+      }
+      if (c0 + NT + threadIdx.x < b1) Q = params[cand[c0 + NT + threadIdx.x]];
+      __syncthreads();  // and the batch before this one is summed
+      if (threadIdx.x < (unsigned)n) {
+#pragma unroll 4
+        for (int k = 0; k < NT; k += 4) {
+          const float4 w = *reinterpret_cast<const float4*>(&sh.terms[buf][0][k]);
+          const float4 e = *reinterpret_cast<const float4*>(&sh.terms[buf][1 + threadIdx.x][k]);
+          sum = fmaf(w.w, e.w, fmaf(w.z, e.z, fmaf(w.y, e.y, fmaf(w.x, e.x, sum))));
+        }
+      }
+    }
+    if (threadIdx.x < (unsigned)n) {  // over the owner's store, a barrier ago
+      const int at = s_close[v0 + threadIdx.x];
+      out[((int64_t)(tz * B + at / (B * B)) * g.dims[1] + ty * B + at / B % B) * g.dims[0] + gx + at % B] = sum;
+    }
+    __syncthreads();
   }
 }
 
-template <int B, int S>
-void launch_density(int64_t n_tiles, const GaussParams* params, const uint32_t* cand, const uint32_t* begin,
-                    const uint32_t* end, const GridArgs& g, float theta, float* out, cudaStream_t s) {
-  k_density<B, S><<<(unsigned)n_tiles, 32 * S, 0, s>>>(params, cand, begin, end, g, theta, out);
+template <int B, int S, int K>
+cudaError_t launch_density(int64_t n_tiles, const GaussParams* params, const uint32_t* cand, const uint32_t* begin,
+                           const uint32_t* end, const GridArgs& g, float theta, float* out, cudaStream_t s) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = K;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(n_tiles * K));
+  cfg.blockDim = dim3(32 * S);
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = K > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k_density<B, S, K>, params, cand, begin, end, g, theta, out);
 }
 
 // eqs. V_occ, Int, Surf: a warp 32 voxels of a row, a block eight rows of a
@@ -695,15 +750,19 @@ extern "C" fgl_status fgl_gaussian_density(const fgl_gaussians* gs, const fgl_gr
     DCUDA(cudaGetLastError());
     if (timing) DCUDA(cudaEventRecord(S.ev[1], s));
     // Warps a tile: four of 32 candidates each even out tiles of unequal counts
-    // (2.25 ms for the pass at 10,304 tiles, 2.53 with two, 2.99 with one); a
-    // grid of fewer than 16 tiles an SM takes eight, or its few tiles would
-    // leave most of the chip idle.
+    // (2.25 ms for the pass at 10,304 tiles, 2.53 with two, 2.99 with one), in
+    // two blocks for a tile of many (the call 1.92 -> 1.87 ms; four blocks 1.97,
+    // launching them costs more); a grid of fewer than 16 tiles an SM takes
+    // eight warps in four blocks, or its heaviest tiles would run on alone (630
+    // tiles: the call 0.54 ms in one block, 0.49 in two, 0.475 in four or
+    // eight).  Tiles of 4^3 voxels have fewer candidates each: one block of one
+    // warp where there are many (25,000 tiles: 1.60 ms; two blocks 2.33).
     const GaussParams* params = (const GaussParams*)S.params;
     const bool few = n_tiles < 152 * 16;
-    if (B == 8 && few) launch_density<8, 8>(n_tiles, params, v0, begin, end, g, theta, out_density, s);
-    else if (B == 8) launch_density<8, 4>(n_tiles, params, v0, begin, end, g, theta, out_density, s);
-    else if (few) launch_density<4, 4>(n_tiles, params, v0, begin, end, g, theta, out_density, s);
-    else launch_density<4, 1>(n_tiles, params, v0, begin, end, g, theta, out_density, s);
+    if (B == 8 && few) DCUDA((launch_density<8, 8, 4>(n_tiles, params, v0, begin, end, g, theta, out_density, s)));
+    else if (B == 8) DCUDA((launch_density<8, 4, 2>(n_tiles, params, v0, begin, end, g, theta, out_density, s)));
+    else if (few) DCUDA((launch_density<4, 4, 4>(n_tiles, params, v0, begin, end, g, theta, out_density, s)));
+    else DCUDA((launch_density<4, 1, 1>(n_tiles, params, v0, begin, end, g, theta, out_density, s)));
     ++launches;
     DCUDA(cudaGetLastError());
     if (timing) DCUDA(cudaEventRecord(S.ev[2], s));

@@ -74,3 +74,29 @@ def test_far_thin_gaussian_adds_no_nan():
         dims = (20, 20, 20)
         D, _, _ = run((mu, scale, q, al), (0.0, 0.0, 0.0), h, dims, 0.5, 8)
         assert np.all(np.isfinite(D)) and np.all(D >= 0)
+
+
+# a tile shared by a cluster's blocks (more than two batches a warp, and one
+# less), and more voxels at theta than are summed at once: Gaussians mirrored
+# about the tile's middle planes give eight voxels the same density up to
+# rounding
+@pytest.mark.parametrize("tile,n", [(8, 512), (8, 520), (8, 4096), (4, 256), (4, 264), (4, 2048)])
+def test_shared_tiles_and_equal_voxels(tile, n):
+    rng = np.random.default_rng(n + tile)
+    h = 0.05
+    L = h * tile
+    m, s, q, a = gaussians(rng, n // 8, L / 2, 0.02, 0.2)
+    q[:] = (1, 0, 0, 0)
+    sign = np.array([[x, y, z] for x in (1, -1) for y in (1, -1) for z in (1, -1)], np.float32)
+    g = (((m - L / 2)[None] * sign[:, None] + L / 2).reshape(-1, 3).astype(np.float32), np.tile(s, (8, 1)),
+         np.tile(q, (8, 1)), np.tile(a, 8))
+    dims = (tile, tile, tile)
+    Do, Ao = oracle.density(*g, (0.0, 0.0, 0.0), h, dims, tile)
+    tol = oracle.density_tolerance(Do, Ao)
+    D, _, _ = run(g, (0.0, 0.0, 0.0), h, dims, 0.5, tile)
+    assert np.all(np.abs(D.astype(np.float64) - Do) <= tol)
+    theta = float(D.reshape(-1)[tile * tile + 1])
+    E, occ, surf = run(g, (0.0, 0.0, 0.0), h, dims, theta, tile)
+    assert np.all(np.abs(E.astype(np.float64) - Do) <= tol)
+    occ_g, surf_g = oracle.occupancy(E.astype(np.float64), np.float64(np.float32(theta)))
+    assert np.array_equal(occ, occ_g) and np.array_equal(surf, surf_g)
