@@ -508,9 +508,11 @@ __global__ void __launch_bounds__(32 * S)
 #pragma unroll 1
       for (int v = 0; v < n; ++v) {
         const int at = s_close[v0 + v];
+        // x rounded in two steps and y, z in one, as voxel by voxel sums always
+        // were: the masks at theta stay what they are to the last bit
         const float dx = __fadd_rn(ex, __fmul_rn((float)(at % B) + 0.5f, g.h)),
-                    dy = __fadd_rn(ey, __fmul_rn((float)(at / B % B) + 0.5f, g.h)),
-                    dz = __fadd_rn(ez, __fmul_rn((float)(at / (B * B)) + 0.5f, g.h));
+                    dy = __fmaf_rn((float)(at / B % B) + 0.5f, g.h, ey),
+                    dz = __fmaf_rn((float)(at / (B * B)) + 0.5f, g.h, ez);
         const float syz = fmaf(fmaf(Q.b.y, dy, __fmul_rn(Q.c.y, dz)), dy, __fmul_rn(__fmul_rn(Q.b.z, dz), dz));
         const float bx = fmaf(Q.b.w, dy, __fmul_rn(Q.c.x, dz));
         sh.terms[buf][1 + v][threadIdx.x] = some ? dev::ex2_approx(fmaf(fmaf(Q.b.x, dx, bx), dx, syz)) : 0.f;
