@@ -124,25 +124,36 @@ __global__ void k_pack_u8(const uint8_t* __restrict__ V, BitGrid g, uint32_t* __
   }
 }
 
+constexpr int kPackInside = 16;  // the same for float samples: 27 M in rows of 375, 44 us with eight -> 21
+
 // the same on the sample grid m (every step-th voxel of the nx x ny voxel
 // grid): bit = phi < iso
+template <bool STEP1>
 __global__ void k_pack_inside(const float* __restrict__ phi, int nx, int ny, int step, BitGrid m,
                               float iso, uint32_t* __restrict__ out) {
   const int lane = threadIdx.x & 31;
   const int64_t n_warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   for (int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < m.rows(); row += n_warps) {
-    const int j = (int)((uint32_t)row % (uint32_t)m.ny), k = (int)((uint32_t)row / (uint32_t)m.ny);
+    const int k = (int)m.by_ny.div((uint32_t)row), j = (int)((uint32_t)row - (uint32_t)k * (uint32_t)m.ny);
     const float* src = phi + ((int64_t)k * step * ny + (int64_t)j * step) * nx;
     uint32_t* dst = out + row * m.mw;
-    for (int xw0 = 0; xw0 < m.mw; xw0 += kPackWords) {
+    for (int xw0 = 0; xw0 < m.mw; xw0 += kPackInside) {
+      float f[kPackInside];
+      const float* at = src + (int64_t)(xw0 * 32 + lane) * step;
+      const int left = m.nx - xw0 * 32 - lane;  // samples of the row from this lane's on
+#pragma unroll
+      for (int u = 0; u < kPackInside; ++u) {
+        if (u % 4 == 0 && xw0 + u >= m.mw) break;
+        f[u] = u * 32 < left ? __ldg(at + (STEP1 ? u * 32 : (int64_t)(u * 32) * step)) : INFINITY;
+      }
       uint32_t mine = 0;
 #pragma unroll
-      for (int u = 0; u < kPackWords; ++u) {
-        const int x = (xw0 + u) * 32 + lane;
-        const uint32_t mk = __ballot_sync(0xFFFFFFFFu, x < m.nx && src[(int64_t)x * step] < iso);
+      for (int u = 0; u < kPackInside; ++u) {
+        if (u % 4 == 0 && xw0 + u >= m.mw) break;
+        const uint32_t mk = __ballot_sync(0xFFFFFFFFu, f[u] < iso);
         if (lane == u) mine = mk;
       }
-      if (lane < kPackWords && xw0 + lane < m.mw) dst[xw0 + lane] = mine;
+      if (lane < kPackInside && xw0 + lane < m.mw) dst[xw0 + lane] = mine;
     }
   }
 }
@@ -221,10 +232,11 @@ __global__ void k_blur(const TIn* __restrict__ in, float* __restrict__ out, int 
 constexpr int kBTX = 32, kBTY = 32, kBQ = kBTY / 8;  // kBQ rows a thread
 
 template <int R>
-__global__ void __launch_bounds__(256, R <= 2 ? 4 : 3) k_blur_fused(const uint8_t* __restrict__ in, int nx, int ny, int nz,
+__global__ void __launch_bounds__(256, 3) k_blur_fused(const uint8_t* __restrict__ in, int nx, int ny, int nz,
                                                     int zc, Taps taps, float thr, float* __restrict__ out_blur,
                                                     uint8_t* __restrict__ out_mask) {
   constexpr int K = 2 * R + 1, EY = kBTY + 2 * R, NT = 1 << K, RPW = (EY + 7) / 8;
+  constexpr int RPH = 32 / (2 * R), NH = (RPW + RPH - 1) / RPH;  // rows whose last 2R voxels one load takes
   __shared__ float s_tab[NT];
   __shared__ float s_x[2][EY][kBTX];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -239,27 +251,32 @@ __global__ void __launch_bounds__(256, R <= 2 ? 4 : 3) k_blur_fused(const uint8_
     for (int t = 0; t < K; ++t) acc = __fmaf_rn(w[t], ((p >> t) & 1) ? 1.f : 0.f, acc);
     s_tab[p] = acc;
   }
-  // this warp's input rows r = wid + 8 rr; lane l holds x = x0 - R + l and x0 - R + 32 + l
-  const int gx0 = x0 - R + lane, gx1 = x0 - R + 32 + lane;
-  const bool c0 = gx0 >= 0 && gx0 < nx, c1 = lane < 2 * R && gx1 < nx;
+  // this warp's input rows r = wid + 8 rr; lane l holds x = x0 - R + l of each,
+  // and of the voxels from x0 - R + 32 on those of row rr = l / 2R
+  const int gx0 = x0 - R + lane, gx1 = x0 - R + 32 + lane % (2 * R);
+  const bool c0 = gx0 >= 0 && gx0 < nx, c1 = lane < 2 * R * RPH && gx1 < nx;
   const int64_t plane = (int64_t)ny * nx;
-  const int off0 = (y0 - R + wid) * nx + gx0;  // offset in a plane of row rr = 0 (ny nx < 2^31)
+  const int off0 = (y0 - R + wid) * nx + gx0, off1 = (y0 - R + wid) * nx + gx1;  // offsets in a plane of row rr = 0 (ny nx < 2^31)
   uint32_t rows_ok = 0;
 #pragma unroll
   for (int rr = 0; rr < RPW; ++rr) {
     const int r = wid + 8 * rr, gy = y0 - R + r;
     if (r < EY && gy >= 0 && gy < ny) rows_ok |= 1u << rr;
   }
-  uint32_t v[RPW][2];
+  uint32_t v[RPW], vh[NH];
   auto load_plane = [&](int z) {
     const uint32_t ok_rows = (z >= 0 && z < nz) ? rows_ok : 0u;
     const uint8_t* pl = in + (int64_t)z * plane;
 #pragma unroll
     for (int rr = 0; rr < RPW; ++rr) {
       const bool ok = (ok_rows >> rr) & 1u;
-      const int o = off0 + 8 * rr * nx;
-      v[rr][0] = (ok && c0) ? pl[o] : 0u;
-      v[rr][1] = (ok && c1) ? pl[o + 32] : 0u;
+      v[rr] = (ok && c0) ? pl[off0 + 8 * rr * nx] : 0u;
+    }
+#pragma unroll
+    for (int q = 0; q < NH; ++q) {
+      const int rr = q * RPH + lane / (2 * R);
+      const bool ok = rr < RPW && ((ok_rows >> rr) & 1u);
+      vh[q] = (ok && c1) ? pl[off1 + 8 * rr * nx] : 0u;
     }
   };
   load_plane(z0 - R);
@@ -277,12 +294,16 @@ __global__ void __launch_bounds__(256, R <= 2 ? 4 : 3) k_blur_fused(const uint8_
       const int pz = pz0 + u;
       if (pz >= n_planes) break;  // block-uniform
       const int buf = pz & 1;
+      uint32_t hi[NH];
+#pragma unroll
+      for (int q = 0; q < NH; ++q) hi[q] = __ballot_sync(0xFFFFFFFFu, vh[q] != 0u);
 #pragma unroll
       for (int rr = 0; rr < RPW; ++rr) {
-        const uint32_t lo = __ballot_sync(0xFFFFFFFFu, v[rr][0] != 0u);
-        const uint32_t hi = __ballot_sync(0xFFFFFFFFu, v[rr][1] != 0u);
+        const uint32_t lo = __ballot_sync(0xFFFFFFFFu, v[rr] != 0u);
         const int r = wid + 8 * rr;
-        if (r < EY) s_x[buf][r][lane] = s_tab[__funnelshift_r(lo, hi, lane) & (uint32_t)(NT - 1)];
+        // only the lowest 2R bits of the high word reach a sum
+        if (r < EY)
+          s_x[buf][r][lane] = s_tab[__funnelshift_r(lo, hi[rr / RPH] >> (rr % RPH * 2 * R), lane) & (uint32_t)(NT - 1)];
       }
       if (pz + 1 < n_planes) load_plane(z0 - R + pz + 1);
       __syncthreads();
@@ -954,6 +975,149 @@ __global__ void k_phi(const uint32_t* __restrict__ Ob, const uint32_t* __restric
   }
 }
 
+// The shells and phi of a narrow band (L <= kTileShells) in one launch: a block
+// takes 8 x 8 rows of up to 8 words, with the L + 1 rows around them and one
+// word on each side in shared memory, where S_0 and the growing masks are
+// formed over the shrinking halo (a step moves a border's error by one bit, and
+// the side words have 32); a word's sign and count bits then reach its 32
+// voxels as one 16-byte broadcast.  Bound by issue (80%; the 106 MB of phi at
+// 27 M voxels take 17 us): L = 3 there, 88 us for k_s0, three k_dilate and
+// k_phi -> 60; at 0.5 M voxels and L = 2, 25 -> 10.
+constexpr int kTileShells = 6;  // counts up to 7: three bits
+constexpr int kShellRows = 8, kShellWords = 8, kShellThreads = 256;
+
+struct ShellPlan {
+  int tw;  // words a tile, the same for all tiles of a row but the last
+  dim3 grid;
+  size_t smem;
+};
+
+ShellPlan plan_shells(const BitGrid& g, int L) {
+  ShellPlan p;
+  const int nx = (g.mw + kShellWords - 1) / kShellWords;
+  p.tw = (g.mw + nx - 1) / nx;
+  p.grid = dim3((unsigned)((g.mw + p.tw - 1) / p.tw), (unsigned)((g.ny + kShellRows - 1) / kShellRows),
+                (unsigned)((g.nz + kShellRows - 1) / kShellRows));
+  const int side = kShellRows + 2 * (L + 1);
+  p.smem = sizeof(uint32_t) * 2 * (size_t)side * side * (p.tw + 2);
+  return p;
+}
+
+template <bool EXTRA>  // writes the signs or shells too
+__global__ void __launch_bounds__(kShellThreads) k_shell_phi(const uint32_t* __restrict__ Vb,
+                                                             const uint32_t* __restrict__ Ob, int L, BitGrid g, int tw,
+                                                             float h, float r, float off, float* __restrict__ phi,
+                                                             uint8_t* __restrict__ out_outside,
+                                                             uint8_t* __restrict__ out_shell) {
+  extern __shared__ uint32_t shm[];
+  __shared__ uint4 s_word[kShellRows * kShellRows * kShellWords];  // count bits and sign of the tile's words
+  __shared__ float s_delta[16];                                    // by count and sign
+  __shared__ uint8_t s_p[8];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int H = L + 1, side = kShellRows + 2 * H, W = tw + 2, plane = side * W, cells = side * plane;
+  const int x0 = blockIdx.x * tw - 1, y0 = blockIdx.y * kShellRows - H, z0 = blockIdx.z * kShellRows - H;
+  const uint32_t by_w = 65536u / (uint32_t)W + 1u;  // exact quotients below 65536 / W
+  if (tid < 16) {
+    const int held = tid & 7, p = held ? max(L + 1 - held, 0) : 255;
+    // (p + off) is exact in float32, so its product with h rounds once,
+    // like the product of the exact values
+    const float delta = p == 255 ? r : fminf(((float)p + off) * h, r);
+    s_delta[tid] = tid & 8 ? delta : -delta;
+    if (tid < 8) s_p[tid] = (uint8_t)p;
+  }
+  uint32_t *cur = shm, *nxt = shm + cells;
+  const uint32_t by_side = 65536u / (uint32_t)side + 1u;
+  for (int i = tid; i < cells; i += kShellThreads) {
+    const int row = (int)((uint32_t)i * by_w >> 16), xw = x0 + i - row * W;
+    const int zz = (int)((uint32_t)row * by_side >> 16), j = y0 + row - zz * side, k = z0 + zz;
+    const bool in = xw >= 0 && xw < g.mw && j >= 0 && j < g.ny && k >= 0 && k < g.nz;
+    cur[i] = in ? Vb[((int64_t)k * g.ny + j) * g.mw + xw] : 0u;
+  }
+  // this thread's words of the tile
+  const int n_core = kShellRows * kShellRows * tw;
+  uint32_t c[2][3] = {};
+  __syncthreads();
+  for (int m = 0; m <= L; ++m) {  // the rows at least m + 1 from the halo's border
+    const int e = side - 2 * (m + 1), n = e * e * W;
+    const uint32_t by_e = 65536u / (uint32_t)e + 1u;
+    for (int i = tid; i < n; i += kShellThreads) {
+      const int row = (int)((uint32_t)i * by_w >> 16), x = i - row * W;
+      const int rz = (int)((uint32_t)row * by_e >> 16), zz = rz + m + 1, yy = row - rz * e + m + 1;
+      const int at = zz * plane + yy * W + x, xw = x0 + x, j = y0 + yy, k = z0 + zz;
+      uint32_t d = 0;
+      if (xw >= 0 && xw < g.mw && j >= 0 && j < g.ny && k >= 0 && k < g.nz) {
+        const uint32_t v = cur[at], prev = x > 0 ? cur[at - 1] : 0u, next = x + 1 < W ? cur[at + 1] : 0u;
+        const uint32_t xm = (v << 1) | (prev >> 31), xp = (v >> 1) | (next << 31);
+        const uint32_t ym = cur[at - W], yp = cur[at + W], zm = cur[at - plane], zp = cur[at + plane];
+        if (m == 0) {  // eq. S_0: an in-grid face neighbour of the other value
+          d = ((v ^ xm) & (xw == 0 ? ~1u : ~0u)) | ((v ^ xp) & valid_bits_next(g, xw));
+          if (j > 0) d |= v ^ ym;
+          if (j + 1 < g.ny) d |= v ^ yp;
+          if (k > 0) d |= v ^ zm;
+          if (k + 1 < g.nz) d |= v ^ zp;
+        } else {  // the mask grown by its face neighbours
+          d = v | xm | xp | ym | yp | zm | zp;
+        }
+        d &= valid_bits(g, xw);
+      }
+      nxt[at] = d;
+    }
+    __syncthreads();
+    uint32_t* t = cur;
+    cur = nxt;
+    nxt = t;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int i = tid + u * kShellThreads;
+      if (i >= n_core) break;
+      const int row = i / tw, x = i - row * tw;
+      uint32_t carry = cur[(row / kShellRows + H) * plane + (row % kShellRows + H) * W + x + 1];
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const uint32_t old = c[u][q];
+        c[u][q] = old ^ carry;
+        carry &= old;
+      }
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int i = tid + u * kShellThreads;
+    if (i >= n_core) break;
+    const int row = i / tw, xw = x0 + 1 + i - row * tw;
+    const int j = y0 + H + row % kShellRows, k = z0 + H + row / kShellRows;
+    const uint32_t ob = xw < g.mw && j < g.ny && k < g.nz ? Ob[((int64_t)k * g.ny + j) * g.mw + xw] : 0u;
+    s_word[i] = make_uint4(c[u][0], c[u][1], c[u][2], ob);
+  }
+  __syncthreads();
+  const int xb = (x0 + 1) * 32 + lane;
+#pragma unroll 1
+  for (int row = wid; row < kShellRows * kShellRows; row += kShellThreads / 32) {
+    const int j = y0 + H + row % kShellRows, k = z0 + H + row / kShellRows;
+    if (j >= g.ny || k >= g.nz) continue;
+    const int64_t v0 = ((int64_t)k * g.ny + j) * g.nx;
+    float* dst = phi + v0 + xb;
+    const uint4* words = s_word + row * tw;
+    int left = g.nx - xb;  // voxels of the row from this lane's on
+#pragma unroll 2
+    for (int x = 0; x < tw; ++x, left -= 32) {
+      const uint4 w = words[x];
+      const int out = (int)((w.w >> lane) & 1u);
+      int held = 0;
+      float f = out ? r : -r;
+      if ((w.x | w.y | w.z) != 0u) {  // most words are all outside the band
+        held = (int)(((w.x >> lane) & 1u) | ((w.y >> lane) & 1u) << 1 | ((w.z >> lane) & 1u) << 2);
+        f = s_delta[held | out << 3];
+      }
+      if (left > 0) {
+        dst[32 * x] = f;
+        if (EXTRA && out_outside) out_outside[v0 + xb + 32 * x] = (uint8_t)out;
+        if (EXTRA && out_shell) out_shell[v0 + xb + 32 * x] = s_p[held];
+      }
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------
 // marching tetrahedra
 // ---------------------------------------------------------------------------
@@ -1016,56 +1180,61 @@ __device__ __forceinline__ uint32_t active_cubes(const uint32_t C[8], uint32_t c
   return cubes & any1 & ~all1;
 }
 
-// Offsets.  The words (plus the end position nw, which counts nothing) split
-// into chunks of kMtChunk; a word's vertex, triangle and active-sample |
-// active-cube offsets are its chunk's prefix (pre[3 c + q], q = vertex,
-// triangle, active) plus the exclusive sum of the lower words of its chunk
-// (loc_v, loc_t, loc_a).  Every sum stays below 2^32 within a chunk, and the
-// two halves of an active count each below 2^32 overall (samples < 2^32).
-constexpr int kMtChunkLog = 11, kMtChunk = 1 << kMtChunkLog, kMtThreads = 256;
-constexpr int kMtPer = kMtChunk / kMtThreads;  // words a thread counts
-
-__device__ __forceinline__ unsigned long long mt_base(const unsigned long long* __restrict__ pre, int q,
-                                                      uint32_t loc, int64_t w) {
-  return pre[3 * (w >> kMtChunkLog) + q] + loc;
+// word id -> (j, k, xw) of the sample grid
+__device__ __forceinline__ void word_coords(const BitGrid& m, uint32_t w, int* j, int* k, int* xw) {
+  const uint32_t row = m.by_mw.div(w), kk = m.by_ny.div(row);  // words < 2^31
+  *xw = (int)(w - row * (uint32_t)m.mw);
+  *j = (int)(row - kk * (uint32_t)m.ny);
+  *k = (int)kk;
 }
 
-__device__ __forceinline__ int mt_pad(int p) { return p + (p >> 5); }  // no bank conflicts at stride kMtPer
+// Offsets.  The words (plus the end position nw, which counts nothing) split
+// into chunks of a block's threads times PER words; a word's vertex, triangle
+// and active-sample | active-cube offsets are its chunk's prefix (pre[3 c + q],
+// q = vertex, triangle, active) plus the exclusive sum of the lower words of
+// its chunk (loc_v, loc_t, loc_a).  Every sum stays below 2^32 within a chunk,
+// and the two halves of an active count each below 2^32 overall (samples <
+// 2^32).
+constexpr int kMtThreads = 256;  // chunks of 2^8 PER words
 
-// Per word of chunk blockIdx.x: the seven crossing words, then its offsets
-// within the chunk; the chunk's totals go to pre[3 c + q].  Counts are staged
-// in shared memory so the loads and stores stay coalesced while each thread
-// scans kMtPer consecutive words.
+__device__ __forceinline__ int mt_pad(int p) { return p + (p >> 5); }  // no bank conflicts at stride PER
+
+// Per word of chunk blockIdx.x: the seven crossing words and their union, then
+// its offsets within the chunk; the chunk's totals go to pre[3 c + q].  Counts
+// are staged in shared memory so the loads and stores stay coalesced while each
+// thread scans PER consecutive words.  QUERY: the totals alone.
+template <int PER, bool QUERY>
 __global__ void __launch_bounds__(kMtThreads) k_mt_count(const uint32_t* __restrict__ I, BitGrid m,
-                                                         uint32_t* __restrict__ X, uint32_t* __restrict__ loc_v,
+                                                         uint32_t* __restrict__ X, uint32_t* __restrict__ A,
+                                                         uint32_t* __restrict__ loc_v,
                                                          uint32_t* __restrict__ loc_t,
                                                          unsigned long long* __restrict__ loc_a,
                                                          unsigned long long* __restrict__ pre) {
-  constexpr int kPad = kMtChunk + kMtChunk / 32;
+  constexpr int kMtChunk = kMtThreads * PER, kPad = kMtChunk + kMtChunk / 32;
   __shared__ uint32_t sc[4][kPad];  // vertices, triangles, active samples, active cubes
   __shared__ uint32_t warp_tot[kMtThreads / 32][4];
   const int64_t nw = m.words();
   const int64_t base = (int64_t)blockIdx.x * kMtChunk;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 #pragma unroll 1
-  for (int u = 0; u < kMtPer; ++u) {
+  for (int u = 0; u < PER; ++u) {
     const int idx = u * kMtThreads + tid;
     const int64_t w = base + idx;
     uint32_t nv = 0, nt = 0, ns = 0, nc = 0;
     if (w < nw) {
-      const uint32_t row = (uint32_t)w / (uint32_t)m.mw;  // words < 2^31
-      const int xw = (int)((uint32_t)w - row * (uint32_t)m.mw);
-      const int j = (int)(row % (uint32_t)m.ny), k = (int)(row / (uint32_t)m.ny);
+      int j, k, xw;
+      word_coords(m, (uint32_t)w, &j, &k, &xw);
       uint32_t C[8], Xw[7];
       corner_words(I, m, j, k, xw, C);
       crossing_words(C, m, j, k, xw, Xw);
       uint32_t any = 0;
 #pragma unroll
       for (int t = 0; t < 7; ++t) {
-        X[t * nw + w] = Xw[t];
+        if (!QUERY) X[t * nw + w] = Xw[t];
         nv += __popc(Xw[t]);
         any |= Xw[t];
       }
+      if (!QUERY) A[w] = any;
       const uint32_t cubes = cube_bits(m, j, k, xw);
       nt = tri_count(C, cubes);
       ns = __popc(any);
@@ -1080,8 +1249,8 @@ __global__ void __launch_bounds__(kMtThreads) k_mt_count(const uint32_t* __restr
   __syncthreads();
   uint32_t run[4] = {0, 0, 0, 0};  // this thread's words: exclusive sums in place
 #pragma unroll
-  for (int u = 0; u < kMtPer; ++u) {
-    const int pi = mt_pad(tid * kMtPer + u);
+  for (int u = 0; u < PER; ++u) {
+    const int pi = mt_pad(tid * PER + u);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const uint32_t c = sc[q][pi];
@@ -1101,26 +1270,27 @@ __global__ void __launch_bounds__(kMtThreads) k_mt_count(const uint32_t* __restr
     if (lane == 31) warp_tot[wid][q] = incl[q];
   }
   __syncthreads();
-  uint32_t off[4];
+  uint32_t off[4];  // of this thread's words
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     off[q] = incl[q] - run[q];
     for (int v = 0; v < wid; ++v) off[q] += warp_tot[v][q];
-  }
-#pragma unroll
-  for (int u = 0; u < kMtPer; ++u) {
-    const int pi = mt_pad(tid * kMtPer + u);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) sc[q][pi] += off[q];
   }
   if (tid == kMtThreads - 1) {  // chunk totals
     pre[3 * blockIdx.x + 0] = off[0] + run[0];
     pre[3 * blockIdx.x + 1] = off[1] + run[1];
     pre[3 * blockIdx.x + 2] = (unsigned long long)(off[2] + run[2]) | ((unsigned long long)(off[3] + run[3]) << 32);
   }
+  if constexpr (QUERY) return;
+#pragma unroll
+  for (int u = 0; u < PER; ++u) {
+    const int pi = mt_pad(tid * PER + u);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) sc[q][pi] += off[q];
+  }
   __syncthreads();
 #pragma unroll 1
-  for (int u = 0; u < kMtPer; ++u) {
+  for (int u = 0; u < PER; ++u) {
     const int idx = u * kMtThreads + tid;
     const int64_t w = base + idx;
     if (w > nw) break;
@@ -1139,19 +1309,30 @@ __global__ void __launch_bounds__(1024) k_mt_chunks(unsigned long long* __restri
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   if (tid < 3) carry[tid] = 0;
   __syncthreads();
-  for (int64_t c0 = 0; c0 < n_chunks; c0 += 1024) {  // block-uniform trip count
-    const int64_t c = c0 + tid;
-    unsigned long long v[3], incl[3];
+  constexpr int V = 4;  // chunks a thread
+  for (int64_t c0 = 0; c0 < n_chunks; c0 += 1024 * V) {  // block-uniform trip count
+    const int64_t c = c0 + V * tid;
+    unsigned long long v[V][3], incl[3] = {};
+#pragma unroll
+    for (int u = 0; u < V; ++u)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) v[u][q] = c + u < n_chunks ? pre[3 * (c + u) + q] : 0ull;
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
-      v[q] = c < n_chunks ? pre[3 * c + q] : 0ull;
-      incl[q] = v[q];
+#pragma unroll
+      for (int u = 0; u < V; ++u) {  // each chunk's sum before it, of this thread's
+        const unsigned long long t = v[u][q];
+        v[u][q] = incl[q];
+        incl[q] += t;
+      }
+      const unsigned long long own = incl[q];
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const unsigned long long u = __shfl_up_sync(0xFFFFFFFFu, incl[q], o);
         if (lane >= o) incl[q] += u;
       }
       if (lane == 31) warp_tot[q][wid] = incl[q];
+      incl[q] -= own;
     }
     __syncthreads();
     if (wid == 0) {
@@ -1171,33 +1352,35 @@ __global__ void __launch_bounds__(1024) k_mt_chunks(unsigned long long* __restri
     }
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < 3; ++q)
-      if (c < n_chunks) pre[3 * c + q] = warp_tot[q][wid] + incl[q] - v[q];
+    for (int u = 0; u < V; ++u)
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        if (c + u < n_chunks) pre[3 * (c + u) + q] = warp_tot[q][wid] + incl[q] + v[u][q];
     __syncthreads();
   }
   if (tid < 3) pre[3 * n_chunks + tid] = carry[tid];
 }
 
 // the ids (32 w + b) of the samples with a vertex and of the cubes with a
-// triangle, in order
-__global__ void k_mt_list(const uint32_t* __restrict__ I, BitGrid m, const uint32_t* __restrict__ X,
-                          const unsigned long long* __restrict__ pre, const unsigned long long* __restrict__ loc_a,
-                          uint32_t* __restrict__ samples, uint32_t* __restrict__ cubes_out) {
+// triangle, in order; per word its active samples and the first one's place in
+// the list
+__global__ void k_mt_list(const uint32_t* __restrict__ I, BitGrid m, const uint32_t* __restrict__ A,
+                          const unsigned long long* __restrict__ pre, int chunk_log,
+                          const unsigned long long* __restrict__ loc_a, uint32_t* __restrict__ samples,
+                          uint32_t* __restrict__ cubes_out, uint2* __restrict__ places) {
   const int64_t nw = m.words();
   for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < nw;
        w += (int64_t)gridDim.x * blockDim.x) {
-    const unsigned long long b0 = pre[3 * (w >> kMtChunkLog) + 2] + loc_a[w];
-    const unsigned long long b1 = pre[3 * ((w + 1) >> kMtChunkLog) + 2] + loc_a[w + 1];
-    if (b0 == b1) continue;
-    uint32_t any = 0;
-#pragma unroll
-    for (int t = 0; t < 7; ++t) any |= X[t * nw + w];
+    const unsigned long long b0 = pre[3 * (w >> chunk_log) + 2] + loc_a[w];
+    const unsigned long long b1 = pre[3 * ((w + 1) >> chunk_log) + 2] + loc_a[w + 1];
+    const uint32_t any = A[w];
     uint32_t pos = (uint32_t)(b0 & 0xFFFFFFFFull);
+    places[w] = make_uint2(any, pos);
+    if (b0 == b1) continue;
     for (uint32_t M = any; M; M &= M - 1) samples[pos++] = (uint32_t)w * 32u + (uint32_t)(__ffs(M) - 1);
     if ((b0 >> 32) == (b1 >> 32)) continue;
-    const uint32_t row = (uint32_t)w / (uint32_t)m.mw;
-    const int xw = (int)((uint32_t)w - row * (uint32_t)m.mw);
-    const int j = (int)(row % (uint32_t)m.ny), k = (int)(row / (uint32_t)m.ny);
+    int j, k, xw;
+    word_coords(m, (uint32_t)w, &j, &k, &xw);
     uint32_t C[8];
     corner_words(I, m, j, k, xw, C);
     pos = (uint32_t)(b0 >> 32);
@@ -1215,246 +1398,321 @@ struct EmitArgs {
   const uint32_t* I;
   const uint32_t* X;
   const unsigned long long* pre;  // chunk prefixes (see k_mt_count)
+  int chunk_log;                  // log2 of the words a chunk
   const uint32_t* loc_v;
   const uint32_t* loc_t;
+  const uint2* places;  // per word: active samples, the first one's list place
+  uint2* first;         // per listed sample: first vertex, edge types (bit t)
   float* verts;
   int32_t* tris;
   float* normals;
   int64_t n_verts, n_tris;  // totals: every write is checked against them
 };
 
-__device__ __forceinline__ float sample_phi(const EmitArgs& a, int x, int j, int k) {
-  return a.phi[((int64_t)k * a.step * a.ny + (int64_t)j * a.step) * a.nx + (int64_t)x * a.step];
-}
+// the vertex a warp emits: from its samples' positions, values and gradients
+struct MtSample {
+  int x, j, k;
+  float f, g[3];
+};
 
-// central-difference gradient of phi on the sample grid (one-sided on the border)
-__device__ void sample_grad(const EmitArgs& a, int x, int j, int k, float g[3]) {
+// central-difference gradient of phi on the sample grid (one-sided on the
+// border) at the sample p points to
+__device__ __forceinline__ void sample_grad(const EmitArgs& a, const float* p, int x, int j, int k, int64_t sy,
+                                            int64_t sz, float g[3]) {
   const int c[3] = {x, j, k}, lim[3] = {a.m.nx, a.m.ny, a.m.nz};
+  const int64_t stride[3] = {a.step, sy, sz};
 #pragma unroll
   for (int ax = 0; ax < 3; ++ax) {
-    int lo[3] = {x, j, k}, hi[3] = {x, j, k};
-    if (c[ax] > 0) lo[ax] -= 1;
-    if (c[ax] < lim[ax] - 1) hi[ax] += 1;
-    const int span = hi[ax] - lo[ax];
-    g[ax] = span > 0 ? (sample_phi(a, hi[0], hi[1], hi[2]) - sample_phi(a, lo[0], lo[1], lo[2])) /
-                           ((float)(span * a.step) * a.h)
-                     : 0.f;
+    const int lo = c[ax] > 0 ? 1 : 0, hi = c[ax] < lim[ax] - 1 ? 1 : 0;
+    g[ax] = lo + hi > 0 ? (p[hi ? stride[ax] : 0] - p[lo ? -stride[ax] : 0]) / ((float)((lo + hi) * a.step) * a.h) : 0.f;
   }
 }
-
-__device__ void emit_vertex(const EmitArgs& a, int x, int j, int k, int t, int64_t id) {
-  if (id >= a.n_verts) return;
-  const int dx = t & 1, dy = (t >> 1) & 1, dz = (t >> 2) & 1;
-  const float fa = sample_phi(a, x, j, k), fb = sample_phi(a, x + dx, j + dy, k + dz);
-  const float tau = (a.iso - fa) / (fb - fa);
-  const float span = (float)a.step * a.h;
-  float p[3] = {a.ox + ((float)(x * a.step) + 0.5f) * a.h, a.oy + ((float)(j * a.step) + 0.5f) * a.h,
-                a.oz + ((float)(k * a.step) + 0.5f) * a.h};
-  if (dx) p[0] += tau * span;
-  if (dy) p[1] += tau * span;
-  if (dz) p[2] += tau * span;
-  a.verts[id * 3 + 0] = p[0];
-  a.verts[id * 3 + 1] = p[1];
-  a.verts[id * 3 + 2] = p[2];
-  if (a.normals) {
-    float ga[3], gb[3], n[3];
-    sample_grad(a, x, j, k, ga);
-    sample_grad(a, x + dx, j + dy, k + dz, gb);
-    float len2 = 0.f;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      n[c] = (1.f - tau) * ga[c] + tau * gb[c];
-      len2 += n[c] * n[c];
-    }
-    const float len = sqrtf(len2);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) a.normals[id * 3 + c] = len > 0.f ? n[c] / len : 0.f;
-  }
-}
-
-__device__ __forceinline__ int3 corner_xyz(int c) { return make_int3(c & 1, (c >> 1) & 1, (c >> 2) & 1); }
 
 // Triangle table: for tetrahedron T (corners 0, kTetMid[T][0], kTetMid[T][1],
 // 7 at positions 0..3) and the inside pattern of those corners (bit q =
-// position q inside), its triangles, each as the three tetrahedron edges its
-// vertices lie on, in output order.  Edge numbers: 0 (0,1) 1 (0,2) 2 (0,3)
-// 3 (1,2) 4 (1,3) 5 (2,3) in positions.  Entry: bits 0-1 the count, triangle
-// m at bits 2 + 9 m, its vertex v at 3 v within.
+// position q inside), its triangles in output order.  A triangle's vertex v is
+// the edge of type t from corner lo: bits 6 v .. 6 v + 2 hold lo, the next
+// three t; bits 18-19 of the first entry the count.
 //   one corner on its side: one triangle on the three edges from that
 //     corner, the others in position order;
 //   two inside: two triangles (i0,o0)(i0,o1)(i1,o1) and (i0,o0)(i1,o1)(i1,o0);
 //   each oriented so its normal points from the inside corners to the outside
 //   ones (integer cross product of the doubled edge midpoints).
-__device__ __forceinline__ int tet_edge(int qa, int qb) {
-  const int lo = min(qa, qb), hi = max(qa, qb);
-  return lo == 0 ? hi - 1 : lo + hi;  // (0,1) 0 (0,2) 1 (0,3) 2 (1,2) 3 (1,3) 4 (2,3) 5
-}
+struct TetTable {
+  uint32_t tri[6 * 16][2];
+};
 
-__device__ uint32_t tet_triangle(const int tet[4], const bool in[4], const int e[3][2]) {
-  int3 mp[3];  // doubled edge midpoints
-#pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    const int3 u = corner_xyz(tet[e[q][0]]), v = corner_xyz(tet[e[q][1]]);
-    mp[q] = make_int3(u.x + v.x, u.y + v.y, u.z + v.z);
-  }
-  int nin = 0;
-  int3 sin = make_int3(0, 0, 0), sout = make_int3(0, 0, 0);
-#pragma unroll
+constexpr int corner_axis(int c, int axis) { return (c >> axis) & 1; }
+
+constexpr uint32_t tet_triangle(const int (&tet)[4], const bool (&in)[4], const int (&e)[3][2]) {
+  int mp[3][3] = {}, sin[3] = {}, sout[3] = {}, nin = 0;  // doubled edge midpoints, sums of the corners
+  for (int q = 0; q < 3; ++q)
+    for (int x = 0; x < 3; ++x) mp[q][x] = corner_axis(tet[e[q][0]], x) + corner_axis(tet[e[q][1]], x);
   for (int q = 0; q < 4; ++q) {
-    const int3 c = corner_xyz(tet[q]);
-    if (in[q]) {
-      ++nin;
-      sin.x += c.x, sin.y += c.y, sin.z += c.z;
-    } else {
-      sout.x += c.x, sout.y += c.y, sout.z += c.z;
-    }
+    nin += in[q] ? 1 : 0;
+    for (int x = 0; x < 3; ++x) (in[q] ? sin : sout)[x] += corner_axis(tet[q], x);
   }
-  const int nout = 4 - nin;
-  const int3 G = make_int3(nin * sout.x - nout * sin.x, nin * sout.y - nout * sin.y, nin * sout.z - nout * sin.z);
-  const int3 U = make_int3(mp[1].x - mp[0].x, mp[1].y - mp[0].y, mp[1].z - mp[0].z);
-  const int3 V = make_int3(mp[2].x - mp[0].x, mp[2].y - mp[0].y, mp[2].z - mp[0].z);
-  const int3 N = make_int3(U.y * V.z - U.z * V.y, U.z * V.x - U.x * V.z, U.x * V.y - U.y * V.x);
-  const bool flip = N.x * G.x + N.y * G.y + N.z * G.z < 0;
-  const int order[3] = {0, flip ? 2 : 1, flip ? 1 : 2};
+  int G[3] = {}, U[3] = {}, V[3] = {};
+  for (int x = 0; x < 3; ++x) {
+    G[x] = nin * sout[x] - (4 - nin) * sin[x];
+    U[x] = mp[1][x] - mp[0][x];
+    V[x] = mp[2][x] - mp[0][x];
+  }
+  const int along = (U[1] * V[2] - U[2] * V[1]) * G[0] + (U[2] * V[0] - U[0] * V[2]) * G[1] +
+                    (U[0] * V[1] - U[1] * V[0]) * G[2];
+  const int order[3] = {0, along < 0 ? 2 : 1, along < 0 ? 1 : 2};
   uint32_t code = 0;
-#pragma unroll
-  for (int v = 0; v < 3; ++v) code |= (uint32_t)tet_edge(e[order[v]][0], e[order[v]][1]) << (3 * v);
+  for (int v = 0; v < 3; ++v) {
+    const int qa = e[order[v]][0], qb = e[order[v]][1];
+    const int lo = tet[qa < qb ? qa : qb], hi = tet[qa < qb ? qb : qa];
+    code |= ((uint32_t)lo | (uint32_t)(hi ^ lo) << 3) << (6 * v);
+  }
   return code;
 }
 
-__device__ uint32_t tet_entry(int T, int pat) {
-  const int tet[4] = {0, kTetMid[T][0], kTetMid[T][1], 7};
-  bool in[4];
-  int nin = 0;
-  for (int q = 0; q < 4; ++q) {
-    in[q] = (pat >> q) & 1;
-    nin += in[q];
-  }
-  if (nin == 0 || nin == 4) return 0;
-  if (nin & 1) {
-    const bool lone_in = nin == 1;
-    int lone = 0, o[3], no = 0;
-    for (int q = 0; q < 4; ++q) {
-      if (in[q] == lone_in) lone = q;
-      else o[no++] = q;
+constexpr TetTable make_tet_table() {
+  constexpr int mid[6][2] = {{1, 3}, {1, 5}, {2, 3}, {2, 6}, {4, 5}, {4, 6}};  // kTetMid
+  TetTable tab{};
+  for (int T = 0; T < 6; ++T)
+    for (int pat = 1; pat < 15; ++pat) {
+      const int tet[4] = {0, mid[T][0], mid[T][1], 7};
+      bool in[4] = {};
+      int ins[4] = {}, outs[4] = {}, ni = 0, no = 0;
+      for (int q = 0; q < 4; ++q) {
+        in[q] = (pat >> q) & 1;
+        if (in[q]) ins[ni++] = q;
+        else outs[no++] = q;
+      }
+      uint32_t* tri = tab.tri[T * 16 + pat];
+      if (ni == 2) {
+        const int e1[3][2] = {{ins[0], outs[0]}, {ins[0], outs[1]}, {ins[1], outs[1]}};
+        const int e2[3][2] = {{ins[0], outs[0]}, {ins[1], outs[1]}, {ins[1], outs[0]}};
+        tri[0] = tet_triangle(tet, in, e1) | 2u << 18;
+        tri[1] = tet_triangle(tet, in, e2);
+      } else {
+        const int lone = ni == 1 ? ins[0] : outs[0];
+        const int* o = ni == 1 ? outs : ins;
+        const int e[3][2] = {{lone, o[0]}, {lone, o[1]}, {lone, o[2]}};
+        tri[0] = tet_triangle(tet, in, e) | 1u << 18;
+      }
     }
-    const int e[3][2] = {{lone, o[0]}, {lone, o[1]}, {lone, o[2]}};
-    return 1u | tet_triangle(tet, in, e) << 2;
-  }
-  int ins[2], outs[2], ni = 0, nu = 0;
-  for (int q = 0; q < 4; ++q) {
-    if (in[q]) ins[ni++] = q;
-    else outs[nu++] = q;
-  }
-  const int e1[3][2] = {{ins[0], outs[0]}, {ins[0], outs[1]}, {ins[1], outs[1]}};
-  const int e2[3][2] = {{ins[0], outs[0]}, {ins[1], outs[1]}, {ins[1], outs[0]}};
-  return 2u | tet_triangle(tet, in, e1) << 2 | tet_triangle(tet, in, e2) << 11;
+  return tab;
 }
 
-// word id -> (j, k, xw) of the sample grid
-__device__ __forceinline__ void word_coords(const BitGrid& m, uint32_t w, int* j, int* k, int* xw) {
-  const uint32_t row = w / (uint32_t)m.mw;
-  *xw = (int)(w - row * (uint32_t)m.mw);
-  *j = (int)(row % (uint32_t)m.ny);
-  *k = (int)(row / (uint32_t)m.ny);
+__device__ const TetTable kTetTable = make_tet_table();
+
+// Three words for each of a warp's n items (n <= 32 a call, the lane's own in
+// v) to dst, 12 bytes an item, in whole lines; words past `limit` are dropped.
+__device__ __forceinline__ void store3(uint32_t* stage, const uint32_t v[3], int n, uint32_t* dst, int64_t first,
+                                       int64_t limit) {
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+#pragma unroll
+  for (int c = 0; c < 3; ++c) stage[3 * lane + c] = v[c];
+  __syncwarp();
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int i = 32 * c + lane;
+    if (i < 3 * n && 3 * first + i < 3 * limit) dst[3 * first + i] = stage[i];
+  }
 }
 
-// one thread per sample with a vertex: its vertices, by type, from the
-// word's vertex offset and the crossings of the lower samples in the word
-__global__ void k_mt_verts(EmitArgs a, const uint32_t* __restrict__ samples, uint32_t n_samples) {
+// A warp takes 32 samples with a vertex at once: a lane a sample for its edge
+// types, value and gradient, then a lane a vertex (1 to 7 a sample), written in
+// whole lines -- the samples' vertices lie next to each other, as their list
+// does.  Bound by issue and the latency of the gathers from phi.  1.3 M
+// vertices with normals: 83 us (a thread a sample, its vertices in turn) -> 54.
+constexpr int kMtWarps = 8;
+
+template <bool NORMALS>
+__global__ void __launch_bounds__(32 * kMtWarps) k_mt_verts(EmitArgs a, const uint32_t* __restrict__ samples,
+                                                            uint32_t n_samples) {
+  __shared__ MtSample s_sample[kMtWarps][32];
+  __shared__ uint8_t s_vert[kMtWarps][7 * 32];  // sample << 3 | type
+  __shared__ uint32_t s_out[kMtWarps][96];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t nw = a.m.words();
-  for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < n_samples; q += gridDim.x * blockDim.x) {
-    const uint32_t id = samples[q], w = id >> 5, b = id & 31u;
-    int j, k, xw;
-    word_coords(a.m, w, &j, &k, &xw);
-    uint32_t ty = 0, before = 0;
-#pragma unroll
-    for (int t = 1; t <= 7; ++t) {
-      const uint32_t xt = a.X[(t - 1) * nw + w];
-      ty |= ((xt >> b) & 1u) << t;
-      before += __popc(xt & ((1u << b) - 1u));
-    }
-    int64_t vid = (int64_t)mt_base(a.pre, 0, a.loc_v[w], w) + before;
-#pragma unroll 1
-    for (int t = 1; t <= 7; ++t)
-      if ((ty >> t) & 1u) emit_vertex(a, xw * 32 + (int)b, j, k, t, vid++);
-  }
-}
-
-// one thread per cube with a triangle: its triangles by tetrahedron, from
-// the word's triangle offset plus the bit-sliced count of the lower cubes.
-// Corner c = dx + 2 dy + 4 dz owns the edges of types t from its sample; its
-// first vertex is the word's vertex offset plus the crossings of the lower
-// samples of the word.  Corners 0..6 sit in four words (one a (dy, dz)
-// row; the dx = 1 corner in the next word when x is its word's last bit).
-// Each thread keeps its corners' (first vertex, edge types) in its own
-// column of shared memory, so a vertex can name its corner at run time.
-constexpr int kMtTriThreads = 256;
-
-__global__ void __launch_bounds__(kMtTriThreads) k_mt_tris(EmitArgs a, const uint32_t* __restrict__ cubes_in,
-                                                           uint32_t n_cubes) {
-  __shared__ uint32_t s_tet[6 * 16];
-  __shared__ uint32_t s_first[7][kMtTriThreads], s_types[7][kMtTriThreads];
-  for (int i = threadIdx.x; i < 6 * 16; i += blockDim.x) s_tet[i] = tet_entry(i >> 4, i & 15);
-  __syncthreads();
-  const int tx = threadIdx.x;
-  const int64_t nw = a.m.words();
-  for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < n_cubes; q += gridDim.x * blockDim.x) {
-    const uint32_t id = cubes_in[q], w = id >> 5;
-    const int b = (int)(id & 31u);
-    int j, k, xw;
-    word_coords(a.m, w, &j, &k, &xw);
-    uint32_t C[8];
-    corner_words(a.I, a.m, j, k, xw, C);
-    const uint32_t below = (1u << b) - 1u;
-    int64_t tid = (int64_t)mt_base(a.pre, 1, a.loc_t[w], w) + tri_count(C, cube_bits(a.m, j, k, xw) & below);
-    uint32_t cb = 0;  // bit c: corner c inside
-#pragma unroll
-    for (int c = 0; c < 8; ++c) cb |= ((C[c] >> b) & 1u) << c;
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {  // rows (dy, dz) = (r & 1, r >> 1)
-      const int c0 = 2 * (r & 1) + 4 * (r >> 1);
-      const int64_t wr = ((int64_t)(k + (r >> 1)) * a.m.ny + (j + (r & 1))) * a.m.mw + xw;
-      uint32_t f = (uint32_t)mt_base(a.pre, 0, a.loc_v[wr], wr), ty = 0, ty1 = 0;
+  const int64_t sy = (int64_t)a.step * a.nx, sz = sy * a.ny;
+  for (uint32_t q0 = (blockIdx.x * kMtWarps + wid) * 32; q0 < n_samples; q0 += gridDim.x * kMtWarps * 32) {
+    const uint32_t q = q0 + lane;
+    const bool some = q < n_samples;
+    uint32_t ty = 0, before = 0, w = 0;
+    __syncwarp();
+    if (some) {
+      const uint32_t id = samples[q], b = id & 31u;
+      w = id >> 5;
+      MtSample me;
+      word_coords(a.m, w, &me.j, &me.k, &me.x);
+      me.x = me.x * 32 + (int)b;
 #pragma unroll
       for (int t = 1; t <= 7; ++t) {
-        const uint32_t xt = __ldg(a.X + (t - 1) * nw + wr);
-        f += __popc(xt & below);
+        const uint32_t xt = a.X[(t - 1) * nw + w];
         ty |= ((xt >> b) & 1u) << t;
-        if (b < 31) ty1 |= ((xt >> (b + 1)) & 1u) << t;
+        before += __popc(xt & ((1u << b) - 1u));
       }
-      s_first[c0][tx] = f;
-      s_types[c0][tx] = ty;
-      if (c0 + 1 < 7) {  // the dx = 1 corner
-        uint32_t f1 = f + __popc(ty);
-        if (b == 31) {
-          f1 = (uint32_t)mt_base(a.pre, 0, a.loc_v[wr + 1], wr + 1);
+      const float* p = a.phi + (me.k * sz + me.j * sy + (int64_t)me.x * a.step);
+      me.f = *p;
+      if (NORMALS) sample_grad(a, p, me.x, me.j, me.k, sy, sz, me.g);
+      s_sample[wid][lane] = me;
+    }
+    int64_t vid0 = 0;  // the warp's first vertex
+    if (lane == 0) vid0 = (int64_t)(a.pre[3 * (w >> a.chunk_log)] + a.loc_v[w] + before);
+    vid0 = __shfl_sync(0xFFFFFFFFu, vid0, 0);
+    const int n = __popc(ty);
+    int off = n;
 #pragma unroll
-          for (int t = 1; t <= 7; ++t) ty1 |= (__ldg(a.X + (t - 1) * nw + wr + 1) & 1u) << t;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xFFFFFFFFu, off, o);
+      if (lane >= o) off += u;
+    }
+    const int total = __shfl_sync(0xFFFFFFFFu, off, 31);
+    off -= n;
+    if (some) a.first[q] = make_uint2((uint32_t)(vid0 + off), ty);
+    for (uint32_t m = ty; m; m &= m - 1) s_vert[wid][off++] = (uint8_t)(lane << 3 | (__ffs(m) - 1));
+    __syncwarp();
+    for (int v0 = 0; v0 < total; v0 += 32) {
+      const int n_now = min(32, total - v0);
+      float pos[3] = {}, nrm[3] = {};
+      if (lane < n_now) {
+        const int e = s_vert[wid][v0 + lane], t = e & 7;
+        const MtSample& me = s_sample[wid][e >> 3];
+        const int dx = t & 1, dy = t >> 1 & 1, dz = t >> 2;
+        const int x = me.x + dx, j = me.j + dy, k = me.k + dz;
+        const float* p = a.phi + (k * sz + j * sy + (int64_t)x * a.step);
+        const float tau = (a.iso - me.f) / (*p - me.f);
+        const float span = (float)a.step * a.h;
+        // contracted by hand: with and without normals give the same vertices
+        pos[0] = fmaf((float)(me.x * a.step) + 0.5f, a.h, a.ox);
+        pos[1] = fmaf((float)(me.j * a.step) + 0.5f, a.h, a.oy);
+        pos[2] = fmaf((float)(me.k * a.step) + 0.5f, a.h, a.oz);
+        if (dx) pos[0] = fmaf(tau, span, pos[0]);
+        if (dy) pos[1] = fmaf(tau, span, pos[1]);
+        if (dz) pos[2] = fmaf(tau, span, pos[2]);
+        if (NORMALS) {
+          float g[3];
+          sample_grad(a, p, x, j, k, sy, sz, g);
+          float len2 = 0.f;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            nrm[c] = (1.f - tau) * me.g[c] + tau * g[c];
+            len2 += nrm[c] * nrm[c];
+          }
+          const float len = sqrtf(len2);
+#pragma unroll
+          for (int c = 0; c < 3; ++c) nrm[c] = len > 0.f ? nrm[c] / len : 0.f;
         }
-        s_first[c0 + 1][tx] = f1;
-        s_types[c0 + 1][tx] = ty1;
+      }
+      uint32_t bits[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) bits[c] = __float_as_uint(pos[c]);
+      store3(s_out[wid], bits, n_now, (uint32_t*)a.verts, vid0 + v0, a.n_verts);
+      if (NORMALS) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) bits[c] = __float_as_uint(nrm[c]);
+        store3(s_out[wid], bits, n_now, (uint32_t*)a.normals, vid0 + v0, a.n_verts);
       }
     }
-#pragma unroll 1
+  }
+}
+
+// A warp takes 32 cubes with a triangle at once: a lane a cube for its corners'
+// first vertices and edge types (looked up by the corner sample's place in the
+// list) and its triangles' table codes, then a lane a triangle (1 to 12 a
+// cube), written in whole lines.  Corner c = dx + 2 dy + 4 dz owns the edges of
+// types t from its sample; corners 0..6 sit in four words (one a (dy, dz) row;
+// the dx = 1 corner in the next word when x is its word's last bit).  2.6 M
+// triangles: 66 us (a thread a cube, its triangles in turn, the corners'
+// vertices counted from the seven crossing words each) -> 34.
+__global__ void __launch_bounds__(32 * kMtWarps) k_mt_tris(EmitArgs a, const uint32_t* __restrict__ cubes_in,
+                                                           uint32_t n_cubes) {
+  __shared__ uint32_t s_tet[6 * 16][2];
+  __shared__ uint2 s_corner[kMtWarps][32][7];   // first vertex, edge types
+  __shared__ uint32_t s_tri[kMtWarps][12 * 32];  // code | cube << 20
+  __shared__ uint32_t s_out[kMtWarps][96];
+  for (int i = threadIdx.x; i < 6 * 16 * 2; i += blockDim.x) (&s_tet[0][0])[i] = (&kTetTable.tri[0][0])[i];
+  __syncthreads();
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t plane = (int64_t)a.m.mw * a.m.ny;
+  for (uint32_t q0 = (blockIdx.x * kMtWarps + wid) * 32; q0 < n_cubes; q0 += gridDim.x * kMtWarps * 32) {
+    const uint32_t q = q0 + lane;
+    uint32_t cb = 0;  // bit c: corner c inside
+    int64_t tid0 = 0;  // the warp's first triangle
+    __syncwarp();
+    if (q < n_cubes) {
+      const uint32_t id = cubes_in[q], w = id >> 5;
+      const int b = (int)(id & 31u);
+      const uint32_t below = (1u << b) - 1u;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {  // rows (dy, dz) = (r & 1, r >> 1)
+        const int c0 = 2 * (r & 1) + 4 * (r >> 1);
+        const int64_t wr = w + (r & 1) * a.m.mw + (r >> 1) * plane;
+        uint2 at = __ldg(a.places + wr);
+        uint32_t in = __ldg(a.I + wr);
+        cb |= ((in >> b) & 1u) << c0;
+        uint32_t pos = at.y + __popc(at.x & below);
+        uint2 fv = make_uint2(0u, 0u);
+        if ((at.x >> b) & 1u) fv = __ldg(a.first + pos++);
+        s_corner[wid][lane][c0] = fv;
+        int b1 = b + 1;
+        if (b1 == 32) {  // a cube's row goes on in the next word
+          at = __ldg(a.places + wr + 1);
+          in = __ldg(a.I + wr + 1);
+          pos = at.y;
+          b1 = 0;
+        }
+        cb |= ((in >> b1) & 1u) << (c0 + 1);
+        if (c0 + 1 < 7) {
+          fv = make_uint2(0u, 0u);
+          if ((at.x >> b1) & 1u) fv = __ldg(a.first + pos);
+          s_corner[wid][lane][c0 + 1] = fv;
+        }
+      }
+      if (lane == 0) {
+        int j, k, xw;
+        word_coords(a.m, w, &j, &k, &xw);
+        uint32_t C[8];
+        corner_words(a.I, a.m, j, k, xw, C);
+        tid0 = (int64_t)(a.pre[3 * (w >> a.chunk_log) + 1] + a.loc_t[w]) + tri_count(C, cube_bits(a.m, j, k, xw) & below);
+      }
+    }
+    tid0 = __shfl_sync(0xFFFFFFFFu, tid0, 0);
+    int n = 0;
+    uint32_t ent[6];
+#pragma unroll
     for (int T = 0; T < 6; ++T) {
       const int m0 = kTetMid[T][0], m1 = kTetMid[T][1];
       const uint32_t pat = (cb & 1u) | ((cb >> m0) & 1u) << 1 | ((cb >> m1) & 1u) << 2 | ((cb >> 7) & 1u) << 3;
-      const uint32_t ent = s_tet[T * 16 + pat];
-      for (uint32_t m = 0; m < (ent & 3u); ++m, ++tid) {
-        const uint32_t code = ent >> (2 + 9 * m);
-        if (tid >= a.n_tris) continue;
+      ent[T] = T * 16 + pat;
+      n += (int)(s_tet[ent[T]][0] >> 18);
+    }
+    int off = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xFFFFFFFFu, off, o);
+      if (lane >= o) off += u;
+    }
+    const int total = __shfl_sync(0xFFFFFFFFu, off, 31);
+    off -= n;
+#pragma unroll
+    for (int T = 0; T < 6; ++T) {
+      const uint32_t t0 = s_tet[ent[T]][0], some = t0 >> 18;
+      if (some) s_tri[wid][off++] = (t0 & 0x3FFFFu) | (uint32_t)lane << 20;
+      if (some > 1) s_tri[wid][off++] = s_tet[ent[T]][1] | (uint32_t)lane << 20;
+    }
+    __syncwarp();
+    for (int v0 = 0; v0 < total; v0 += 32) {
+      const int n_now = min(32, total - v0);
+      uint32_t id[3] = {};
+      if (lane < n_now) {
+        const uint32_t code = s_tri[wid][v0 + lane];
+        const uint2* corner = s_corner[wid][code >> 20];
 #pragma unroll
         for (int v = 0; v < 3; ++v) {
-          // edge e joins positions (qa, qb), qa < qb; position q is corner 0, m0, m1 or 7
-          const int e = (int)((code >> (3 * v)) & 7u);
-          const int qa = e < 3 ? 0 : (e < 5 ? 1 : 2), qb = e < 3 ? e + 1 : (e < 5 ? e - 1 : 3);
-          const int lo = qa == 0 ? 0 : (qa == 1 ? m0 : m1);
-          const int hi = qb == 1 ? m0 : (qb == 2 ? m1 : 7);
-          const int t = hi ^ lo;
-          a.tris[tid * 3 + v] = (int32_t)(s_first[lo][tx] + __popc(s_types[lo][tx] & ((1u << t) - 1u)));
+          const uint2 fv = corner[(code >> (6 * v)) & 7u];
+          id[v] = fv.x + __popc(fv.y & ((1u << ((code >> (6 * v + 3)) & 7u)) - 1u));
         }
       }
+      store3(s_out[wid], id, n_now, (uint32_t*)a.tris, tid0 + v0, a.n_tris);
     }
   }
 }
@@ -1468,7 +1726,7 @@ struct Buf {
 };
 
 struct Scratch {
-  Buf bits_a, bits_b, shells, parent, tiles, x_words, cnt_v, cnt_t, cnt_a, lists, scan_tmp, blur_a, blur_b, sel;
+  Buf bits_a, bits_b, shells, parent, tiles, x_words, a_words, places, cnt_v, cnt_t, cnt_a, lists, scan_tmp, blur_a, blur_b, sel;
   int* err = nullptr;        // device: union-find limit reached (bits 0/1 global find/unite, 2/3 in a tile)
   unsigned long long* host = nullptr;  // pinned: [2] the TSDF error flag, [4..6] the mesh totals read back
   cudaEvent_t err_ready = nullptr;     // recorded after the flag's copy to host[2]
@@ -1688,13 +1946,16 @@ extern "C" fgl_status fgl_tsdf(const uint8_t* surf, const fgl_grid* grid, float 
   MCUDA(ensure(S.bits_a, sizeof(uint32_t) * nw, s));
   MCUDA(ensure(S.bits_b, sizeof(uint32_t) * nw, s));
   const int n_planes = 32 - __builtin_clz((unsigned)(L + 1));  // bits of the count L + 1
-  MCUDA(ensure(S.shells, sizeof(uint32_t) * nw * (2 + n_planes), s));
+  // wider bands, whose halo would be most of a tile, and grids past a launch's
+  // limits go mask by mask
+  const ShellPlan sp = plan_shells(g, L);
+  const bool tiled_shells = L <= kTileShells && sp.grid.y <= 65535u && sp.grid.z <= 65535u;
+  if (!tiled_shells) MCUDA(ensure(S.shells, sizeof(uint32_t) * nw * (2 + n_planes), s));
   MCUDA(ensure(S.parent, sizeof(uint32_t) * (n + 1), s));
   const TilePlan tp = plan_tiles(g);
   if (tp.ty) MCUDA(ensure(S.tiles, (size_t)tp.n_tiles, s));
   uint32_t* Vb = (uint32_t*)S.bits_a.p;
   uint32_t* Ob = (uint32_t*)S.bits_b.p;
-  uint32_t* D = (uint32_t*)S.shells.p;
   uint32_t* parent = (uint32_t*)S.parent.p;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   const bool timing = stats && stats->timing;
@@ -1719,15 +1980,22 @@ extern "C" fgl_status fgl_tsdf(const uint8_t* surf, const fgl_grid* grid, float 
     launches += 3;
   }
   k_run_outside<<<rb, 256, 0, s>>>(Vb, g, parent, Ob, S.err);
-  uint32_t* Dm[2] = {D, D + nw};       // ping-pong shell masks
-  uint32_t* planes = D + 2 * nw;       // bit-sliced counts of the masks holding each voxel
-  k_s0<<<word_blocks(nw, 256), 256, 0, s>>>(Vb, g, Dm[0], planes, n_planes);
-  launches += 2;
-  for (int m = 1; m <= L; ++m, ++launches)
-    k_dilate<<<word_blocks(nw, 256), 256, 0, s>>>(Dm[(m - 1) & 1], g, Dm[m & 1], planes, n_planes);
+  ++launches;
   const float off = stats && stats->delta_mode == 1 ? 0.f : 0.5f;
-  k_phi<<<word_blocks(nw, 256), 256, 0, s>>>(Ob, planes, L, g, grid->h, trunc, off, out_phi,
-                                             out_outside, out_shell);
+  if (tiled_shells) {
+    auto* shell_phi = out_outside || out_shell ? k_shell_phi<true> : k_shell_phi<false>;
+    shell_phi<<<sp.grid, kShellThreads, sp.smem, s>>>(Vb, Ob, L, g, sp.tw, grid->h, trunc, off, out_phi, out_outside,
+                                                      out_shell);
+  } else {
+    uint32_t* D = (uint32_t*)S.shells.p;
+    uint32_t* Dm[2] = {D, D + nw};  // ping-pong shell masks
+    uint32_t* planes = D + 2 * nw;  // bit-sliced counts of the masks holding each voxel
+    k_s0<<<word_blocks(nw, 256), 256, 0, s>>>(Vb, g, Dm[0], planes, n_planes);
+    ++launches;
+    for (int m = 1; m <= L; ++m, ++launches)
+      k_dilate<<<word_blocks(nw, 256), 256, 0, s>>>(Dm[(m - 1) & 1], g, Dm[m & 1], planes, n_planes);
+    k_phi<<<word_blocks(nw, 256), 256, 0, s>>>(Ob, planes, L, g, grid->h, trunc, off, out_phi, out_outside, out_shell);
+  }
   ++launches;
   MCUDA(cudaGetLastError());
   MCUDA(cudaMemcpyAsync(S.host + 2, S.err, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -1773,21 +2041,32 @@ extern "C" fgl_status fgl_marching_tets(const float* phi, const fgl_grid* grid, 
   Scratch& S = *get_scratch(s);
   std::lock_guard<std::mutex> lk(S.mu);
   MCUDA(ensure_small(S));
-  const int64_t n_chunks = nw / kMtChunk + 1;  // positions 0 .. nw
+  // Words a thread counts: one where there are few (12,000 words: 6 us; eight,
+  // 15); four beyond 2^17, so that one block's pass over the chunks' totals
+  // stays short (0.85 M words: 24 + 7 us; with one word 23 + 12).
+  const int per = nw <= ((int64_t)1 << 17) ? 1 : 4, chunk_log = per == 1 ? 8 : 10;
+  const int64_t n_chunks = (nw >> chunk_log) + 1;  // positions 0 .. nw
   MCUDA(ensure(S.bits_a, sizeof(uint32_t) * nw, s));
-  MCUDA(ensure(S.x_words, sizeof(uint32_t) * nw * 7, s));
-  MCUDA(ensure(S.cnt_v, sizeof(uint32_t) * (nw + 1), s));
-  MCUDA(ensure(S.cnt_t, sizeof(uint32_t) * (nw + 1), s));
-  MCUDA(ensure(S.cnt_a, sizeof(unsigned long long) * (nw + 1), s));
+  if (!query) {
+    MCUDA(ensure(S.x_words, sizeof(uint32_t) * nw * 7, s));
+    MCUDA(ensure(S.a_words, sizeof(uint32_t) * nw, s));
+    MCUDA(ensure(S.cnt_v, sizeof(uint32_t) * (nw + 1), s));
+    MCUDA(ensure(S.cnt_t, sizeof(uint32_t) * (nw + 1), s));
+    MCUDA(ensure(S.cnt_a, sizeof(unsigned long long) * (nw + 1), s));
+  }
   MCUDA(ensure(S.scan_tmp, sizeof(unsigned long long) * 3 * (n_chunks + 1), s));
   uint32_t* I = (uint32_t*)S.bits_a.p;
   uint32_t* X = (uint32_t*)S.x_words.p;
+  uint32_t* A = (uint32_t*)S.a_words.p;
   auto* lv = (uint32_t*)S.cnt_v.p;
   auto* lt = (uint32_t*)S.cnt_t.p;
   auto* la = (unsigned long long*)S.cnt_a.p;
   auto* pre = (unsigned long long*)S.scan_tmp.p;
-  k_pack_inside<<<word_blocks(m.rows() * 32, 256), 256, 0, s>>>(phi, nx, ny, step, m, iso, I);
-  k_mt_count<<<(unsigned)n_chunks, kMtThreads, 0, s>>>(I, m, X, lv, lt, la, pre);
+  auto* pack = step == 1 ? k_pack_inside<true> : k_pack_inside<false>;
+  pack<<<word_blocks(m.rows() * 32, 256), 256, 0, s>>>(phi, nx, ny, step, m, iso, I);
+  auto* count = per == 1 ? (query ? k_mt_count<1, true> : k_mt_count<1, false>)
+                         : (query ? k_mt_count<4, true> : k_mt_count<4, false>);
+  count<<<(unsigned)n_chunks, kMtThreads, 0, s>>>(I, m, X, A, lv, lt, la, pre);
   k_mt_chunks<<<1, 1024, 0, s>>>(pre, n_chunks);
   MCUDA(cudaGetLastError());
   // totals: vertices, triangles, active samples | active cubes
@@ -1817,6 +2096,7 @@ extern "C" fgl_status fgl_marching_tets(const float* phi, const fgl_grid* grid, 
   a.I = I;
   a.X = X;
   a.pre = pre;
+  a.chunk_log = chunk_log;
   a.loc_v = lv;
   a.loc_t = lt;
   a.verts = out_verts;
@@ -1824,12 +2104,19 @@ extern "C" fgl_status fgl_marching_tets(const float* phi, const fgl_grid* grid, 
   a.normals = out_normals;
   a.n_verts = nv;
   a.n_tris = nt;
-  MCUDA(ensure(S.lists, sizeof(uint32_t) * ((size_t)n_samples + n_cubes + 1), s));
-  uint32_t* samples = (uint32_t*)S.lists.p;
+  // 8 bytes a sample for its vertices, then the two lists
+  MCUDA(ensure(S.lists, sizeof(uint32_t) * ((size_t)3 * n_samples + n_cubes + 1), s));
+  MCUDA(ensure(S.places, sizeof(uint2) * nw, s));
+  a.first = (uint2*)S.lists.p;
+  a.places = (const uint2*)S.places.p;
+  uint32_t* samples = (uint32_t*)(a.first + n_samples);
   uint32_t* cubes = samples + n_samples;
-  k_mt_list<<<word_blocks(nw, 256), 256, 0, s>>>(I, m, X, pre, la, samples, cubes);
-  if (n_samples) k_mt_verts<<<word_blocks(n_samples, 256), 256, 0, s>>>(a, samples, n_samples);
-  if (n_cubes) k_mt_tris<<<word_blocks(n_cubes, kMtTriThreads), kMtTriThreads, 0, s>>>(a, cubes, n_cubes);
+  k_mt_list<<<word_blocks(nw, 256), 256, 0, s>>>(I, m, A, pre, chunk_log, la, samples, cubes, (uint2*)S.places.p);
+  if (n_samples) {
+    auto* verts = out_normals ? k_mt_verts<true> : k_mt_verts<false>;
+    verts<<<word_blocks(n_samples, 32 * kMtWarps), 32 * kMtWarps, 0, s>>>(a, samples, n_samples);
+  }
+  if (n_cubes) k_mt_tris<<<word_blocks(n_cubes, 32 * kMtWarps), 32 * kMtWarps, 0, s>>>(a, cubes, n_cubes);
   MCUDA(cudaGetLastError());
   return FGL_OK;
 }
