@@ -20,8 +20,9 @@ using namespace fgl;
 
 struct fgl_scene_s {
   HostBVH bvh;
-  void* d_nodes = nullptr;
-  void* d_tris = nullptr;
+  void* d_nodes = nullptr;       // the node records, then the top cut
+  void* d_tris = nullptr;        // the triangle records, then the cut's
+  const void* d_top = nullptr;   // the cut within d_nodes; null: none
   int device = -1;
 };
 
@@ -223,6 +224,7 @@ ItemDesc make_desc(const fgl_cast_item& it) {
   d.min_range = it.min_range;
   d.n_nodes = count32(it.scene->bvh.n_nodes);
   d.n_tris = count32(it.scene->bvh.n_tris);
+  d.top = it.scene->d_top;
   return d;
 }
 
@@ -626,14 +628,18 @@ fgl_status fgl_scene_upload(fgl_scene s) {
   if (!s) return fail(FGL_ERR_INVALID, "null scene");
   if (s->d_nodes) return FGL_OK;
   size_t nb = s->bvh.nodes.size(), tb = s->bvh.tris.size() * sizeof(float);
-  cudaError_t ae = cudaMalloc(&s->d_nodes, nb);
+  TopBox cut[kTopBoxes];
+  std::vector<float> cut_tris;
+  const bool has_cut = top_cut(s->bvh, cut, &cut_tris);
+  const size_t cut_tb = cut_tris.size() * sizeof(float);
+  cudaError_t ae = cudaMalloc(&s->d_nodes, nb + sizeof(cut));  // nb is a multiple of 16
   if (ae != cudaSuccess) {
     s->d_nodes = nullptr;
     cudaGetLastError();
     if (ae == cudaErrorMemoryAllocation) return fail(FGL_ERR_OOM, "cannot allocate device BVH nodes");
     return cuda_fail(ae, "cudaMalloc(BVH nodes)");
   }
-  if (cudaMalloc(&s->d_tris, tb) != cudaSuccess) {
+  if (cudaMalloc(&s->d_tris, tb + cut_tb) != cudaSuccess) {
     cudaFree(s->d_nodes);
     s->d_nodes = s->d_tris = nullptr;
     cudaGetLastError();
@@ -641,12 +647,16 @@ fgl_status fgl_scene_upload(fgl_scene s) {
   }
   cudaError_t e = cudaMemcpy(s->d_nodes, s->bvh.nodes.data(), nb, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(s->d_tris, s->bvh.tris.data(), tb, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && has_cut) e = cudaMemcpy((char*)s->d_nodes + nb, cut, sizeof(cut), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && cut_tb)
+    e = cudaMemcpy((char*)s->d_tris + tb, cut_tris.data(), cut_tb, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     cudaFree(s->d_nodes);
     cudaFree(s->d_tris);
     s->d_nodes = s->d_tris = nullptr;
     return cuda_fail(e, "scene upload");
   }
+  s->d_top = has_cut ? (const char*)s->d_nodes + nb : nullptr;
   cudaGetDevice(&s->device);
   return FGL_OK;
 }
@@ -658,6 +668,7 @@ fgl_status fgl_scene_evict(fgl_scene s) {
     cudaFree(s->d_nodes);
     cudaFree(s->d_tris);
     s->d_nodes = s->d_tris = nullptr;
+    s->d_top = nullptr;
   }
   return FGL_OK;
 }

@@ -513,6 +513,73 @@ int build_bvh(const float* V, int64_t nv, const int32_t* T, int64_t nt, int widt
   return 0;
 }
 
+bool top_cut(const HostBVH& b, TopBox out[kTopBoxes], std::vector<float>* tris) {
+  const int W = b.width;
+  constexpr uint32_t kLeaf = 1u << 31;
+  int n = 0, n_tris = 0;
+  tris->clear();
+  // replaces box `at` (n: the root) by its node's children
+  auto open = [&](int at, uint32_t node) {
+    const uint8_t* rec = b.nodes.data() + (size_t)node * b.stride;
+    float p[3];
+    uint32_t imask, cbase, tbase, hb[8];
+    std::memcpy(p, rec, 12);
+    std::memcpy(&imask, rec + 12, 4);
+    std::memcpy(&cbase, rec + 16, 4);
+    std::memcpy(&tbase, rec + 20, 4);
+    std::memcpy(hb, rec + node_hb_offset(W), 4 * W);
+    int kids = 0, leaf_tris = 0;
+    for (int c = 0; c < W; ++c) {
+      kids += hb[c] != 0 ? 1 : 0;
+      leaf_tris += __builtin_popcount(hb[c] & 0x00FFFFFFu);
+    }
+    if ((at < n ? n - 1 : n) + kids > kTopBoxes || n_tris + leaf_tris > kMaxNodeTris) return false;
+    for (int c = 0; c < W; ++c) {
+      if (hb[c] == 0) continue;
+      TopBox& k = out[at < n ? at : n];
+      if (at >= n) ++n;
+      at = n;  // the others go to the end
+      for (int a = 0; a < 3; ++a) {
+        float lo, hi;
+        std::memcpy(&lo, rec + node_plane_offset() + 4 * (a * W + c), 4);
+        std::memcpy(&hi, rec + node_plane_offset() + 4 * ((3 + a) * W + c), 4);
+        k.lo[a] = float_down((double)p[a] + (double)lo);
+        k.hi[a] = float_up((double)p[a] + (double)hi);
+      }
+      k.parent = node << 3 | (uint32_t)c;
+      if (hb[c] >> 24) {
+        k.child = cbase + (uint32_t)__builtin_popcount(imask & ((1u << c) - 1u));
+        continue;
+      }
+      k.child = kLeaf;
+      for (uint32_t m = hb[c]; m; m &= m - 1, ++n_tris) {
+        k.child |= 1u << n_tris;
+        const float* t = b.tris.data() + ((size_t)tbase + __builtin_ctz(m)) * kTriFloats;
+        tris->insert(tris->end(), t, t + kTriFloats);
+      }
+    }
+    return true;
+  };
+  if (b.n_nodes < 1 || !open(0, 0)) return false;
+  bool shut[kTopBoxes] = {};  // does not fit opened
+  for (;;) {
+    int best = -1;
+    float best_area = -1.f;
+    for (int i = 0; i < n; ++i) {
+      const float x = out[i].hi[0] - out[i].lo[0], y = out[i].hi[1] - out[i].lo[1], z = out[i].hi[2] - out[i].lo[2];
+      const float area = x * y + y * z + z * x;
+      if (!shut[i] && out[i].child < (1u << 29) && area > best_area) {
+        best = i;
+        best_area = area;
+      }
+    }
+    if (best < 0) break;
+    shut[best] = !open(best, out[best].child);
+  }
+  for (int i = n; i < kTopBoxes; ++i) out[i] = TopBox{{0.f, 0.f, 0.f}, kLeaf, {0.f, 0.f, 0.f}, 0u};
+  return true;
+}
+
 int64_t verify_bvh(const HostBVH& b, std::string* first_error) {
   const int W = b.width, S = b.stride;
   const int64_t N = b.n_nodes;

@@ -96,6 +96,23 @@ struct HostBVH {
 // Host build (bvh_build.cpp).  Returns 0 on success, else writes *err.
 int build_bvh(const float* verts, int64_t nv, const int32_t* tris, int64_t nt, int width,
               int bins, int threads, HostBVH* out, std::string* err);
+// A cut through the top of the tree: up to kTopBoxes disjoint subtrees and leaf
+// runs that hold every triangle, from which a packet starts instead of the
+// root.  The runs' triangles, kMaxNodeTris at most, are repeated after the
+// scene's triangle records.
+constexpr int kTopBoxes = 32;
+struct alignas(16) TopBox {
+  float lo[3];
+  uint32_t child;   // node index, or 1 << 31 | the run's bits among those triangles (0: an unused box)
+  float hi[3];
+  uint32_t parent;  // its parent's index << 3 | its slot there
+};
+static_assert(sizeof(TopBox) == 32, "TopBox layout");
+
+// The cut made by opening the largest box (by area) while kTopBoxes hold the
+// result; boxes round outward.  tris: the runs' triangle records.  False when
+// even the root's children do not fit (too many leaf triangles).
+bool top_cut(const HostBVH& b, TopBox out[kTopBoxes], std::vector<float>* tris);
 // Containment / structure check with the float32 decode arithmetic; returns
 // the number of violations.
 int64_t verify_bvh(const HostBVH& b, std::string* first_error);
@@ -119,8 +136,10 @@ struct alignas(16) ItemDesc {
   float min_range;       // t_min: hits nearer than this are discarded
   uint32_t n_nodes;      // record counts of `nodes` and `tris` (saturated at 2^32 - 1),
   uint32_t n_tris;       // for the checked library's bounds checks
+  const void* top;       // TopBox[kTopBoxes] of the tree, or null: packets start at the root
+  int64_t pad;
 };
-static_assert(sizeof(ItemDesc) == 96, "ItemDesc layout");
+static_assert(sizeof(ItemDesc) == 112, "ItemDesc layout");
 
 // One instance pass: cast the rays of an item against instance k of each
 // environment (its BVH in its own frame, its pose per environment), keeping

@@ -332,7 +332,7 @@ __device__ __forceinline__ void trace_packet(const ItemDesc& it, int env, int fi
     dev::setup_ray(tr.r, ox, oy, oz, dx, dy, dz);
     tr.start(it.nodes, it.tris, it.min_range, it.max_range, it.n_nodes, it.n_tris);
     if (COUNT) tr.n_rounds = tr.n_pops = 0;
-    end = dev::packet_phase(tr, dx, dy, dz, pl, lane, live, status, c[3], c[4]);
+    end = dev::packet_phase(tr, dx, dy, dz, (const uint4*)it.top, it.n_tris, pl, lane, live, status, c[3], c[4]);
   }
   if (end != dev::kPacketDone) {
     bool active = live && (end == dev::kPacketNone || tr.next_entry(pl));

@@ -680,8 +680,11 @@ enum PacketEnd { kPacketNone = 0, kPacketDone = 1, kPacketEntries = 2 };
 // triangle it meets against all 32 rays.  The frustum is a rectangle in the
 // plane z = 1 of the dominant axis: a0 <= x / z <= a1, b0 <= y / z <= b1 over
 // all rays (widened far beyond float32 rounding), so a box needs four
-// compares against two scaled coordinates each.  The two nearest nodes are
-// opened together: lane W g + c tests child c of node g.  The boxes still to
+// compares against two scaled coordinates each.  It starts from the scene's top
+// cut (`top`, a box a lane, its leaf triangles from top_tris on) where there is
+// one: that step stands for the root's and several more (4096 x 5760 rays on
+// 1 M triangles 3.66 -> 3.45 ms with 32 boxes; with 24 3.46, with 16 3.52).
+// The two nearest nodes are opened together: lane W g + c tests child c of node g.  The boxes still to
 // visit sit one a lane (distance bits with the slot in the low 3, node,
 // parent), and a warp minimum picks the nearest.
 //
@@ -697,6 +700,7 @@ enum PacketEnd { kPacketNone = 0, kPacketDone = 1, kPacketEntries = 2 };
 // without a ray of its own carries a copy of another lane's (live = false).
 template <int W, bool COUNT, bool TMIN>
 __device__ __forceinline__ PacketEnd packet_phase(Tracer<W, COUNT, TMIN>& tr, float dx, float dy, float dz,
+                                                  const uint4* top, uint32_t top_tris,
                                                   const PacketList& pl, int lane, bool live, unsigned* status,
                                                   uint32_t& c_iters, uint32_t& c_lane_iters) {
   const unsigned FULL = 0xFFFFFFFFu;
@@ -740,8 +744,82 @@ __device__ __forceinline__ PacketEnd packet_phase(Tracer<W, COUNT, TMIN>& tr, fl
               toZ = sel3(tr.r.ox, tr.r.oy, tr.r.oz, tkz);
 
   uint32_t tkey = __float_as_uint(tr.best_t) | 7u;  // the farthest best hit of the packet, as a key
+  // a box in the packet's frame: the earliest entry of a ray (tn), and whether
+  // some ray may meet it (then these differences are all non-negative)
+  auto meets = [&](float X0, float X1, float Y0, float Y1, float zn, float zf, float zc, float& tn) {
+    tn = max3f(max3f(zc * iz, X0 * ixp, X1 * ixn), Y0 * iyp, Y1 * iyn);
+    const float in = min3f(min3f(X1 - fminf(a0 * zc, a0 * zf), fmaxf(a1 * zc, a1 * zf) - X0, zf),
+                           Y1 - fminf(b0 * zc, b0 * zf), fmaxf(b1 * zc, b1 * zf) - Y0);
+    return (in >= 0.f) & (__float_as_uint(tn) <= tkey);
+  };
+  // the triangles tb + (bits set) against every ray; false: an index out of range
+  auto test_run = [&](uint32_t bits, uint32_t tb, uint32_t past) {
+    while (bits) {
+      const uint32_t pos = __ffs(bits) - 1;
+      bits &= bits - 1;
+#ifdef FGL_CHECKED
+      if ((size_t)tb + pos >= (size_t)tr.lim_tris + past) {
+        if (lane == 0) atomicOr(status, 4u);
+        return false;
+      }
+#else
+      (void)status;
+      (void)past;
+#endif
+      if (COUNT) {
+        tr.n_tris += live ? 1u : 0u;
+        tr.n_rounds += lane == 0 ? 1u : 0u;
+      }
+      const float* tp = (const float*)tr.tris + 12 * ((size_t)tb + pos);
+      const float* px = tp + tkx;
+      const float* py = tp + tky;
+      const float* pz = tp + tkz;
+      const int32_t id = __ldg((const int32_t*)tp + 3);
+      tr.consider(tri_hit_axes<true>(tr.r, __ldg(px) - toX, __ldg(py) - toY, __ldg(pz) - toZ, __ldg(px + 4) - toX,
+                               __ldg(py + 4) - toY, __ldg(pz + 4) - toZ, __ldg(px + 8) - toX, __ldg(py + 8) - toY,
+                               __ldg(pz + 8) - toZ, tr.best_t),
+                  id);
+    }
+    return true;
+  };
   uint32_t fkey = lane == 0 ? 0u : kNoEntry, fnode = 0u, fpar = 0u;
   int live_n = 1;  // boxes waiting
+  if (top != nullptr) {  // from the cut, a box a lane
+    const uint4 A = __ldg(top + 2 * lane), B = __ldg(top + 2 * lane + 1);
+    const float X0 = sel3(__uint_as_float(A.x), __uint_as_float(A.y), __uint_as_float(A.z), kx) - oX;
+    const float X1 = sel3(__uint_as_float(B.x), __uint_as_float(B.y), __uint_as_float(B.z), kx) - oX;
+    const float Y0 = sel3(__uint_as_float(A.x), __uint_as_float(A.y), __uint_as_float(A.z), ky) - oY;
+    const float Y1 = sel3(__uint_as_float(B.x), __uint_as_float(B.y), __uint_as_float(B.z), ky) - oY;
+    const float z0 = sel3(__uint_as_float(A.x), __uint_as_float(A.y), __uint_as_float(A.z), kz) - oZ;
+    const float z1 = sel3(__uint_as_float(B.x), __uint_as_float(B.y), __uint_as_float(B.z), kz) - oZ;
+    const float zn = sg > 0.f ? z0 : -z1, zf = sg > 0.f ? z1 : -z0, zc = fmaxf(zn, 0.f);
+    float tn;
+    const bool hit = meets(X0, X1, Y0, Y1, zn, zf, zc, tn), leaf = A.w >> 31;
+    const int n = __popc(__ballot_sync(FULL, hit & !leaf));
+    if (COUNT) {
+      c_iters += lane == 0 ? 1u : 0u;
+      c_lane_iters += live ? 1u : 0u;
+      tr.n_nodes += live ? 1u : 0u;
+    }
+    if (n <= 32 - W) {  // else there is no room to go on from here
+      const bool small = max3f(X1 - X0, Y1 - Y0, zf - zn) < narrow * zc;
+      fkey = hit & !leaf ? (__float_as_uint(tn) & ~7u) | (B.w & 7u) : kNoEntry;
+      fnode = small ? A.w | kSmallNode : A.w;
+      fpar = B.w >> 3;
+      live_n = n;
+#ifdef FGL_CHECKED
+      if (__any_sync(FULL, fkey != kNoEntry && fpar >= tr.lim_nodes)) {
+        if (lane == 0) atomicOr(status, 4u);
+        return kPacketDone;
+      }
+#endif
+      const uint32_t bits = __reduce_or_sync(FULL, hit & leaf ? A.w & 0x00FFFFFFu : 0u);
+      if (bits) {
+        if (!test_run(bits, top_tris, kMaxNodeTris)) return kPacketDone;
+        tkey = __float_as_uint(redux_maxf(tr.best_t)) | 7u;
+      }
+    }
+  }
   for (;;) {
     const uint32_t m0 = __reduce_min_sync(FULL, fkey);
     if (m0 > tkey) return kPacketDone;
@@ -782,11 +860,8 @@ __device__ __forceinline__ PacketEnd packet_phase(Tracer<W, COUNT, TMIN>& tr, fl
     const float rz = (sel3(__uint_as_float(h0.x), __uint_as_float(h0.y), __uint_as_float(h0.z), kz) - oZ) * sg;
     const float X0 = x0r + rx, X1 = x1r + rx, Y0 = y0r + ry, Y1 = y1r + ry;
     const float zn = fmaf(znr, sg, rz), zf = fmaf(zfr, sg, rz), zc = fmaxf(zn, 0.f);
-    const float tn = max3f(max3f(zc * iz, X0 * ixp, X1 * ixn), Y0 * iyp, Y1 * iyn);
-    // inside: every one of these differences is non-negative
-    const float in = min3f(min3f(X1 - fminf(a0 * zc, a0 * zf), fmaxf(a1 * zc, a1 * zf) - X0, zf),
-                           Y1 - fminf(b0 * zc, b0 * zf), fmaxf(b1 * zc, b1 * zf) - Y0);
-    const bool hit = use & (in >= 0.f) & (__float_as_uint(tn) <= tkey);
+    float tn;
+    const bool hit = use & meets(X0, X1, Y0, Y1, zn, zf, zc, tn);
     const uint32_t got = hit ? hb : 0u;  // 0 for an empty slot
     if (COUNT) {
       const uint32_t nodes_now = __popc(__ballot_sync(FULL, use)) / W;
@@ -818,33 +893,8 @@ __device__ __forceinline__ PacketEnd packet_phase(Tracer<W, COUNT, TMIN>& tr, fl
     if (__any_sync(FULL, got & 0x00FFFFFFu)) {
 #pragma unroll 1
       for (int g = 0; g < 2; ++g) {
-        uint32_t bits = __reduce_or_sync(FULL, lane / W == g ? got & 0x00FFFFFFu : 0u);
-        const uint32_t tb = __shfl_sync(FULL, base.y, g * W);
-        while (bits) {
-          const uint32_t pos = __ffs(bits) - 1;
-          bits &= bits - 1;
-#ifdef FGL_CHECKED
-          if ((size_t)tb + pos >= tr.lim_tris) {
-            if (lane == 0) atomicOr(status, 4u);
-            return kPacketDone;
-          }
-#else
-          (void)status;
-#endif
-          if (COUNT) {
-            tr.n_tris += live ? 1u : 0u;
-            tr.n_rounds += lane == 0 ? 1u : 0u;
-          }
-          const float* tp = (const float*)tr.tris + 12 * ((size_t)tb + pos);
-          const float* px = tp + tkx;
-          const float* py = tp + tky;
-          const float* pz = tp + tkz;
-          const int32_t id = __ldg((const int32_t*)tp + 3);
-          tr.consider(tri_hit_axes<true>(tr.r, __ldg(px) - toX, __ldg(py) - toY, __ldg(pz) - toZ, __ldg(px + 4) - toX,
-                                   __ldg(py + 4) - toY, __ldg(pz + 4) - toZ, __ldg(px + 8) - toX, __ldg(py + 8) - toY,
-                                   __ldg(pz + 8) - toZ, tr.best_t),
-                      id);
-        }
+        const uint32_t bits = __reduce_or_sync(FULL, lane / W == g ? got & 0x00FFFFFFu : 0u);
+        if (!test_run(bits, __shfl_sync(FULL, base.y, g * W), 0u)) return kPacketDone;
       }
       tkey = __float_as_uint(redux_maxf(tr.best_t)) | 7u;
     }
