@@ -735,6 +735,7 @@ static size_t packets_smem_bytes(int W, int block, int sdepth) {
 }
 
 bool packets_fit(int W, int block, int sdepth) {
+  if (packets_smem_bytes(W, block, sdepth) <= 48 * 1024) return true;  // any block's: no need to ask the device
   int dev = 0, optin = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
