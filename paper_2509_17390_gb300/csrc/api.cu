@@ -397,6 +397,7 @@ fgl_status enqueue_batch(BatchCtx& c, const std::vector<Group>& groups,
         }
         a.sphere[k][3] = std::nextafter((float)std::sqrt(r2), INFINITY);
       }
+      a.out_points = it.out_points;
       FGL_CUDA(launch_instances_fused(a, it.min_range > 0.f, 128, o.sdepth, s));
     }
     for (int k = 0; !fuse && k < it.n_instances; ++k) {
@@ -422,7 +423,7 @@ fgl_status enqueue_batch(BatchCtx& c, const std::vector<Group>& groups,
     }
     if (it.n_instances == 0 && it.out_instance)
       FGL_CUDA(cudaMemsetAsync(it.out_instance, 0xFF, (size_t)d.n_env * d.n_rays * sizeof(int32_t), s));
-    if (it.out_points) FGL_CUDA(launch_points(d, it.out_points, s));
+    if (it.out_points && !fuse) FGL_CUDA(launch_points(d, it.out_points, s));
   }
   return FGL_OK;
 }

@@ -169,6 +169,7 @@ struct InstanceSet {
   const void* tris[kMaxFusedInstances];
   float sphere[kMaxFusedInstances][4];  // instance-frame bounding sphere: centre, radius (rounded up)
   uint32_t n_nodes[kMaxFusedInstances], n_tris[kMaxFusedInstances];  // record counts
+  float* out_points;                    // world-frame return points, or null
 };
 
 struct alignas(16) BatchHeader {
