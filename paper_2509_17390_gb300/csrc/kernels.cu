@@ -539,8 +539,9 @@ __device__ __forceinline__ void store_point(float* out, int64_t o, bool hit, flo
 // return, replacing it only when strictly nearer -- the per-instance passes'
 // result, bit for bit, with the ray's record read and written once and its
 // return point beside it.  Bound by issue, at part of the lanes: 5.9 M rays and
-// four objects 0.41 ms, 0.44 with the points in a pass of their own.  (Walking an object's upper tree a packet at a time, as
-// the scene's, was slower: 6% of the whole cast with eight or more rays left.)
+// four objects 0.41 ms, 0.44 with the points in a pass of their own.  (Walking
+// an object's upper tree a packet at a time, as the scene's, was slower: by 7%
+// of the whole cast where eight or more rays are left.)
 template <int W, bool TMIN>
 __global__ void __maxnreg__(72) k_instances_fused(const InstanceSet a, int sdepth) {
   using Keys = typename dev::KeyWords<W>::T;

@@ -558,39 +558,71 @@ __global__ void k_run_init(const uint32_t* __restrict__ Vb, BitGrid g, uint32_t*
 }
 
 // Runs of adjacent rows (-y, -z) that share a free voxel are one component:
-// one union per overlap segment.  One warp per row.  With tile flags (from
-// k_run_tiles) a pair of rows inside one tile is skipped unless that tile
-// fell back to the global path: its unions are done already.
-__global__ void k_run_union(const uint32_t* __restrict__ Vb, BitGrid g, uint32_t* parent, int* err,
-                            int ty, int tz, const uint8_t* __restrict__ tile_global) {
+// one union per overlap segment.  One warp per pair of rows.
+__device__ __forceinline__ void unite_rows(const uint32_t* __restrict__ Vb, const BitGrid& g, uint32_t* parent,
+                                           int64_t row, int64_t row2, uint32_t limit, int* err) {
   const int lane = threadIdx.x & 31;
+  int cp = -1, cp2 = -1;
+  uint32_t cb = 0, cb2 = 0, ocarry = 0;
+  for (int base = 0; base < g.mw; base += 32) {
+    const RowChunk a = row_chunk(Vb, g, row, base, lane, cp, cb);
+    const RowChunk b = row_chunk(Vb, g, row2, base, lane, cp2, cb2);
+    const uint32_t O = a.F & b.F;
+    uint32_t oprev = __shfl_up_sync(0xFFFFFFFFu, O, 1) >> 31;
+    if (lane == 0) oprev = ocarry;
+    ocarry = __shfl_sync(0xFFFFFFFFu, O, 31) >> 31;
+    const int xw = base + lane;
+    for (uint32_t m = O & ~((O << 1) | oprev); m; m &= m - 1) {
+      const int s = __ffs(m) - 1;
+      uf_unite(parent, run_label(a, xw, s, row, g.nx), run_label(b, xw, s, row2, g.nx), limit, err);
+    }
+  }
+}
+
+// The pairs of a grid without tiles, or of the tiles that fell back to the
+// global path (tile_global).
+__device__ __forceinline__ void unite_all_rows(const uint32_t* __restrict__ Vb, const BitGrid& g, uint32_t* parent,
+                                               int* err, int ty, int tz, const uint8_t* __restrict__ tile_global) {
   const int64_t n_warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   const uint32_t limit = (uint32_t)(g.rows() * g.nx + 2);
   const int n_ty = tile_global ? (g.ny + ty - 1) / ty : 0;
   for (int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < g.rows(); row += n_warps) {
-    const int j = (int)(row % g.ny), k = (int)(row / g.ny);
-    const bool all_pairs = !tile_global || tile_global[(k / tz) * n_ty + j / ty];
-    for (int nb = 0; nb < 2; ++nb) {
-      if (nb == 0 ? j == 0 : k == 0) continue;
-      if (!all_pairs && (nb == 0 ? j % ty : k % tz) != 0) continue;
-      const int64_t row2 = nb == 0 ? row - 1 : row - g.ny;
-      int cp = -1, cp2 = -1;
-      uint32_t cb = 0, cb2 = 0, ocarry = 0;
-      for (int base = 0; base < g.mw; base += 32) {
-        const RowChunk a = row_chunk(Vb, g, row, base, lane, cp, cb);
-        const RowChunk b = row_chunk(Vb, g, row2, base, lane, cp2, cb2);
-        const uint32_t O = a.F & b.F;
-        uint32_t oprev = __shfl_up_sync(0xFFFFFFFFu, O, 1) >> 31;
-        if (lane == 0) oprev = ocarry;
-        ocarry = __shfl_sync(0xFFFFFFFFu, O, 31) >> 31;
-        const int xw = base + lane;
-        for (uint32_t m = O & ~((O << 1) | oprev); m; m &= m - 1) {
-          const int s = __ffs(m) - 1;
-          uf_unite(parent, run_label(a, xw, s, row, g.nx), run_label(b, xw, s, row2, g.nx), limit, err);
-        }
-      }
-    }
+    const int k = (int)g.by_ny.div((uint32_t)row), j = (int)((uint32_t)row - (uint32_t)k * (uint32_t)g.ny);
+    if (tile_global && !tile_global[(k / tz) * n_ty + j / ty]) continue;
+    if (j > 0) unite_rows(Vb, g, parent, row, row - 1, limit, err);
+    if (k > 0) unite_rows(Vb, g, parent, row, row - g.ny, limit, err);
   }
+}
+
+__global__ void k_run_union(const uint32_t* __restrict__ Vb, BitGrid g, uint32_t* parent, int* err) {
+  unite_all_rows(Vb, g, parent, err, 1, 1, nullptr);
+}
+
+// After k_run_tiles: the pairs across tile borders, a warp a pair -- the pairs
+// (j, j - 1) at j = ty, 2 ty, .. of every plane, then (k, k - 1) at k = tz, ..
+// of every row -- and, when a tile fell back (*fell_back == call), those
+// within such tiles.  Bound by the latency of the walks to the roots.
+__global__ void k_tile_union(const uint32_t* __restrict__ Vb, BitGrid g, uint32_t* parent, int* err, int ty, int tz,
+                             const uint8_t* __restrict__ tile_global, const uint32_t* __restrict__ fell_back,
+                             uint32_t call) {
+  const uint32_t limit = (uint32_t)(g.rows() * g.nx + 2);
+  const uint32_t by_y = (uint32_t)((g.ny - 1) / ty), by_z = (uint32_t)((g.nz - 1) / tz);  // borders
+  const uint32_t n_y = by_y * (uint32_t)g.nz, n = n_y + by_z * (uint32_t)g.ny;
+  const uint32_t n_warps = gridDim.x * (blockDim.x >> 5);
+  for (uint32_t t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < n; t += n_warps) {
+    uint32_t j, k;
+    if (t < n_y) {
+      k = t / by_y;
+      j = (t - k * by_y + 1) * (uint32_t)ty;
+    } else {
+      const uint32_t q = g.by_ny.div(t - n_y);
+      k = (q + 1) * (uint32_t)tz;
+      j = t - n_y - q * (uint32_t)g.ny;
+    }
+    const int64_t row = (int64_t)k * g.ny + j;
+    unite_rows(Vb, g, parent, row, t < n_y ? row - 1 : row - g.ny, limit, err);
+  }
+  if (*fell_back == call) unite_all_rows(Vb, g, parent, err, ty, tz, tile_global);
 }
 
 // Tiled first pass: one block per tile of ty x tz rows (all of x) does, in
@@ -670,11 +702,13 @@ __device__ __forceinline__ void tile_unite(uint32_t* par, uint32_t a, uint32_t b
   atomicOr(err, 8);
 }
 
-__global__ void __launch_bounds__(kTileThreads) k_run_tiles(const uint8_t* __restrict__ surf, BitGrid g, int ty,
-                                                            int tz, int cap, uint32_t* __restrict__ Vb,
+template <int T>  // ty = tz = T
+__global__ void __launch_bounds__(kTileThreads) k_run_tiles(const uint8_t* __restrict__ surf, BitGrid g, int cap, uint32_t* __restrict__ Vb,
                                                             uint32_t* __restrict__ parent,
-                                                            uint8_t* __restrict__ tile_global, int* err) {
+                                                            uint8_t* __restrict__ tile_global,
+                                                            uint32_t* __restrict__ fell_back, uint32_t call, int* err) {
   extern __shared__ uint32_t tsm[];
+  constexpr int ty = T, tz = T;
   const int rows_t = ty * tz, mw = g.mw, nwt = rows_t * mw;
   uint32_t* sF = tsm;                        // free bits of the tile's words
   uint32_t* sSt = sF + nwt;                  // run starts
@@ -700,14 +734,23 @@ __global__ void __launch_bounds__(kTileThreads) k_run_tiles(const uint8_t* __res
     const uint8_t* src_a = surf + ((int64_t)ka * g.ny + ja) * g.nx;
     const uint8_t* src_b = surf + ((int64_t)kb * g.ny + jb) * g.nx;
     uint32_t mine_a = 0, mine_b = 0;
-#pragma unroll 4
-    for (int xw = 0; xw < mw; ++xw) {
-      const int x = xw * 32 + lane;
-      const uint32_t ba = __ballot_sync(0xFFFFFFFFu, in_a && x < g.nx && src_a[x] != 0);
-      const uint32_t bb = __ballot_sync(0xFFFFFFFFu, in_b && x < g.nx && src_b[x] != 0);
-      if (lane == xw) {
-        mine_a = ba;
-        mine_b = bb;
+    for (int xw0 = 0; xw0 < mw; xw0 += 8) {
+      uint8_t va[8], vb[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if (u == 4 && xw0 + 4 >= mw) break;
+        const int x = (xw0 + u) * 32 + lane;
+        va[u] = in_a && x < g.nx ? src_a[x] : 0;
+        vb[u] = in_b && x < g.nx ? src_b[x] : 0;
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if (u == 4 && xw0 + 4 >= mw) break;
+        const uint32_t ba = __ballot_sync(0xFFFFFFFFu, va[u] != 0), bb = __ballot_sync(0xFFFFFFFFu, vb[u] != 0);
+        if (lane == xw0 + u) {
+          mine_a = ba;
+          mine_b = bb;
+        }
       }
     }
     if (lane < mw) {
@@ -725,7 +768,7 @@ __global__ void __launch_bounds__(kTileThreads) k_run_tiles(const uint8_t* __res
     uint32_t c = 0;
     if (i < nwt) {
       const uint32_t F = sF[i];
-      const uint32_t prev = (i % mw) ? sF[i - 1] >> 31 : 0u;
+      const uint32_t prev = i != (int)g.by_mw.div((uint32_t)i) * mw ? sF[i - 1] >> 31 : 0u;
       const uint32_t st = F & ~((F << 1) | prev);
       sSt[i] = st;
       c = __popc(st);
@@ -751,7 +794,7 @@ __global__ void __launch_bounds__(kTileThreads) k_run_tiles(const uint8_t* __res
   for (int i = tid; i < nwt; i += kTileThreads) {
     const uint32_t st = sSt[i];
     if (!st) continue;
-    const int lr = i / mw, xw = i - lr * mw;
+    const int lr = (int)g.by_mw.div((uint32_t)i), xw = i - lr * mw;
     const int j = j0 + lr % ty, k = k0 + lr / ty;
     const bool face = j == 0 || k == 0 || j == g.ny - 1 || k == g.nz - 1;
     const uint32_t row_base = (uint32_t)(((int64_t)k * g.ny + j) * g.nx) + 1u;
@@ -769,7 +812,10 @@ __global__ void __launch_bounds__(kTileThreads) k_run_tiles(const uint8_t* __res
       }
     }
   }
-  if (tid == 0) tile_global[blockIdx.x] = global_path ? 1 : 0;
+  if (tid == 0) {
+    tile_global[blockIdx.x] = global_path ? 1 : 0;
+    if (global_path) *fell_back = call;
+  }
   if (global_path) return;
   if (tid == 0) sPar[0] = sLab[0] = 0u;
   __syncthreads();
@@ -781,7 +827,7 @@ __global__ void __launch_bounds__(kTileThreads) k_run_tiles(const uint8_t* __res
   for (int phase = 0; phase < 2; ++phase) {
     const int n_tasks = (phase == 0 ? n_py : n_pz) * mw;
     for (int t = tid; t < n_tasks; t += kTileThreads) {
-      const int p = t / mw, xw = t - p * mw;
+      const int p = (int)g.by_mw.div((uint32_t)t), xw = t - p * mw;
       int a, b;
       if (phase == 0) {
         a = (p / (ty - 1)) * ty + p % (ty - 1) + 1;
@@ -1731,6 +1777,7 @@ struct Scratch {
   unsigned long long* host = nullptr;  // pinned: [2] the TSDF error flag, [4..6] the mesh totals read back
   cudaEvent_t err_ready = nullptr;     // recorded after the flag's copy to host[2]
   int pending_err_check = 0;
+  uint32_t tsdf_calls = 0;  // the mark of a call's tiles that fell back
   std::mutex mu;
 };
 std::mutex g_scr_mu;
@@ -1953,7 +2000,7 @@ extern "C" fgl_status fgl_tsdf(const uint8_t* surf, const fgl_grid* grid, float 
   if (!tiled_shells) MCUDA(ensure(S.shells, sizeof(uint32_t) * nw * (2 + n_planes), s));
   MCUDA(ensure(S.parent, sizeof(uint32_t) * (n + 1), s));
   const TilePlan tp = plan_tiles(g);
-  if (tp.ty) MCUDA(ensure(S.tiles, (size_t)tp.n_tiles, s));
+  if (tp.ty) MCUDA(ensure(S.tiles, (size_t)tp.n_tiles + 8, s));
   uint32_t* Vb = (uint32_t*)S.bits_a.p;
   uint32_t* Ob = (uint32_t*)S.bits_b.p;
   uint32_t* parent = (uint32_t*)S.parent.p;
@@ -1969,14 +2016,19 @@ extern "C" fgl_status fgl_tsdf(const uint8_t* surf, const fgl_grid* grid, float 
   const unsigned rb = word_blocks(g.rows() * 32, 256);
   if (tp.ty) {  // tiles pack the surface themselves
     uint8_t* tile_global = (uint8_t*)S.tiles.p;
-    k_run_tiles<<<(unsigned)tp.n_tiles, kTileThreads, tp.smem, s>>>(surf, g, tp.ty, tp.tz, tp.cap, Vb, parent,
-                                                                  tile_global, S.err);
-    k_run_union<<<rb, 256, 0, s>>>(Vb, g, parent, S.err, tp.ty, tp.tz, tile_global);
+    uint32_t* fell_back = (uint32_t*)(tile_global + (tp.n_tiles + 3) / 4 * 4);
+    const uint32_t call = ++S.tsdf_calls;
+    auto* tiles = tp.ty == 8 ? k_run_tiles<8> : k_run_tiles<4>;
+    tiles<<<(unsigned)tp.n_tiles, kTileThreads, tp.smem, s>>>(surf, g, tp.cap, Vb, parent, tile_global, fell_back, call,
+                                                              S.err);
+    const int64_t pairs = (int64_t)(g.ny - 1) / tp.ty * g.nz + (int64_t)(g.nz - 1) / tp.tz * g.ny;
+    k_tile_union<<<word_blocks(std::max<int64_t>(pairs, 152) * 32, 256), 256, 0, s>>>(
+        Vb, g, parent, S.err, tp.ty, tp.tz, tile_global, fell_back, call);
     launches += 2;
   } else {
     k_pack_u8<<<word_blocks(g.rows() * 32, 256), 256, 0, s>>>(surf, g, Vb);
     k_run_init<<<rb, 256, 0, s>>>(Vb, g, parent);
-    k_run_union<<<rb, 256, 0, s>>>(Vb, g, parent, S.err, 1, 1, nullptr);
+    k_run_union<<<rb, 256, 0, s>>>(Vb, g, parent, S.err);
     launches += 3;
   }
   k_run_outside<<<rb, 256, 0, s>>>(Vb, g, parent, Ob, S.err);
