@@ -52,14 +52,16 @@ WORKLOAD = ("batched_walk: 4096 envs x (16 beams -15..+15 deg x 360 az) = 23,592
 # the sources each profiled kernel is built from: a committed ncu figure is
 # used only while its kernel's sources are unchanged
 KERNEL_SOURCES = {
-    # the wide kernel's work per ray also depends on the tree its builder makes
-    "k_persistent": ["paper_2509_17390_gb300/csrc/trace.cuh", "paper_2509_17390_gb300/csrc/kernels.cu",
-                     "paper_2509_17390_gb300/csrc/bvh_build.cpp"],
-    "k_lbvh_cast": ["paper_2509_17390_gb300/csrc/trace.cuh", "paper_2509_17390_gb300/csrc/lbvh.cu"],
+    # the wide kernels' work per ray also depends on the tree its builder makes
+    "k_packets": ["paper_2509_17390_gb300/csrc/trace.cuh", "paper_2509_17390_gb300/csrc/kernels.cu",
+                  "paper_2509_17390_gb300/csrc/bvh_build.cpp"],
+    "k_plain_packets": ["paper_2509_17390_gb300/csrc/trace.cuh", "paper_2509_17390_gb300/csrc/kernels.cu",
+                        "paper_2509_17390_gb300/csrc/lbvh.cu"],
+    "k_density": ["paper_2509_17390_gb300/csrc/density.cu"],
 }
 
 
-def kernel_hash(name: str = "k_persistent") -> str:
+def kernel_hash(name: str = "k_packets") -> str:
     h = hashlib.sha256()
     for p in KERNEL_SOURCES[name]:
         h.update(open(os.path.join(ROOT, p), "rb").read())
@@ -113,6 +115,26 @@ def issue_roofline(kernel, entry, rays_per_s, clocks, dev, extra=None):
                     "its issue slots, not HBM, bound it"}
     if extra:
         out.update(extra)
+    return out
+
+
+def density_roofline(evals, kern_s, clocks, dev):
+    """k_density's bound, instruction issue: executed warp instructions per
+    (voxel, candidate) evaluation (ncu, a committed capture of the current
+    sources over the same sets) x evaluations / kernel time, against four
+    warp schedulers an SM.  Without a matching capture the rate alone."""
+    import torch
+    sms = torch.cuda.get_device_properties(dev).multi_processor_count
+    mhz = (clocks or {}).get("sm_mhz") or 2070.0
+    peak = 4.0 * sms * mhz * 1e6 / 1e9
+    ipe = read_profile("k_density", "warp_inst_per_eval")
+    out = {"bound": "alu", "kernel": "k_density<8>", "unit": "G warp-inst/s", "peak": round(peak, 1),
+           "peak_source": "derived",
+           "peak_basis": f"4 warp schedulers x {sms} SMs x {mhz:.0f} MHz (instruction issue)",
+           "Geval_per_s": round(evals / kern_s / 1e9, 1), "kernel_ms_per_step": round(kern_s * 1e3, 3)}
+    ach = None if ipe is None else ipe * evals / kern_s / 1e9
+    out.update({"achieved": None if ach is None else round(ach, 1),
+                "frac": None if ach is None else round(ach / peak, 4), "warp_inst_per_eval": ipe})
     return out
 
 
@@ -279,7 +301,7 @@ def counted_bytes(fgl, items, stream, opts=None):
     return tot_b, tot_r, tot_n, tot_t
 
 
-def hbm_roofline(bytes_, seconds, rays, nodes, tris, kernel="k_persistent"):
+def hbm_roofline(bytes_, seconds, rays, nodes, tris, kernel="k_packets"):
     peak, kind = read_peaks()
     achieved = bytes_ / seconds / 1e9
     return {"bound": "hbm", "kernel": kernel, "achieved": round(achieved, 1), "peak": peak,
@@ -631,12 +653,12 @@ def main():
     # measured traffic beside the cost model: DRAM bytes of one full launch and
     # L2 (lts__t_bytes) bytes per ray from the committed ncu captures, as rates;
     # the L2 rate against an L2 copy bandwidth measured here
-    traffic = read_traffic("k_persistent")
+    traffic = read_traffic("k_packets")
     measured = {"dram_bytes_per_launch": traffic}
     if traffic is not None:
         measured["dram_gbs"] = round(traffic / (kern_ms / 1e3) / 1e9, 1)
         measured["dram_frac"] = round(traffic / (kern_ms / 1e3) / 1e9 / peak, 4)
-    lpr = read_profile("k_persistent", "lts_bytes_per_ray")
+    lpr = read_profile("k_packets", "lts_bytes_per_ray")
     l2pk = l2_read_peak(dev)
     l2 = {"achieved": None, "peak": l2pk["gbs"], "unit": "GB/s", "peak_basis": l2pk["basis"]}
     if lpr is not None:
@@ -646,7 +668,7 @@ def main():
     # committed capture of these sources); without a matching capture the
     # line falls back to the cost model
     rps = n_rays / (kern_ms / 1e3)
-    roofline = issue_roofline("k_persistent", None, rps, clocks, dev,
+    roofline = issue_roofline("k_packets", None, rps, clocks, dev,
                               {"cost_model": cost_model, "dram": measured, "l2": l2})
     if roofline is None:
         roofline = dict(cost_model, traffic=traffic, dram=measured, l2=l2,
@@ -1009,13 +1031,13 @@ def run_walk_instances(args):
         e2e = {"value": round(ws * n_rays * ksteps / t_e / 1e9, 4), "unit": UNIT,
                "h2d_bytes_per_step": n_env * 48 * (1 + K), "d2h_bytes_per_step": n_rays * 24,
                "ms_per_step": round(t_e * 1e3 / ksteps, 3)}
-    # the dominant kernel is the scene cast (k_persistent): its cost-model
+    # the dominant kernel is the scene cast (k_packets): its cost-model
     # bytes from a counting pass, over its own time (the step without instances)
     with torch.cuda.stream(stream):
         pose_state.copy_(walk_d[args.warmup % S])
     cb, cr, cn, ct = counted_bytes(fgl, items0, stream, opts)
-    cost = hbm_roofline(cb, tot0 / args.steps, cr, cn, ct, kernel="k_persistent (the scene cast)")
-    roofline = issue_roofline("k_persistent", "k_persistent@walk_instances", n_rays * args.steps / tot0,
+    cost = hbm_roofline(cb, tot0 / args.steps, cr, cn, ct, kernel="k_packets (the scene cast)")
+    roofline = issue_roofline("k_packets", "k_packets@walk_instances", n_rays * args.steps / tot0,
                               clocks, torch.device("cuda"), {"cost_model": cost,
                               "note": "the scene cast, over its own time (the step without instances)"})
     if roofline is None:
@@ -1034,14 +1056,14 @@ def run_walk_instances(args):
                            "returns_on_instances": round(seen, 4),
                            "l2": "flushed between timed steps (256 MiB write)"},
                 "without_instances_ms_per_step": round(tot0 * 1e3 / args.steps, 3),
-                "gpu_launches": args.steps * 3,   # scene cast, fused instance pass, return points
+                "gpu_launches": args.steps * 2,   # scene cast, instance pass (which writes the return points)
                 "e2e": e2e, "roofline": roofline, "clocks": clocks}
         print(json.dumps(line), flush=True)
 
 
 def run_lbvh(args):
     """The paper's route on the batched walk: a triangle LBVH built on the GPU
-    and cast one thread per beam, against the host-built wide SAH BVH and its
+    and opened into wide nodes, against the host-built wide SAH BVH and its
     persistent batched kernel; plus a dynamic-scene step (every vertex moved,
     the LBVH rebuilt, then cast)."""
     import torch
@@ -1113,23 +1135,23 @@ def run_lbvh(args):
     clocks = clk.summary()
     t_wide = timed(cast_wide)
     t_dyn = timed(dynamic)
-    # the LBVH cast is bound by instruction issue like the wide kernel: warp
+    # the LBVH cast is bound by instruction issue like the batched kernel: warp
     # instructions per ray (ncu, committed with its sources' hash) x rays/s
     # against 4 warp instructions per SM per cycle at the sampled clock
     roofline = None
-    ipr = read_profile("k_lbvh_cast", "warp_inst_per_ray")
+    ipr = read_profile("k_plain_packets", "warp_inst_per_ray")
     if ipr is not None:
         sms = torch.cuda.get_device_properties(dev).multi_processor_count
         mhz = (clocks or {}).get("sm_mhz") or 2070.0
         ach = ipr * n_rays * args.steps / t_lbvh / 1e9
         pk = 4.0 * sms * mhz * 1e6 / 1e9
-        roofline = {"bound": "alu", "kernel": "k_lbvh_cast", "achieved": round(ach, 1), "peak": round(pk, 1),
+        roofline = {"bound": "alu", "kernel": "k_plain_packets", "achieved": round(ach, 1), "peak": round(pk, 1),
                     "unit": "G warp-inst/s", "frac": round(ach / pk, 4), "warp_inst_per_ray": ipr,
-                    "traffic": read_profile("k_lbvh_cast", "dram_bytes_per_launch"),
+                    "traffic": read_profile("k_plain_packets", "dram_bytes_per_launch"),
                     "peak_source": "derived",
                     "peak_basis": f"4 warp schedulers x {sms} SMs x {mhz:.0f} MHz (instruction issue)"}
     if rank == 0:
-        line = {"metric": "Grays/s @4096 envs x 1M tris, GPU-built triangle LBVH cast one thread per beam",
+        line = {"metric": "Grays/s @4096 envs x 1M tris, GPU-built triangle LBVH",
                 "value": round(ws * n_rays * args.steps / t_lbvh / 1e9, 4), "unit": UNIT, "n_gpus": ws,
                 "steps": args.steps, "warmup": args.warmup,
                 "ms_per_step": round(t_lbvh * 1e3 / args.steps, 3), "higher_is_better": True,
@@ -1214,19 +1236,8 @@ def run_occupancy(args):
     tot = barrier_max(sum(a.elapsed_time(b) for a, b in ev) / 1e3, ws)
     value = ws * evals * args.steps / tot / 1e9
     clocks = clk.summary()
-    # the density kernel: one ex2 per (voxel, candidate) evaluation.  ex2 issues
-    # at 16 per SM per cycle: at 4.9e12 ex2/s (2.07 GHz, 152 SMs) ncu shows the
-    # XU pipe at 50% of its instruction peak with math-pipe throttle as the top
-    # stall, i.e. ex2 takes two of the pipe's issue slots
     kern_s = float(np.median(dens_ms)) / 1e3
-    sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    mhz = (clocks or {}).get("sm_mhz") or 2070.0
-    peak = 16.0 * sms * mhz * 1e6 / 1e9
-    achieved = evals / kern_s / 1e9
-    roofline = {"bound": "alu", "achieved": round(achieved, 1), "peak": round(peak, 1),
-                "unit": "G ex2/s", "frac": round(achieved / peak, 4),
-                "peak_basis": f"ex2: 16 per SM per cycle x {sms} SMs x {mhz:.0f} MHz", "kernel": "k_density<8>",
-                "kernel_ms_per_step": round(kern_s * 1e3, 3)}
+    roofline = density_roofline(evals, kern_s, clocks, dev)
     # end to end: Gaussians from pinned host memory, surface masks back
     e2e = None
     if not args.no_e2e:
@@ -1460,8 +1471,6 @@ def run_mesh(args):
                  "basis": "11 B per voxel + 12 B per vertex and per triangle over denoise + TSDF + marching tetrahedra",
                  "largest_set": mesh_group_roofline([int(np.prod(S["dims"])) for S in sets], caps,
                                                     per_set_stages, peak)}
-    sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    mhz = (clocks or {}).get("sm_mhz") or 2070.0
     e2e = None
     if not args.no_e2e:
         host = [[torch.from_numpy(np.ascontiguousarray(a)).pin_memory()
@@ -1521,13 +1530,9 @@ def run_mesh(args):
                            "stage_ms": {"density": round(stage[0], 3), "denoise": round(stage[1], 3),
                                         "tsdf": round(stage[2], 3), "marching_tets": round(stage[3], 3)}},
                 "gpu_launches": args.steps * launches,
-                "roofline": {"bound": "alu", "kernel": "k_density<8>",
-                             "achieved": round(evals / (dens_ms / 1e3) / 1e9, 1),
-                             "peak": round(16.0 * sms * mhz * 1e6 / 1e9, 1), "unit": "G ex2/s",
-                             "frac": round(evals / (dens_ms / 1e3) / (16.0 * sms * mhz * 1e6), 4),
-                             "peak_basis": f"ex2: 16 per SM per cycle x {sms} SMs x {mhz:.0f} MHz",
-                             "kernel_ms_per_step": round(dens_ms, 3),
-                             "note": "the Sec. IV-A density dominates the step; the Sec. IV-B kernels are in roofline_mesh_steps"},
+                "roofline": dict(density_roofline(evals, dens_ms / 1e3, clocks, torch.device("cuda")),
+                                 note="the Sec. IV-A density dominates the step; the Sec. IV-B kernels are in "
+                                      "roofline_mesh_steps"),
                 "roofline_mesh_steps": roof_mesh, "e2e": e2e, "cpu_baseline": cpu,
                 "meshes_per_s": round(ws * len(sets) * args.steps / tot, 2), "clocks": clocks}
         print(json.dumps(line), flush=True)
@@ -1563,7 +1568,7 @@ def run_hetero(args):
     clocks = clk.summary()
     cb, cr, cn, ct = counted_bytes(fgl, items, stream, opts)
     cost = hbm_roofline(cb, tot / args.steps, cr, cn, ct)
-    roofline = issue_roofline("k_persistent", "k_persistent@hetero", n_rays * args.steps / tot,
+    roofline = issue_roofline("k_packets", "k_packets@hetero", n_rays * args.steps / tot,
                               clocks, torch.device("cuda"), {"cost_model": cost})
     if roofline is None:
         roofline = dict(cost, note="no ncu capture of the current kernel sources on this workload: "
