@@ -374,7 +374,7 @@ typedef struct {
  * prefixes (eq. LCP; equal codes ordered by position), then node boxes bottom
  * up; leaf boxes are grown by 2^-17 max(1, max |coord|).  The binary tree is
  * then opened into the 8-wide nodes that the casts walk (91 B a triangle, plus
- * 48 B for the triangles in their order; the build's scratch, about 140 B a
+ * 48 B for the triangles in their order; the build's scratch, about 110 B a
  * triangle, stays with the LBVH for the next rebuild).  Synchronises
  * `stream` at the end.  Errors: FGL_ERR_INVALID (empty mesh, nt >= 2^30, a
  * vertex id out of range or a non-finite vertex), FGL_ERR_OOM, FGL_ERR_CUDA. */

@@ -86,6 +86,7 @@ fgl_status device_info(DeviceInfo* out) {
 struct Opts {
   int packet = 32, block = 128, sdepth = 6, bpsm = 0, graph = 0, refill = 32, postpone = 20,
       count = 0, tri_mode = 0;
+  bool own_packet = false;  // packet_rays was given
 };
 
 }  // namespace
@@ -144,6 +145,7 @@ fgl_status resolve_opts(const fgl_batch_opts* o, Opts* r) {
   if (s != FGL_OK) return s;
   if (stack_smem_bytes(8, d.block, d.sdepth) > di.smem_optin)
     return fail(FGL_ERR_INVALID, "block_threads * (8 + 24 * stack_smem) bytes (the width-8 stack) exceed shared memory");
+  d.own_packet = o && o->packet_rays;
   *r = d;
   return FGL_OK;
 }
@@ -272,6 +274,7 @@ struct Group {
   bool tmin = false;  // some item has min_range > 0
   std::vector<ItemDesc> items;
   int64_t n_packets = 0;
+  int packet_rays = 32;
 };
 
 // Options under which a warp may walk whole packets: they leave the leaf
@@ -289,16 +292,22 @@ bool packet_opts(int W, const Opts& o) {
 // percent there.
 void build_table(const fgl_cast_item* items, int n, const Opts& o, std::vector<Group>& groups,
                  std::vector<uint8_t>& table, std::vector<size_t>& offsets) {
-  const int P = o.packet;
   groups.clear();
   for (int W : {8, 4}) {
     Group g;
     g.W = W;
-    int64_t narrow = 0;  // packets of narrow sensors less those of the others
+    int64_t narrow = 0, rays = 0;  // packets of narrow sensors less those of the others
     for (int i = 0; i < n; ++i) {
       if (items[i].scene->bvh.width != W || items[i].n_env == 0) continue;
       const int64_t packets = (int64_t)items[i].n_env * ((items[i].sensor->n_rays + 31) / 32);
       narrow += items[i].sensor->narrow ? packets : -packets;
+      rays += (int64_t)items[i].n_env * items[i].sensor->n_rays;
+    }
+    g.packets = narrow >= 0 && packet_opts(W, o);
+    const int P = g.packets && !o.own_packet && small_cast(rays) ? 16 : o.packet;
+    g.packet_rays = P;
+    for (int i = 0; i < n; ++i) {
+      if (items[i].scene->bvh.width != W || items[i].n_env == 0) continue;
       ItemDesc d = make_desc(items[i]);
       d.pk_per_env = (d.n_rays + P - 1) / P;
       d.pk_begin = g.n_packets;
@@ -306,7 +315,6 @@ void build_table(const fgl_cast_item* items, int n, const Opts& o, std::vector<G
       g.tmin = g.tmin || d.min_range > 0.f;
       g.items.push_back(d);
     }
-    g.packets = narrow >= 0 && packet_opts(W, o);
     if (!g.items.empty()) groups.push_back(std::move(g));
   }
   table.clear();
@@ -319,7 +327,7 @@ void build_table(const fgl_cast_item* items, int n, const Opts& o, std::vector<G
     h.head = 0;
     h.n_packets = g.n_packets;
     h.n_items = (int32_t)g.items.size();
-    h.packet_rays = P;
+    h.packet_rays = g.packet_rays;
     table.resize(off + sizeof(BatchHeader) + g.items.size() * sizeof(ItemDesc));
     std::memcpy(table.data() + off, &h, sizeof(h));
     std::memcpy(table.data() + off + sizeof(h), g.items.data(), g.items.size() * sizeof(ItemDesc));
@@ -1119,7 +1127,7 @@ fgl_status fgl_autotune(const fgl_cast_item* items, int32_t n_items, const fgl_t
   const Dim dims[] = {
       {&fgl_batch_opts::tri_mode, {0, 1}},
       {&fgl_batch_opts::refill_min, {8, 16, 32}},
-      {&fgl_batch_opts::packet_rays, {32, 64, 128, 256}},
+      {&fgl_batch_opts::packet_rays, {0, 32, 64, 128, 256}},  // 0: the library's choice
       {&fgl_batch_opts::block_threads, {64, 128, 256}},
       {&fgl_batch_opts::stack_smem, {4, 8, 12, 16}},
   };

@@ -370,9 +370,10 @@ __device__ __forceinline__ void trace_packet(const ItemDesc& it, int env, int fi
   }
 }
 
-// k_plain with packet phases: warp w of the grid takes packet w of the item.
+// k_plain with packet phases: warp w of the grid takes packet w of the item,
+// `rays` rays (32, or 16 in a small cast; the other lanes copy the first).
 template <int W, bool COUNT, bool TMIN>
-__global__ void __maxnreg__(72) k_plain_packets(const ItemDesc it, int sdepth, unsigned* status) {
+__global__ void __maxnreg__(72) k_plain_packets(const ItemDesc it, int sdepth, unsigned* status, int rays) {
   using Keys = typename dev::KeyWords<W>::T;
   if (status == nullptr) status = &g_status;
   if (it.width != W) {  // never read nodes laid out for another width
@@ -382,13 +383,14 @@ __global__ void __maxnreg__(72) k_plain_packets(const ItemDesc it, int sdepth, u
   const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t env = (p >> 32) ? p / it.pk_per_env : (int64_t)((uint32_t)p / (uint32_t)it.pk_per_env);
   if (env >= it.n_env) return;
-  const int first = (int)(p - env * it.pk_per_env) * 32;
+  const int first = (int)(p - env * it.pk_per_env) * rays;
   const Smem<W> sm = smem_layout<W>(sdepth);
   uint2 ls[kStackLocal];
   Keys lq[kStackLocal];
   const dev::StackRefs<Keys> st{sm.ss, sm.sq, ls, lq, (int)blockDim.x, sdepth};
   uint32_t c[kWorkCounters] = {};
-  trace_packet<W, COUNT, TMIN>(it, (int)env, first, min(32, it.n_rays - first), sm, packet_smem(W, sdepth), st, status, c);
+  trace_packet<W, COUNT, TMIN>(it, (int)env, first, min(rays, it.n_rays - first), sm, packet_smem(W, sdepth), st, status,
+                               c);
   flush_counters<COUNT>(c);
 }
 
@@ -794,7 +796,8 @@ cudaError_t launch_plain(int W, bool count, bool packets, bool tmin, const ItemD
   if (total == 0) return cudaSuccess;
   if (tmin && (W != 8 || count)) return cudaErrorInvalidValue;  // no such form
   ItemDesc arg = it;
-  arg.pk_per_env = (it.n_rays + 31) / 32;
+  int rays = small_cast(total) ? 16 : 32;  // a packet
+  arg.pk_per_env = (it.n_rays + rays - 1) / rays;
   const int64_t threads = packets ? (int64_t)it.n_env * arg.pk_per_env * 32 : total;
   const int64_t grid = (threads + block - 1) / block;
   const size_t smem = packets ? packets_smem_bytes(W, block, sdepth) : stack_smem_bytes(W, block, sdepth);
@@ -802,7 +805,7 @@ cudaError_t launch_plain(int W, bool count, bool packets, bool tmin, const ItemD
   const cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
   void* plain_args[] = {&arg, &sdepth, &tri_mode, &postpone_pct, &status};
-  void* packet_args[] = {&arg, &sdepth, &status};
+  void* packet_args[] = {&arg, &sdepth, &status, &rays};
   return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(block), packets ? packet_args : plain_args, smem, s);
 }
 

@@ -16,6 +16,14 @@ size_t stack_smem_bytes(int W, int block, int sdepth);
 // tri_mode 0: warp-pooled leaf tests; 1: lane-serial with postponing.
 // packets: one packet of 32 rays of an environment a warp, walked together
 // before the per-ray traversal (needs tri_mode 0; see packets_fit).
+// A cast or batch of so few rays that packets of 16 come to at most two for each
+// of the 28 warps an SM holds leaves the chip waiting for its slowest packets:
+// half of the lanes idle there, but a packet ends sooner (1 M triangles, 57,600
+// rays 42 -> 35 us, 5,760 53 -> 44, 131,072 51 -> 44; 184,320 would take 82
+// instead of 75).
+constexpr int64_t kSmallCastRays = 16 * 2 * 28 * 152;
+inline bool small_cast(int64_t rays) { return rays <= kSmallCastRays; }
+
 // tmin honours it.min_range (8-wide nodes, not counted); status: the word that
 // takes traversal errors (null: the shared one).
 cudaError_t launch_plain(int W, bool count, bool packets, bool tmin, const ItemDesc& it, unsigned* status, int block,

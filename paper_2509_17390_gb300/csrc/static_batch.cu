@@ -137,14 +137,20 @@ extern "C" fgl_status fgl_cast_batched_static(const fgl_cast_item* items, int32_
     const size_t hdr_off = used;
     size_t off = used + sizeof(BatchHeader);
     int n_in = 0;
-    int64_t packets = 0;
+    int64_t packets = 0, rays = 0;
     bool tmin = false;
+    for (int i = 0; i < n_items; ++i) {
+      if (widths[i] != W) continue;
+      const int64_t warps = (int64_t)descs[i].n_env * ((descs[i].n_rays + 31) / 32);
+      together += narrow[i] ? warps : -warps;
+      rays += (int64_t)descs[i].n_env * descs[i].n_rays;
+    }
+    const bool walk = together >= 0 && tri_mode == 0 && refill == 32 && packets_fit(W, block, sdepth);
+    const int per = walk && !(opts && opts->packet_rays) && small_cast(rays) ? 16 : packet;
     for (int i = 0; i < n_items; ++i) {
       ItemDesc d = descs[i];
       if (widths[i] != W || d.n_env == 0) continue;
-      const int64_t warps = (int64_t)d.n_env * ((d.n_rays + 31) / 32);
-      together += narrow[i] ? warps : -warps;
-      d.pk_per_env = (d.n_rays + packet - 1) / packet;
+      d.pk_per_env = (d.n_rays + per - 1) / per;
       d.pk_begin = packets;
       packets += (int64_t)d.pk_per_env * d.n_env;
       tmin = tmin || d.min_range > 0.f;
@@ -156,12 +162,12 @@ extern "C" fgl_status fgl_cast_batched_static(const fgl_cast_item* items, int32_
     h.head = 0;  // the queue starts empty on every call
     h.n_packets = packets;
     h.n_items = n_in;
-    h.packet_rays = packet;
+    h.packet_rays = per;
     std::memcpy((char*)img.words + hdr_off, &h, sizeof(h));
     group_off[n_groups] = hdr_off;
     group_w[n_groups] = W;
     group_tmin[n_groups] = tmin;
-    group_packets[n_groups] = together >= 0 && tri_mode == 0 && refill == 32 && packets_fit(W, block, sdepth);
+    group_packets[n_groups] = walk;
     ++n_groups;
     used = off;
   }

@@ -122,3 +122,21 @@ def test_mixed_batch_and_static_form():
         for mode in ("default", "static"):
             for (r0, i0), (r1, i1) in zip(outs["serial"], outs[mode]):
                 assert torch.equal(r0.view(torch.int32), r1.view(torch.int32)) and torch.equal(i0, i1)
+
+
+# either side of the size up to which a packet is 16 rays (136,192 rays), whole
+# and partial packets: one launch, the batch and the batch without allocation
+@pytest.mark.parametrize("beams,az,envs", [(16, 266, 32), (16, 267, 32), (7, 45, 432), (7, 45, 433), (5, 9, 1)])
+def test_small_and_large_casts(beams, az, envs):
+    v, t, room = scene_parts("boxes")
+    sc = fgl.Scene(v, t)
+    se = fgl.Sensor.from_table(synth.grid_sensor(beams, -20, 20, az))
+    P = torch.from_numpy(np.resize(poses(room), (envs, 3, 4))).cuda()
+    ref = cast((sc, se, P, 50.0, 0.0), fgl.BatchOpts(tri_mode=1))
+    got = [cast((sc, se, P, 50.0, 0.0), None), cast((sc, se, P, 50.0, 0.0), fgl.BatchOpts(packet_rays=32)),
+           fgl.cast(sc, se, P, 50.0)]
+    r, i = torch.empty_like(ref[0]), torch.empty_like(ref[1])
+    fgl.cast_batched_static([(sc, se, P, 50.0, r, i)])
+    fgl.sync()
+    for a, b in got + [(r, i)]:
+        assert torch.equal(a.reshape(-1).view(torch.int32), ref[0].view(torch.int32)) and torch.equal(b.reshape(-1), ref[1])
