@@ -656,7 +656,7 @@ extern "C" fgl_status fgl_lbvh_build(const float* d_verts, int64_t nv, const int
   auto take = [&](size_t bytes) { size_t o = off; off = al256(off + bytes); return o; };
   const size_t o_tbox = take((size_t)nt * 32), o_k0 = take((size_t)nt * 4), o_v0 = take((size_t)nt * 4),
                o_k1 = take((size_t)nt * 4), o_v1 = take((size_t)nt * 4), o_par = take((size_t)nt * 4),
-               o_flags = take(n_in * 4), o_nbox = take(n_in * 32), o_lbox = take((size_t)nt * 32),
+               o_flags = take(n_in * 4), o_lbox = take((size_t)nt * 32),
                o_sort = take(radix_sort_tmp_elems(nt) * 4), o_split = take(n_in * 4),
                o_roots = take((size_t)nt * 8), o_wroot = take((size_t)wide_capacity(nt) * 16),
                o_bounds = take(sizeof(int) * (16 + kWideLevels));
@@ -678,7 +678,7 @@ extern "C" fgl_status fgl_lbvh_build(const float* d_verts, int64_t nv, const int
            *v1 = (uint32_t*)(w + o_v1);
   int32_t* par = (int32_t*)(w + o_par);
   uint32_t* flags = (uint32_t*)(w + o_flags);
-  float4* nbox = (float4*)(w + o_nbox);
+  float4* nbox = tbox;  // the triangles' boxes are done with once gathered
   float4* lbox = (float4*)(w + o_lbox);
   int* bounds = (int*)(w + o_bounds);
   // words 0..6 the bounds, 7 the depth, 8 the status, 9 the block roots, 10 the

@@ -1136,15 +1136,16 @@ __global__ void __launch_bounds__(kShellThreads) k_shell_phi(const uint32_t* __r
     s_word[i] = make_uint4(c[u][0], c[u][1], c[u][2], ob);
   }
   __syncthreads();
-  const int xb = (x0 + 1) * 32 + lane;
+  const int xw0 = (x0 + 1) * 32;  // below nx
 #pragma unroll 1
   for (int row = wid; row < kShellRows * kShellRows; row += kShellThreads / 32) {
     const int j = y0 + H + row % kShellRows, k = z0 + H + row / kShellRows;
     if (j >= g.ny || k >= g.nz) continue;
     const int64_t v0 = ((int64_t)k * g.ny + j) * g.nx;
-    float* dst = phi + v0 + xb;
+    const int64_t at = v0 + xw0 + lane;
+    float* dst = phi + at;
     const uint4* words = s_word + row * tw;
-    int left = g.nx - xb;  // voxels of the row from this lane's on
+    int left = g.nx - xw0 - lane;  // voxels of the row from this lane's on
 #pragma unroll 2
     for (int x = 0; x < tw; ++x, left -= 32) {
       const uint4 w = words[x];
@@ -1157,8 +1158,8 @@ __global__ void __launch_bounds__(kShellThreads) k_shell_phi(const uint32_t* __r
       }
       if (left > 0) {
         dst[32 * x] = f;
-        if (EXTRA && out_outside) out_outside[v0 + xb + 32 * x] = (uint8_t)out;
-        if (EXTRA && out_shell) out_shell[v0 + xb + 32 * x] = s_p[held];
+        if (EXTRA && out_outside) out_outside[at + 32 * x] = (uint8_t)out;
+        if (EXTRA && out_shell) out_shell[at + 32 * x] = s_p[held];
       }
     }
   }
