@@ -1567,7 +1567,7 @@ __device__ __forceinline__ void store3(uint32_t* stage, const uint32_t v[3], int
 // A warp takes 32 samples with a vertex at once: a lane a sample for its edge
 // types, value and gradient, then a lane a vertex (1 to 7 a sample), written in
 // whole lines -- the samples' vertices lie next to each other, as their list
-// does.  Bound by issue and the latency of the gathers from phi.  1.3 M
+// does.  Bound by issue and the latency of the gathers from phi.  2.2 M
 // vertices with normals: 83 us (a thread a sample, its vertices in turn) -> 54.
 constexpr int kMtWarps = 8;
 
@@ -1667,7 +1667,7 @@ __global__ void __launch_bounds__(32 * kMtWarps) k_mt_verts(EmitArgs a, const ui
 // list) and its triangles' table codes, then a lane a triangle (1 to 12 a
 // cube), written in whole lines.  Corner c = dx + 2 dy + 4 dz owns the edges of
 // types t from its sample; corners 0..6 sit in four words (one a (dy, dz) row;
-// the dx = 1 corner in the next word when x is its word's last bit).  2.6 M
+// the dx = 1 corner in the next word when x is its word's last bit).  4.5 M
 // triangles: 66 us (a thread a cube, its triangles in turn, the corners'
 // vertices counted from the seven crossing words each) -> 34.
 __global__ void __launch_bounds__(32 * kMtWarps) k_mt_tris(EmitArgs a, const uint32_t* __restrict__ cubes_in,
