@@ -411,6 +411,12 @@ __global__ void __maxnreg__(72) k_plain_packets(const ItemDesc it, int sdepth, u
 constexpr unsigned long long kDrawLeft = 16;
 constexpr unsigned kDrawMany = 3;
 
+// k_packets' own shared memory, beside the launch's dynamic part.
+struct PacketQueue {
+  unsigned long long next[kMaxBlockWarps], end[kMaxBlockWarps];  // the warp's own packets
+  unsigned long long total;  // not read again beside the counter, whose line the draws keep busy
+};
+
 template <int W, bool COUNT, bool TMIN>
 __global__ void __maxnreg__(72) k_packets(BatchHeader* __restrict__ hdr, const ItemDesc* __restrict__ items,
                                            int sdepth) {
@@ -423,26 +429,25 @@ __global__ void __maxnreg__(72) k_packets(BatchHeader* __restrict__ hdr, const I
   Keys lq[kStackLocal];
   const dev::StackRefs<Keys> st{sm.ss, sm.sq, ls, lq, (int)blockDim.x, sdepth};
   uint32_t c[kWorkCounters] = {};
-  __shared__ unsigned long long s_next[kMaxBlockWarps], s_end[kMaxBlockWarps];  // the warp's own packets
-  __shared__ unsigned long long s_total;  // not read again beside the counter, whose line the draws keep busy
+  __shared__ PacketQueue q;
   const int wid = threadIdx.x >> 5;
-  if (lane == 0) s_next[wid] = s_end[wid] = 0ull;
-  if (threadIdx.x == 0) s_total = (unsigned long long)hdr->n_packets;
+  if (lane == 0) q.next[wid] = q.end[wid] = 0ull;
+  if (threadIdx.x == 0) q.total = (unsigned long long)hdr->n_packets;
   __syncthreads();
   for (;;) {
     unsigned long long p = 0;
     if (lane == 0) {
-      p = s_next[wid];
-      if (p == s_end[wid]) {
-        const unsigned long long total = s_total;
+      p = q.next[wid];
+      if (p == q.end[wid]) {
+        const unsigned long long total = q.total;
         const unsigned draw = p + kDrawLeft * (gridDim.x * (blockDim.x >> 5)) < total ? kDrawMany : 1u;
         p = atomicAdd(&hdr->head, (unsigned long long)draw);
-        s_end[wid] = p < total ? min(p + draw, total) : p;
+        q.end[wid] = p < total ? min(p + draw, total) : p;
       }
-      s_next[wid] = p + 1;
+      q.next[wid] = p + 1;
     }
     p = __shfl_sync(FULL, p, 0);
-    if (p >= s_total) break;
+    if (p >= q.total) break;
     int lo = 0, hi = hdr->n_items - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
@@ -776,17 +781,23 @@ static size_t packets_smem_bytes(int W, int block, int sdepth) {
   return stack_smem_bytes(W, block, sdepth) + (size_t)block * (sizeof(uint2) + sizeof(uint32_t));
 }
 
+// The limits hold for a kernel's dynamic and static shared memory together;
+// kStaticSmem covers the static part of every traversal kernel (at most 320 B).
+constexpr size_t kStaticSmem = 512;
+static_assert(sizeof(PacketQueue) + 16 <= kStaticSmem, "static shared memory");
+
 bool packets_fit(int W, int block, int sdepth) {
-  if (packets_smem_bytes(W, block, sdepth) <= 48 * 1024) return true;  // any block's: no need to ask the device
+  const size_t smem = packets_smem_bytes(W, block, sdepth) + kStaticSmem;
+  if (smem <= 48 * 1024) return true;  // any block's: no need to ask the device
   int dev = 0, optin = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
     return false;
-  return packets_smem_bytes(W, block, sdepth) <= (size_t)optin;
+  return smem <= (size_t)optin;
 }
 
 static cudaError_t allow_smem(void* fn, size_t smem) {
-  if (smem <= 48 * 1024) return cudaSuccess;
+  if (smem + kStaticSmem <= 48 * 1024) return cudaSuccess;
   return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
