@@ -437,7 +437,9 @@ fgl_status enqueue_batch(BatchCtx& c, const std::vector<Group>& groups,
 }
 
 // Bytes of the launches beyond the work-queue table (they are baked into a
-// captured graph, so they are part of its key).
+// captured graph, so they are part of its key).  An instance's bounds and record
+// counts are launch arguments too, and a scene built after another was
+// destroyed may have its addresses.
 void extras_key(const fgl_cast_item* items, int n, std::vector<uint8_t>& key) {
   auto put = [&](const void* p, size_t b) {
     key.insert(key.end(), (const uint8_t*)p, (const uint8_t*)p + b);
@@ -453,7 +455,12 @@ void extras_key(const fgl_cast_item* items, int n, std::vector<uint8_t>& key) {
     for (int k = 0; k < it.n_instances; ++k) {
       put(&it.instances[k]->d_nodes, sizeof(void*));
       put(&it.instances[k]->d_tris, sizeof(void*));
-      put(&it.instances[k]->bvh.width, sizeof(int));
+      const HostBVH& b = it.instances[k]->bvh;
+      put(&b.width, sizeof(b.width));
+      put(b.lo, sizeof(b.lo));
+      put(b.hi, sizeof(b.hi));
+      put(&b.n_nodes, sizeof(b.n_nodes));
+      put(&b.n_tris, sizeof(b.n_tris));
     }
   }
 }
