@@ -378,7 +378,9 @@ typedef struct {
  * 48 B for the triangles in their order; the build's scratch, about 110 B a
  * triangle, stays with the LBVH for the next rebuild).  Synchronises
  * `stream` at the end.  Errors: FGL_ERR_INVALID (empty mesh, nt >= 2^30, a
- * vertex id out of range or a non-finite vertex), FGL_ERR_OOM, FGL_ERR_CUDA. */
+ * vertex id out of range or a non-finite vertex), FGL_ERR_OOM, FGL_ERR_CUDA.
+ * A rebuild that fails leaves no tree: casts and exports return
+ * FGL_ERR_INVALID until one succeeds. */
 fgl_status fgl_lbvh_build(const float* verts, int64_t nv, const int32_t* tris, int64_t nt,
                           fgl_stream stream, fgl_lbvh* out);
 fgl_status fgl_lbvh_destroy(fgl_lbvh lbvh);

@@ -856,6 +856,7 @@ fgl_status fgl_cast_lbvh(fgl_lbvh lbvh, fgl_sensor sensor, const float* poses, i
                          float min_range, float max_range, float* out_range, int32_t* out_tri,
                          fgl_stream stream) {
   if (!lbvh || !sensor) return fail(FGL_ERR_INVALID, "null LBVH or sensor");
+  if (!lbvh_built(lbvh)) return fail(FGL_ERR_INVALID, "the LBVH holds no tree: its last build failed");
   if (n_env < 0) return fail(FGL_ERR_INVALID, "n_env < 0");
   if (!(std::isfinite(max_range) && max_range > 0.f))
     return fail(FGL_ERR_INVALID, "max_range must be finite and > 0");

@@ -61,6 +61,7 @@ cudaError_t launch_points(const ItemDesc& it, float* out, cudaStream_t s);
 // ranges and outputs to be filled in) and its own status word (lbvh.cu).
 ItemDesc lbvh_item(const fgl_lbvh_s* L);
 unsigned* lbvh_status(const fgl_lbvh_s* L);
+bool lbvh_built(const fgl_lbvh_s* L);  // false after a build that failed: nothing to cast or export
 
 // Debug export of world rays (beam order).
 cudaError_t launch_l2_read(const void* buf, int64_t bytes, int reps, unsigned* sink, int sms,

@@ -40,6 +40,7 @@ using namespace fgl;
 struct fgl_lbvh_s {
   int device = -1;
   int64_t nt = 0;
+  bool built = false;          // the arrays hold the tree of the last build, which succeeded
   unsigned* status = nullptr;  // device word: bit 0 = a cast's stack overflowed, bit 2 = an
                                // index out of range (checked library)
   void* nodes = nullptr;   // (nt - 1) x 64 B
@@ -606,6 +607,7 @@ ItemDesc lbvh_item(const fgl_lbvh_s* L) {
 }
 
 unsigned* lbvh_status(const fgl_lbvh_s* L) { return L->status; }
+bool lbvh_built(const fgl_lbvh_s* L) { return L->built; }
 }  // namespace fgl
 
 extern "C" fgl_status fgl_lbvh_build(const float* d_verts, int64_t nv, const int32_t* d_tris,
@@ -626,6 +628,7 @@ extern "C" fgl_status fgl_lbvh_build(const float* d_verts, int64_t nv, const int
       return err(FGL_ERR_OOM, "cannot allocate the LBVH status word");
     }
   }
+  L->built = false;  // from here on the arrays change: no casts until the build is through
   if (L->nt != nt) {
     for (void** b : {&L->nodes, &L->tris, &L->wnodes, &L->wtris}) {
       if (*b) cudaFree(*b);
@@ -747,6 +750,7 @@ extern "C" fgl_status fgl_lbvh_build(const float* d_verts, int64_t nv, const int
   }
   L->margin = std::ldexp(std::max(1.f, iord(host[6])), -17);
   L->depth = nt > 1 ? host[7] : 1;
+  L->built = true;
   cudaGetDevice(&L->device);
   L->build_ms =
       (float)std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
@@ -785,6 +789,7 @@ extern "C" fgl_status fgl_lbvh_get_stats(fgl_lbvh L, fgl_lbvh_stats* o) {
 extern "C" fgl_status fgl_lbvh_export(fgl_lbvh L, void* nodes, int64_t node_bytes, void* tris,
                                       int64_t tri_bytes) {
   if (!L) return err(FGL_ERR_INVALID, "null LBVH");
+  if (!L->built) return err(FGL_ERR_INVALID, "the LBVH holds no tree: its last build failed");
   const int64_t nb = (L->nt > 1 ? L->nt - 1 : 0) * (int64_t)sizeof(LbvhNode), tb = L->nt * 48;
   if (nodes) {
     if (node_bytes != nb) return err(FGL_ERR_INVALID, "node_bytes mismatch");
