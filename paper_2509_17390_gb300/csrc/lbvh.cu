@@ -41,11 +41,12 @@ struct fgl_lbvh_s {
   int device = -1;
   int64_t nt = 0;
   bool built = false;          // the arrays hold the tree of the last build, which succeeded
+  int64_t n_wide = 0;
   unsigned* status = nullptr;  // device word: bit 0 = a cast's stack overflowed, bit 2 = an
                                // index out of range (checked library)
   void* nodes = nullptr;   // (nt - 1) x 64 B
   void* tris = nullptr;    // nt x 48 B, Morton order
-  void* wnodes = nullptr;  // wide_capacity(nt) x 256 B: what the casts walk
+  void* wnodes = nullptr;  // wide_capacity(nt) x 256 B, n_wide of them made: what the casts walk
   void* wtris = nullptr;   // nt x 48 B, the wide nodes' leaf runs
   void* work = nullptr;    // build scratch
   size_t work_cap = 0;
@@ -601,7 +602,7 @@ ItemDesc lbvh_item(const fgl_lbvh_s* L) {
   d.nodes = L->wnodes;
   d.tris = L->wtris;
   d.width = 8;
-  d.n_nodes = (uint32_t)wide_capacity(L->nt);
+  d.n_nodes = (uint32_t)L->n_wide;
   d.n_tris = (uint32_t)L->nt;
   return d;
 }
@@ -736,7 +737,7 @@ extern "C" fgl_status fgl_lbvh_build(const float* d_verts, int64_t nv, const int
     void* args[] = {&a};
     LCUDA(cudaLaunchCooperativeKernel((const void*)k_lbvh_wide, dim3(blocks), dim3(256), args, 0, s));
   }
-  int host[16];
+  int host[16 + kWideLevels];
   LCUDA(cudaMemcpyAsync(host, bounds, sizeof(host), cudaMemcpyDeviceToHost, s));
   LCUDA(cudaStreamSynchronize(s));
   const int32_t st = host[8];
@@ -750,6 +751,8 @@ extern "C" fgl_status fgl_lbvh_build(const float* d_verts, int64_t nv, const int
   }
   L->margin = std::ldexp(std::max(1.f, iord(host[6])), -17);
   L->depth = nt > 1 ? host[7] : 1;
+  L->n_wide = 1;
+  for (int lv = 0; lv < kWideLevels; ++lv) L->n_wide += host[16 + lv];
   L->built = true;
   cudaGetDevice(&L->device);
   L->build_ms =
