@@ -865,6 +865,15 @@ fgl_status fgl_cast_lbvh(fgl_lbvh lbvh, fgl_sensor sensor, const float* poses, i
   if (n_env > 0 && (!poses || !out_range || !out_tri))
     return fail(FGL_ERR_INVALID, "null poses or output pointer");
   if (n_env == 0) return FGL_OK;
+  // Rays walked one by one take the binary tree, which is the faster one for
+  // them: 20,000 x 32 of a rosette on 250 k triangles 310 us, 344 over the 8-wide
+  // nodes (2 k triangles 49 and 54); 16 rays x 10,000 125 and 154.
+  const Opts o;
+  if (!sensor->narrow || !packet_opts(8, o)) {
+    FGL_CUDA(launch_lbvh_cast(lbvh, sensor->d_dirs, poses, n_env, sensor->n_rays, min_range, max_range, out_range,
+                              out_tri, (cudaStream_t)stream));
+    return FGL_OK;
+  }
   ItemDesc d = lbvh_item(lbvh);
   d.dirs = sensor->d_dirs;
   d.poses = poses;
@@ -874,9 +883,8 @@ fgl_status fgl_cast_lbvh(fgl_lbvh lbvh, fgl_sensor sensor, const float* poses, i
   d.n_rays = sensor->n_rays;
   d.max_range = max_range;
   d.min_range = min_range;
-  const Opts o;
-  FGL_CUDA(launch_plain(8, false, sensor->narrow && packet_opts(8, o), min_range > 0.f, d, lbvh_status(lbvh),
-                        o.block, o.sdepth, o.tri_mode, o.postpone, (cudaStream_t)stream));
+  FGL_CUDA(launch_plain(8, false, true, min_range > 0.f, d, lbvh_status(lbvh), o.block, o.sdepth, o.tri_mode,
+                        o.postpone, (cudaStream_t)stream));
   return FGL_OK;
 }
 

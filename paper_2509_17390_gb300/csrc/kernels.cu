@@ -67,7 +67,7 @@ __device__ __forceinline__ Smem<W> smem_layout(int sdepth) {
   return m;
 }
 
-template <int W, bool COUNT, bool TMIN>
+template <int W, bool COUNT>
 __global__ void __maxnreg__(72) k_plain(const ItemDesc it, int sdepth, int tri_mode, int postpone_pct,
                                         unsigned* status) {
   using Keys = typename dev::KeyWords<W>::T;
@@ -84,7 +84,7 @@ __global__ void __maxnreg__(72) k_plain(const ItemDesc it, int sdepth, int tri_m
   bool done = gid >= total;
   int env = 0;
   float4 ds = make_float4(0.f, 0.f, 0.f, 0.f);
-  dev::Tracer<W, COUNT, TMIN> tr;
+  dev::Tracer<W, COUNT> tr;
   tr.tg = make_uint2(0u, 0u);
   tr.ng = make_uint2(0u, 0u);
   if (COUNT) tr.n_nodes = tr.n_tris = tr.n_rounds = tr.n_pops = 0;
@@ -750,12 +750,11 @@ void* persistent_fn() {
   return (void*)k_persistent<W, COUNT, TMIN>;
 }
 
-// A minimum range comes with a GPU-built hierarchy only (8-wide, not counted).
-void* pick_plain(int W, bool count, bool tmin) {
-  if (W == 8 && tmin) return (void*)k_plain<8, false, true>;
-  if (W == 8) return count ? (void*)k_plain<8, true, false> : (void*)k_plain<8, false, false>;
-  return count ? (void*)k_plain<4, true, false> : (void*)k_plain<4, false, false>;
+void* pick_plain(int W, bool count) {
+  if (W == 8) return count ? (void*)k_plain<8, true> : (void*)k_plain<8, false>;
+  return count ? (void*)k_plain<4, true> : (void*)k_plain<4, false>;
 }
+// A minimum range comes with a GPU-built hierarchy only (8-wide, not counted).
 void* pick_plain_packets(int W, bool count, bool tmin) {
   if (W == 8 && tmin) return (void*)k_plain_packets<8, false, true>;
   if (W == 8) return count ? (void*)k_plain_packets<8, true, false> : (void*)k_plain_packets<8, false, false>;
@@ -805,14 +804,14 @@ cudaError_t launch_plain(int W, bool count, bool packets, bool tmin, const ItemD
                          int sdepth, int tri_mode, int postpone_pct, cudaStream_t s) {
   const int64_t total = (int64_t)it.n_env * it.n_rays;
   if (total == 0) return cudaSuccess;
-  if (tmin && (W != 8 || count)) return cudaErrorInvalidValue;  // no such form
+  if (tmin && (W != 8 || count || !packets)) return cudaErrorInvalidValue;  // no such form
   ItemDesc arg = it;
   int rays = small_cast(total) ? 16 : 32;  // a packet
   arg.pk_per_env = (it.n_rays + rays - 1) / rays;
   const int64_t threads = packets ? (int64_t)it.n_env * arg.pk_per_env * 32 : total;
   const int64_t grid = (threads + block - 1) / block;
   const size_t smem = packets ? packets_smem_bytes(W, block, sdepth) : stack_smem_bytes(W, block, sdepth);
-  void* fn = packets ? pick_plain_packets(W, count, tmin) : pick_plain(W, count, tmin);
+  void* fn = packets ? pick_plain_packets(W, count, tmin) : pick_plain(W, count);
   const cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
   void* plain_args[] = {&arg, &sdepth, &tri_mode, &postpone_pct, &status};

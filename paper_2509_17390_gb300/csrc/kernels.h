@@ -24,7 +24,7 @@ size_t stack_smem_bytes(int W, int block, int sdepth);
 constexpr int64_t kSmallCastRays = 16 * 2 * 28 * 152;
 inline bool small_cast(int64_t rays) { return rays <= kSmallCastRays; }
 
-// tmin honours it.min_range (8-wide nodes, not counted); status: the word that
+// tmin honours it.min_range (8-wide packets, not counted); status: the word that
 // takes traversal errors (null: the shared one).
 cudaError_t launch_plain(int W, bool count, bool packets, bool tmin, const ItemDesc& it, unsigned* status, int block,
                          int sdepth, int tri_mode, int postpone_pct, cudaStream_t s);
@@ -57,8 +57,12 @@ cudaError_t launch_instance_pass(const InstancePass& a, bool tmin, int block, in
 // World-frame return points of one item, after its scene and instance passes.
 cudaError_t launch_points(const ItemDesc& it, float* out, cudaStream_t s);
 
-// The wide form of a GPU-built triangle LBVH as an item (sensor, poses,
-// ranges and outputs to be filled in) and its own status word (lbvh.cu).
+// One-thread-per-ray cast over a GPU-built triangle LBVH's binary tree; the wide
+// form as an item (sensor, poses, ranges and outputs to be filled in) and the
+// LBVH's own status word (lbvh.cu).
+cudaError_t launch_lbvh_cast(const fgl_lbvh_s* L, const void* dirs, const float* poses, int n_env,
+                             int n_rays, float min_range, float max_range, float* out_range,
+                             int32_t* out_tri, cudaStream_t s);
 ItemDesc lbvh_item(const fgl_lbvh_s* L);
 unsigned* lbvh_status(const fgl_lbvh_s* L);
 bool lbvh_built(const fgl_lbvh_s* L);  // false after a build that failed: nothing to cast or export

@@ -14,11 +14,12 @@
 // grown by the margin 2^-17 max(1, max |coord|), which covers the float32
 // rounding of the slab tests, so culling never drops a triangle the ray meets.
 //
-// Cast: the wide nodes are the host-built BVH's record, so the rays go through
-// the same kernels -- and both give bitwise identical returns.  2.9 M rays on
-// 500 k triangles: 0.76 ms (the binary tree, one thread a beam: 0.96), and the
-// build that makes the wide nodes takes 0.30 ms (without them, before its
-// climb moved to shared memory: 0.40).
+// Cast: the wide nodes are the host-built BVH's record, so packets of rays go
+// through the same kernels; rays walked one by one go through the binary tree.
+// The triangle test and the (t, id) rule are the same everywhere, so all give
+// bitwise identical returns.  2.9 M rays on 500 k triangles: 0.76 ms (the binary
+// tree: 0.96), and the build that makes the wide nodes takes 0.30 ms (without
+// them, before its climb moved to shared memory: 0.40).
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -46,7 +47,7 @@ struct fgl_lbvh_s {
                                // index out of range (checked library)
   void* nodes = nullptr;   // (nt - 1) x 64 B
   void* tris = nullptr;    // nt x 48 B, Morton order
-  void* wnodes = nullptr;  // wide_capacity(nt) x 256 B, n_wide of them made: what the casts walk
+  void* wnodes = nullptr;  // wide_capacity(nt) x 256 B, n_wide of them made: what packets walk
   void* wtris = nullptr;   // nt x 48 B, the wide nodes' leaf runs
   void* work = nullptr;    // build scratch
   size_t work_cap = 0;
@@ -580,6 +581,136 @@ __global__ void __launch_bounds__(256) k_lbvh_wide(const WideArgs a) {
   }
 }
 
+// ---------------------------------------------------------------------------
+// cast over the binary tree: one thread per ray, a local stack of nodes with
+// their entry distances, nearer child first, children and stacked nodes beyond
+// the best hit culled
+// ---------------------------------------------------------------------------
+constexpr int kLbvhStack = 96;
+
+struct LbvhCast {
+  const LbvhNode* nodes;
+  const float4* tris;
+  int64_t nt;
+  const float4* dirs;
+  const float* poses;
+  int32_t n_env, n_rays;
+  float min_range, max_range;
+  float* out_range;
+  int32_t* out_tri;
+};
+
+// Slab test of one child box against (best) with the ray's precomputed
+// -o * inv_d offsets: t = fma(plane, inv_d, -o inv_d).
+__device__ __forceinline__ bool slab(float lx, float ly, float lz, float hx, float hy, float hz,
+                                     const dev::Ray& r, float nox, float noy, float noz,
+                                     float tmin, float tmax, float& tn) {
+  const float x0 = fmaf(lx, r.ix, nox), x1 = fmaf(hx, r.ix, nox);
+  const float y0 = fmaf(ly, r.iy, noy), y1 = fmaf(hy, r.iy, noy);
+  const float z0 = fmaf(lz, r.iz, noz), z1 = fmaf(hz, r.iz, noz);
+  tn = dev::max3f(fminf(x0, x1), fminf(y0, y1), fmaxf(fminf(z0, z1), tmin));
+  const float tf = dev::min3f(fmaxf(x0, x1), fmaxf(y0, y1), fminf(fmaxf(z0, z1), tmax));
+  return tn <= tf;
+}
+
+template <bool TMIN>
+__global__ void k_lbvh_cast(const LbvhCast a, unsigned* status) {
+  const int64_t total = (int64_t)a.n_env * a.n_rays;
+  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (gid >= total) return;
+  const int env = (int)(gid / a.n_rays);
+  const int j = (int)(gid - (int64_t)env * a.n_rays);
+  const float4 ds = __ldg(a.dirs + j);
+  float ox, oy, oz, dx, dy, dz;
+  dev::world_ray(a.poses + 12 * (int64_t)env, ds, ox, oy, oz, dx, dy, dz);
+  dev::Tracer<8, false, TMIN> tr;  // ray, best hit and the (t, id) rule; no wide traversal
+  dev::setup_ray(tr.r, ox, oy, oz, dx, dy, dz);
+  tr.tmin_ = TMIN ? a.min_range : 0.f;
+  tr.best_t = a.max_range;
+  tr.best_id = dev::kNoHit;
+  const float tmin = TMIN ? a.min_range : 0.f;
+  const float nox = -ox * tr.r.ix, noy = -oy * tr.r.iy, noz = -oz * tr.r.iz;
+  auto test_tri = [&](int64_t k) {
+#ifdef FGL_CHECKED
+    if (k < 0 || k >= (int64_t)a.nt) {  // checked library: no read past the triangles
+      atomicOr(status, 4u);
+      return;
+    }
+#endif
+    const float4* tp = a.tris + 3 * k;
+    const float4 v0 = __ldg(tp), v1 = __ldg(tp + 1), v2 = __ldg(tp + 2);
+    tr.consider(dev::tri_hit(tr.r, v0, v1, v2, tr.best_t), __float_as_int(v0.w));
+  };
+  if (a.nt == 1) {
+    test_tri(0);
+  } else {
+    int stack[kLbvhStack];
+    float stq[kLbvhStack];
+    int sp = 0;
+    int node = 0;
+    for (;;) {
+#ifdef FGL_CHECKED
+      if (node < 0 || (int64_t)node >= (int64_t)a.nt - 1) {  // checked library: no read past the nodes
+        atomicOr(status, 4u);
+        break;
+      }
+#endif
+      const LbvhNode* nd = a.nodes + node;
+      const float4 A = __ldg(&nd->a), B = __ldg(&nd->b), C = __ldg(&nd->c);
+      const int4 D = __ldg(&nd->d);
+      float tl, trr;
+      bool hl = slab(A.x, A.y, A.z, A.w, B.x, B.y, tr.r, nox, noy, noz, tmin, tr.best_t, tl);
+      bool hr = slab(B.z, B.w, C.x, C.y, C.z, C.w, tr.r, nox, noy, noz, tmin, tr.best_t, trr);
+      if (hl && D.x < 0) {
+        test_tri(~D.x);
+        hl = false;
+      }
+      if (hr && D.y < 0) {
+        test_tri(~D.y);
+        hr = false;
+      }
+      hl = hl && tl <= tr.best_t;
+      hr = hr && trr <= tr.best_t;
+      if (hl && hr) {
+        const bool lfirst = tl <= trr;
+        if (sp >= kLbvhStack) {
+          atomicOr(status, 1u);
+          break;
+        }
+        stack[sp] = lfirst ? D.y : D.x;
+        stq[sp] = lfirst ? trr : tl;
+        ++sp;
+        node = lfirst ? D.x : D.y;
+        continue;
+      }
+      if (hl) {
+        node = D.x;
+        continue;
+      }
+      if (hr) {
+        node = D.y;
+        continue;
+      }
+      bool found = false;
+      while (sp > 0) {
+        --sp;
+        if (stq[sp] <= tr.best_t) {
+          node = stack[sp];
+          found = true;
+          break;
+        }
+      }
+      if (!found) break;
+    }
+  }
+  float rg;
+  int32_t id;
+  tr.result(rg, id);
+  const int64_t o = (int64_t)env * a.n_rays + __float_as_int(ds.w);
+  __stcs(a.out_range + o, rg);  // evict-first: keep L2 for the tree
+  __stcs(a.out_tri + o, id);
+}
+
 fgl_status err(int status, const std::string& msg) {
   record_error(status, msg.c_str());
   return (fgl_status)status;
@@ -596,6 +727,30 @@ size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 }  // namespace
 
 namespace fgl {
+cudaError_t launch_lbvh_cast(const fgl_lbvh_s* L, const void* dirs, const float* poses, int n_env,
+                             int n_rays, float min_range, float max_range, float* out_range,
+                             int32_t* out_tri, cudaStream_t s) {
+  unsigned* status = L->status;
+  const int64_t total = (int64_t)n_env * n_rays;
+  if (total == 0) return cudaSuccess;
+  LbvhCast a;
+  a.nodes = (const LbvhNode*)L->nodes;
+  a.tris = (const float4*)L->tris;
+  a.nt = L->nt;
+  a.dirs = (const float4*)dirs;
+  a.poses = poses;
+  a.n_env = n_env;
+  a.n_rays = n_rays;
+  a.min_range = min_range;
+  a.max_range = max_range;
+  a.out_range = out_range;
+  a.out_tri = out_tri;
+  const unsigned grid = (unsigned)((total + 127) / 128);
+  if (min_range > 0.f) k_lbvh_cast<true><<<grid, 128, 0, s>>>(a, status);
+  else k_lbvh_cast<false><<<grid, 128, 0, s>>>(a, status);
+  return cudaGetLastError();
+}
+
 // The wide form as a cast item.
 ItemDesc lbvh_item(const fgl_lbvh_s* L) {
   ItemDesc d{};
