@@ -30,7 +30,7 @@ struct fgl_sensor_s {
   int32_t n_rays = 0, rows = 1, cols = 1, tile_rows = 4, tile_cols = 8;
   std::vector<float> dirs;       // beam order, 3 per ray
   std::vector<float> dev_order;  // tile order, 4 per ray (xyz + beam index bits)
-  bool narrow = false;           // most packets of 32 rays are narrow (see narrow_packets)
+  int packets = kSpreadPackets;  // what most packets of 32 rays are like (see sensor_packets)
   void* d_dirs = nullptr;
 };
 
@@ -177,31 +177,49 @@ fgl_status check_item(const fgl_cast_item& it, int idx) {
   return FGL_OK;
 }
 
-// Whether most packets of 32 consecutive rays (tile order) lie within
+// What most packets of 32 consecutive rays (tile order) are like.  Narrow: within
 // kNarrow of their mean direction, so that a warp's rays meet mostly the same
-// boxes and are cheaper walked together: a spinning sensor's 4 x 8 tiles are
-// (about 0.06 at 16 x 360, 1.3x faster on a cluttered room), a rosette's
-// consecutive rays span its whole field of view (1.3: slower by 7%, and half
-// of the lanes would idle in a sensor of fewer than 16 rays).
+// boxes (a rosette's consecutive rays span its whole field of view, 1.3 rad, and
+// are 7% slower together).  Fair or close: narrow, and the way through the rays,
+// each to the next, is at most kFair or kClose long -- a spinning sensor's 4 x 8
+// tiles at 16 x 360 have 0.08 and 0.87, at 5 x 2048 0.23 and 0.55, at 5 x 360 0.24
+// and 1.06, at 16 x 180 0.23 and 1.6, at 5 x 91 0.33 and 3.4.  A sensor whose
+// packets are less than 7/8 full is spread: their empty lanes idle, while rays for
+// themselves fill up warps (33 rays: 1.2-1.6 times as long in packets).  A large
+// sensor is judged by 32 of its packets.
 constexpr double kNarrow = 0.35;
+constexpr float kFair = 1.75f, kClose = 1.03f;
 
-bool narrow_packets(const std::vector<float>& dirs4, int32_t n) {
-  if (n < 16) return false;
-  int64_t narrow = 0, packets = 0;
-  for (int32_t b = 0; b < n; b += 32, ++packets) {
-    const int32_t e = std::min(n, b + 32);
+int sensor_packets(const std::vector<float>& dirs4, int32_t n) {
+  const int64_t packets = ((int64_t)n + 31) / 32, looks = std::min<int64_t>(packets, 32);
+  if (8 * (int64_t)n < 7 * 32 * packets) return kSpreadPackets;
+  const double narrow_cos = std::cos(kNarrow);
+  int64_t kinds[4] = {};  // packets of each kind or better
+  for (int64_t k = 0; k < looks; ++k) {
+    const int64_t b = 32 * (k * packets / looks), e = std::min<int64_t>(n, b + 32);
     double m[3] = {0, 0, 0};
-    for (int32_t i = b; i < e; ++i)
-      for (int a = 0; a < 3; ++a) m[a] += dirs4[4 * (size_t)i + a];
-    const double len = std::sqrt(m[0] * m[0] + m[1] * m[1] + m[2] * m[2]);
-    double least = len > 0 ? 1.0 : -1.0;  // the smallest cosine to the mean direction
-    for (int32_t i = b; len > 0 && i < e; ++i) {
+    float way = 0.f;
+    for (int64_t i = b; i < e; ++i) {
       const float* d = &dirs4[4 * (size_t)i];
-      least = std::min(least, (d[0] * m[0] + d[1] * m[1] + d[2] * m[2]) / len);
+      for (int a = 0; a < 3; ++a) m[a] += d[a];
+      if (i == b) continue;
+      const float x = d[0] - d[-4], y = d[1] - d[-3], z = d[2] - d[-2];
+      way += std::sqrt(x * x + y * y + z * z);
     }
-    if (least >= std::cos(kNarrow)) ++narrow;
+    const double len = std::sqrt(m[0] * m[0] + m[1] * m[1] + m[2] * m[2]);
+    double least = len > 0 ? len : -1.0;  // the smallest cosine to the mean direction, times len
+    for (int64_t i = b; len > 0 && i < e; ++i) {
+      const float* d = &dirs4[4 * (size_t)i];
+      least = std::min(least, d[0] * m[0] + d[1] * m[1] + d[2] * m[2]);
+    }
+    if (len <= 0 || least < narrow_cos * len) continue;
+    ++kinds[kNarrowPackets];
+    if (way <= kFair) ++kinds[kFairPackets];
+    if (way <= kClose) ++kinds[kClosePackets];
   }
-  return 4 * narrow >= 3 * packets;
+  int kind = kClosePackets;
+  while (kind > kSpreadPackets && 4 * kinds[kind] < 3 * looks) --kind;
+  return kind;
 }
 
 // Items with instances or point output need launches beyond the scene pass.
@@ -287,24 +305,24 @@ bool packet_opts(int W, const Opts& o) {
 // BatchHeader (head = 0) followed by its ItemDesc records; packets are
 // numbered per group.  Returns the byte offset of each group's header.
 // A group walks whole packets when at least half of its packets of 32 rays
-// come from sensors of narrow packets: one launch for all of its items costs
-// less than a second launch and drain for the others, which lose a few
-// percent there.
+// come from items that are faster so (batch_packets): one launch for all of its
+// items costs less than a second launch and drain for the others, which lose a
+// few percent there.
 void build_table(const fgl_cast_item* items, int n, const Opts& o, std::vector<Group>& groups,
                  std::vector<uint8_t>& table, std::vector<size_t>& offsets) {
   groups.clear();
   for (int W : {8, 4}) {
     Group g;
     g.W = W;
-    int64_t narrow = 0, rays = 0;  // packets of narrow sensors less those of the others
+    int64_t together = 0, rays = 0;  // packets of items that gain less those of the others
     for (int i = 0; i < n; ++i) {
       if (items[i].scene->bvh.width != W || items[i].n_env == 0) continue;
       const int64_t packets = (int64_t)items[i].n_env * ((items[i].sensor->n_rays + 31) / 32);
-      narrow += items[i].sensor->narrow ? packets : -packets;
+      together += batch_packets(items[i].sensor->packets, items[i].scene->bvh.n_tris) ? packets : -packets;
       rays += (int64_t)items[i].n_env * items[i].sensor->n_rays;
     }
-    g.packets = narrow >= 0 && packet_opts(W, o);
-    const int P = g.packets && !o.own_packet && small_cast(rays) ? 16 : o.packet;
+    g.packets = together >= 0 && packet_opts(W, o);
+    const int P = g.packets && !o.own_packet ? batch_packet_rays(rays) : o.packet;
     g.packet_rays = P;
     for (int i = 0; i < n; ++i) {
       if (items[i].scene->bvh.width != W || items[i].n_env == 0) continue;
@@ -577,7 +595,7 @@ namespace fgl {
 // Item check + descriptor fill for fgl_cast_batched_static (static_batch.cu):
 // the same rules as check_item/make_desc, with constant messages so that a
 // valid item costs no allocation.  Returns nullptr when the item is valid.
-const char* static_item_desc(const fgl_cast_item& it, ItemDesc* d, int* width, bool* narrow) {
+const char* static_item_desc(const fgl_cast_item& it, ItemDesc* d, int* width, bool* together) {
   if (!it.scene || !it.sensor) return "null scene or sensor in an item";
   if (it.n_env < 0) return "n_env < 0 in an item";
   if (!(std::isfinite(it.max_range) && it.max_range > 0.f))
@@ -592,7 +610,7 @@ const char* static_item_desc(const fgl_cast_item& it, ItemDesc* d, int* width, b
     return "instances and return points need fgl_cast_batched";
   *d = make_desc(it);
   *width = it.scene->bvh.width;
-  *narrow = it.sensor->narrow;
+  *together = batch_packets(it.sensor->packets, it.scene->bvh.n_tris);
   return nullptr;
 }
 
@@ -779,7 +797,7 @@ fgl_status fgl_sensor_create(const float* el, const float* az, int32_t n, int32_
           s->dev_order.push_back(s->dirs[3 * j + 2]);
           s->dev_order.push_back(w);
         }
-  s->narrow = narrow_packets(s->dev_order, n);
+  s->packets = sensor_packets(s->dev_order, n);
   size_t bytes = s->dev_order.size() * sizeof(float);
   cudaError_t ae = cudaMalloc(&s->d_dirs, bytes);
   if (ae != cudaSuccess) {
@@ -827,7 +845,9 @@ fgl_status fgl_cast(fgl_scene scene, fgl_sensor sensor, const float* poses, int3
   if (n_env == 0) return FGL_OK;
   Opts o;
   ItemDesc d = make_desc(it);
-  const bool packets = sensor->narrow && packet_opts(scene->bvh.width, o);
+  const int packets = packet_opts(scene->bvh.width, o)
+                          ? cast_packets(sensor->packets, scene->bvh.n_tris, (int64_t)n_env * sensor->n_rays)
+                          : 0;
   FGL_CUDA(launch_plain(scene->bvh.width, false, packets, false, d, nullptr, o.block, o.sdepth, o.tri_mode,
                         o.postpone, (cudaStream_t)stream));
   return FGL_OK;
@@ -845,8 +865,9 @@ fgl_status fgl_cast_opts(fgl_scene scene, fgl_sensor sensor, const float* poses,
   if (n_env == 0) return FGL_OK;
   ItemDesc d = make_desc(it);
   // the refill threshold has no meaning here
-  const bool packets =
-      sensor->narrow && o.tri_mode == 0 && packets_fit(scene->bvh.width, o.block, o.sdepth);
+  const int packets = o.tri_mode == 0 && packets_fit(scene->bvh.width, o.block, o.sdepth)
+                          ? cast_packets(sensor->packets, scene->bvh.n_tris, (int64_t)n_env * sensor->n_rays)
+                          : 0;
   FGL_CUDA(launch_plain(scene->bvh.width, o.count != 0, packets, false, d, nullptr, o.block, o.sdepth, o.tri_mode,
                         o.postpone, (cudaStream_t)stream));
   return FGL_OK;
@@ -869,12 +890,14 @@ fgl_status fgl_cast_lbvh(fgl_lbvh lbvh, fgl_sensor sensor, const float* poses, i
   // them: 20,000 x 32 of a rosette on 250 k triangles 310 us, 344 over the 8-wide
   // nodes (2 k triangles 49 and 54); 16 rays x 10,000 125 and 154.
   const Opts o;
-  if (!sensor->narrow || !packet_opts(8, o)) {
+  ItemDesc d = lbvh_item(lbvh);
+  const int packets =
+      packet_opts(8, o) ? lbvh_packets(sensor->packets, d.n_tris, (int64_t)n_env * sensor->n_rays) : 0;
+  if (!packets) {
     FGL_CUDA(launch_lbvh_cast(lbvh, sensor->d_dirs, poses, n_env, sensor->n_rays, min_range, max_range, out_range,
                               out_tri, (cudaStream_t)stream));
     return FGL_OK;
   }
-  ItemDesc d = lbvh_item(lbvh);
   d.dirs = sensor->d_dirs;
   d.poses = poses;
   d.out_range = out_range;
@@ -883,7 +906,7 @@ fgl_status fgl_cast_lbvh(fgl_lbvh lbvh, fgl_sensor sensor, const float* poses, i
   d.n_rays = sensor->n_rays;
   d.max_range = max_range;
   d.min_range = min_range;
-  FGL_CUDA(launch_plain(8, false, true, min_range > 0.f, d, lbvh_status(lbvh), o.block, o.sdepth, o.tri_mode,
+  FGL_CUDA(launch_plain(8, false, packets, min_range > 0.f, d, lbvh_status(lbvh), o.block, o.sdepth, o.tri_mode,
                         o.postpone, (cudaStream_t)stream));
   return FGL_OK;
 }

@@ -800,23 +800,23 @@ static cudaError_t allow_smem(void* fn, size_t smem) {
   return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
-cudaError_t launch_plain(int W, bool count, bool packets, bool tmin, const ItemDesc& it, unsigned* status, int block,
+cudaError_t launch_plain(int W, bool count, int packet_rays, bool tmin, const ItemDesc& it, unsigned* status, int block,
                          int sdepth, int tri_mode, int postpone_pct, cudaStream_t s) {
   const int64_t total = (int64_t)it.n_env * it.n_rays;
   if (total == 0) return cudaSuccess;
-  if (tmin && (W != 8 || count || !packets)) return cudaErrorInvalidValue;  // no such form
+  if (tmin && (W != 8 || count || !packet_rays)) return cudaErrorInvalidValue;  // no such form
   ItemDesc arg = it;
-  int rays = small_cast(total) ? 16 : 32;  // a packet
-  arg.pk_per_env = (it.n_rays + rays - 1) / rays;
-  const int64_t threads = packets ? (int64_t)it.n_env * arg.pk_per_env * 32 : total;
+  int rays = packet_rays;
+  if (rays) arg.pk_per_env = (it.n_rays + rays - 1) / rays;
+  const int64_t threads = rays ? (int64_t)it.n_env * arg.pk_per_env * 32 : total;
   const int64_t grid = (threads + block - 1) / block;
-  const size_t smem = packets ? packets_smem_bytes(W, block, sdepth) : stack_smem_bytes(W, block, sdepth);
-  void* fn = packets ? pick_plain_packets(W, count, tmin) : pick_plain(W, count);
+  const size_t smem = rays ? packets_smem_bytes(W, block, sdepth) : stack_smem_bytes(W, block, sdepth);
+  void* fn = rays ? pick_plain_packets(W, count, tmin) : pick_plain(W, count);
   const cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
   void* plain_args[] = {&arg, &sdepth, &tri_mode, &postpone_pct, &status};
   void* packet_args[] = {&arg, &sdepth, &status, &rays};
-  return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(block), packets ? packet_args : plain_args, smem, s);
+  return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(block), rays ? packet_args : plain_args, smem, s);
 }
 
 int persistent_blocks_per_sm(int W, bool count, bool tmin, bool packets, int block, int sdepth) {

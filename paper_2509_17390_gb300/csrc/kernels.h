@@ -12,21 +12,57 @@ namespace fgl {
 // shared part of the traversal stacks.
 size_t stack_smem_bytes(int W, int block, int sdepth);
 
-// One thread per ray of one item (grid = ceil(n_env * n_rays / block)).
-// tri_mode 0: warp-pooled leaf tests; 1: lane-serial with postponing.
-// packets: one packet of 32 rays of an environment a warp, walked together
-// before the per-ray traversal (needs tri_mode 0; see packets_fit).
-// A cast or batch of so few rays that packets of 16 come to at most two for each
-// of the 28 warps an SM holds leaves the chip waiting for its slowest packets:
-// half of the lanes idle there, but a packet ends sooner (1 M triangles, 57,600
-// rays 42 -> 35 us, 5,760 53 -> 44, 131,072 51 -> 44; 184,320 would take 82
-// instead of 75).
+// How a cast walks the tree: packets of this many consecutive rays of an
+// environment a warp, together (16 or 32), or each ray for itself (0).  By what the
+// sensor's packets are like (see sensor_packets), the scene's triangles and the
+// rays; the figures are shares of the time ray by ray, over sensors of 5 to 128
+// beams and 91 to 2048 columns and rooms of 108 to 1 M triangles:
+//   sensor   close packets 0.6-1.05 at any number of rays; fair ones 0.9-1.05 from 220 k
+//            rays on, up to 1.15 at 100 k; narrow ones 1.01-1.15
+//   tris     where a walk is short there is little to share: rooms of up to
+//            1,084 triangles 0.75-1.35 up to 220 k rays, from 800 k on 0.65-1.0
+//   16 rays  half of the lanes idle, but a packet ends sooner, which counts when
+//            packets of 16 come to at most two for each of the 28 warps an SM
+//            holds (1 M triangles, 57,600 rays 42 -> 35 us, 131,072 51 -> 44;
+//            184,320 would take 82 instead of 75).  Fair and narrow ones gain up
+//            to half as many rays, on 9,868 triangles and more (0.66-1.05)
 constexpr int64_t kSmallCastRays = 16 * 2 * 28 * 152;
 inline bool small_cast(int64_t rays) { return rays <= kSmallCastRays; }
 
+enum SensorPackets { kSpreadPackets = 0, kNarrowPackets = 1, kFairPackets = 2, kClosePackets = 3 };
+
+inline int cast_packets(int sensor, int64_t n_tris, int64_t rays) {
+  if (sensor == kClosePackets && n_tris >= 2048) return small_cast(rays) ? 16 : 32;
+  if (sensor == kSpreadPackets) return 0;
+  if (2 * rays <= kSmallCastRays) return n_tris >= 8192 ? 16 : 0;
+  return sensor >= kFairPackets && rays >= (n_tris < 2048 ? 1 << 19 : 1 << 18) ? 32 : 0;
+}
+
+// The same for a batch, whose rays go through one launch: its other kernel hands
+// fresh rays to idle lanes, which a walk in packets has to make up for.  Scenes of
+// 9,868 triangles 0.85-1.13 of the time without packets, 30,012 and more 0.65-1.0,
+// whether close or narrow.  Packets of 16 up to one a warp slot (65,536 rays
+// 0.8-0.9, packets of 32 0.85-1.0; 130,000 rays 0.9-1.1 and 0.8-0.95).
+inline bool batch_packets(int sensor, int64_t n_tris) { return sensor != kSpreadPackets && n_tris >= 16384; }
+inline int batch_packet_rays(int64_t rays) { return 2 * rays <= kSmallCastRays ? 16 : 32; }
+
+// The same over a GPU-built LBVH, whose other kernel walks the binary tree ray by
+// ray: close and fair packets 0.4-1.0 of its time (tiny scenes up to 1.1 from 2 M
+// rays on), narrow ones 0.5-1.0 up to 220 k rays, 0.9-1.3 from 800 k on.
+inline int lbvh_packets(int sensor, int64_t n_tris, int64_t rays) {
+  if (sensor == kSpreadPackets) return 0;
+  if (sensor == kNarrowPackets) return 2 * rays <= kSmallCastRays ? 16 : rays <= (1 << 18) ? 32 : 0;
+  if (n_tris < 2048 && rays > (1 << 20)) return 0;
+  return small_cast(rays) ? 16 : 32;
+}
+
+// One launch over one item: a thread per ray (packet_rays 0) or a warp per packet
+// of packet_rays rays, walked together before the per-ray traversal (needs
+// tri_mode 0; see packets_fit).
+// tri_mode 0: warp-pooled leaf tests; 1: lane-serial with postponing.
 // tmin honours it.min_range (8-wide packets, not counted); status: the word that
 // takes traversal errors (null: the shared one).
-cudaError_t launch_plain(int W, bool count, bool packets, bool tmin, const ItemDesc& it, unsigned* status, int block,
+cudaError_t launch_plain(int W, bool count, int packet_rays, bool tmin, const ItemDesc& it, unsigned* status, int block,
                          int sdepth, int tri_mode, int postpone_pct, cudaStream_t s);
 
 // Whether a block of this shape has room for the packet lists beside its

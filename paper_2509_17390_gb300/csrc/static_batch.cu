@@ -28,7 +28,7 @@
 namespace fgl {
 // Allocation-free item check + descriptor fill, and launch-option defaults and
 // checks (api.cu); both return a constant message, or nullptr when valid.
-const char* static_item_desc(const fgl_cast_item& it, ItemDesc* d, int* width, bool* narrow);
+const char* static_item_desc(const fgl_cast_item& it, ItemDesc* d, int* width, bool* together);
 const char* launch_opts(const fgl_batch_opts* o, int* packet, int* block, int* sdepth, int* bpsm,
                         int* graph, int* refill, int* postpone, int* count, int* tri_mode);
 }  // namespace fgl
@@ -118,9 +118,9 @@ extern "C" fgl_status fgl_cast_batched_static(const fgl_cast_item* items, int32_
   // into the image
   ItemDesc descs[kStaticMaxItems];
   int widths[kStaticMaxItems];
-  bool narrow[kStaticMaxItems];
+  bool gains[kStaticMaxItems];
   for (int i = 0; i < n_items; ++i) {
-    const char* msg = static_item_desc(items[i], &descs[i], &widths[i], &narrow[i]);
+    const char* msg = static_item_desc(items[i], &descs[i], &widths[i], &gains[i]);
     if (msg) return err(FGL_ERR_INVALID, msg);
   }
   StaticImage img;
@@ -131,7 +131,7 @@ extern "C" fgl_status fgl_cast_batched_static(const fgl_cast_item* items, int32_
   int n_groups = 0;
   size_t used = 0;
   for (int W : {8, 4}) {
-    int64_t together = 0;  // packets of narrow sensors less those of the others, as for fgl_cast_batched
+    int64_t together = 0;  // packets of items that gain less those of the others, as for fgl_cast_batched
     BatchHeader h;
     std::memset(&h, 0, sizeof(h));
     const size_t hdr_off = used;
@@ -142,11 +142,11 @@ extern "C" fgl_status fgl_cast_batched_static(const fgl_cast_item* items, int32_
     for (int i = 0; i < n_items; ++i) {
       if (widths[i] != W) continue;
       const int64_t warps = (int64_t)descs[i].n_env * ((descs[i].n_rays + 31) / 32);
-      together += narrow[i] ? warps : -warps;
+      together += gains[i] ? warps : -warps;
       rays += (int64_t)descs[i].n_env * descs[i].n_rays;
     }
     const bool walk = together >= 0 && tri_mode == 0 && refill == 32 && packets_fit(W, block, sdepth);
-    const int per = walk && !(opts && opts->packet_rays) && small_cast(rays) ? 16 : packet;
+    const int per = walk && !(opts && opts->packet_rays) ? batch_packet_rays(rays) : packet;
     for (int i = 0; i < n_items; ++i) {
       ItemDesc d = descs[i];
       if (widths[i] != W || d.n_env == 0) continue;
