@@ -20,9 +20,12 @@ using namespace fgl;
 
 struct fgl_scene_s {
   HostBVH bvh;
-  void* d_nodes = nullptr;       // the node records, then the top cut
-  void* d_tris = nullptr;        // the triangle records, then the cut's
-  const void* d_top = nullptr;   // the cut within d_nodes; null: none
+  TopBox cut[kTopBoxes];         // the top cut, where has_cut, and its triangle records
+  std::vector<float> cut_tris;
+  bool has_cut = false;
+  void* d_nodes = nullptr;       // one buffer: the node records,
+  void* d_tris = nullptr;        // the triangle records, those of the cut
+  const void* d_top = nullptr;   // and the cut (null: none)
   int device = -1;
 };
 
@@ -645,6 +648,7 @@ fgl_status fgl_scene_build(const float* verts, int64_t nv, const int32_t* tris, 
   try {
     if (build_bvh(verts, nv, tris, nt, width, bins, threads, &s->bvh, &err))
       return fail(FGL_ERR_INVALID, err);
+    s->has_cut = top_cut(s->bvh, s->cut, &s->cut_tris);
   } catch (const std::bad_alloc&) {
     return fail(FGL_ERR_OOM, "host allocation failed during the BVH build");
   }
@@ -661,36 +665,40 @@ fgl_status fgl_scene_build(const float* verts, int64_t nv, const int32_t* tris, 
 fgl_status fgl_scene_upload(fgl_scene s) {
   if (!s) return fail(FGL_ERR_INVALID, "null scene");
   if (s->d_nodes) return FGL_OK;
-  size_t nb = s->bvh.nodes.size(), tb = s->bvh.tris.size() * sizeof(float);
-  TopBox cut[kTopBoxes];
-  std::vector<float> cut_tris;
-  const bool has_cut = top_cut(s->bvh, cut, &cut_tris);
-  const size_t cut_tb = cut_tris.size() * sizeof(float);
-  cudaError_t ae = cudaMalloc(&s->d_nodes, nb + sizeof(cut));  // nb is a multiple of 16
+  // one allocation, and one copy of a small scene (108 triangles: 24 us with two
+  // of each and no cut, 40 with the cut's own copies)
+  constexpr size_t kStaged = 128 * 1024;
+  const struct {
+    const void* src;
+    size_t bytes;
+  } part[] = {{s->bvh.nodes.data(), s->bvh.nodes.size()},
+              {s->bvh.tris.data(), s->bvh.tris.size() * sizeof(float)},
+              {s->cut_tris.data(), s->cut_tris.size() * sizeof(float)},
+              {s->cut, s->has_cut ? sizeof(s->cut) : 0}};
+  size_t at[5] = {};
+  for (int k = 0; k < 4; ++k) at[k + 1] = at[k] + part[k].bytes + (k == 0 ? -part[k].bytes % 256 : 0);
+  void* buf = nullptr;
+  const cudaError_t ae = cudaMalloc(&buf, at[4]);
   if (ae != cudaSuccess) {
-    s->d_nodes = nullptr;
     cudaGetLastError();
-    if (ae == cudaErrorMemoryAllocation) return fail(FGL_ERR_OOM, "cannot allocate device BVH nodes");
-    return cuda_fail(ae, "cudaMalloc(BVH nodes)");
+    if (ae == cudaErrorMemoryAllocation) return fail(FGL_ERR_OOM, "cannot allocate the device BVH");
+    return cuda_fail(ae, "cudaMalloc(BVH)");
   }
-  if (cudaMalloc(&s->d_tris, tb + cut_tb) != cudaSuccess) {
-    cudaFree(s->d_nodes);
-    s->d_nodes = s->d_tris = nullptr;
-    cudaGetLastError();
-    return fail(FGL_ERR_OOM, "cannot allocate device triangles");
+  std::unique_ptr<char[]> stage(at[4] <= kStaged ? new (std::nothrow) char[at[4]]() : nullptr);
+  cudaError_t e = cudaSuccess;
+  for (int k = 0; k < 4; ++k) {
+    if (!part[k].bytes) continue;
+    if (stage) std::memcpy(stage.get() + at[k], part[k].src, part[k].bytes);
+    else if (e == cudaSuccess) e = cudaMemcpy((char*)buf + at[k], part[k].src, part[k].bytes, cudaMemcpyHostToDevice);
   }
-  cudaError_t e = cudaMemcpy(s->d_nodes, s->bvh.nodes.data(), nb, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(s->d_tris, s->bvh.tris.data(), tb, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess && has_cut) e = cudaMemcpy((char*)s->d_nodes + nb, cut, sizeof(cut), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess && cut_tb)
-    e = cudaMemcpy((char*)s->d_tris + tb, cut_tris.data(), cut_tb, cudaMemcpyHostToDevice);
+  if (stage) e = cudaMemcpy(buf, stage.get(), at[4], cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
-    cudaFree(s->d_nodes);
-    cudaFree(s->d_tris);
-    s->d_nodes = s->d_tris = nullptr;
+    cudaFree(buf);
     return cuda_fail(e, "scene upload");
   }
-  s->d_top = has_cut ? (const char*)s->d_nodes + nb : nullptr;
+  s->d_nodes = buf;
+  s->d_tris = (char*)buf + at[1];
+  s->d_top = s->has_cut ? (const char*)buf + at[3] : nullptr;
   cudaGetDevice(&s->device);
   return FGL_OK;
 }
@@ -700,7 +708,6 @@ fgl_status fgl_scene_evict(fgl_scene s) {
   if (s->d_nodes) {
     cudaDeviceSynchronize();
     cudaFree(s->d_nodes);
-    cudaFree(s->d_tris);
     s->d_nodes = s->d_tris = nullptr;
     s->d_top = nullptr;
   }
