@@ -270,16 +270,32 @@ __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
 // end of the row: E P^j then stays below 2^kRowFall, and where E underflows
 // (below 2^-126) the row's largest value is below 2^-45.  P^2 has to stay
 // finite too (|g h / 2| <= kRowSlope), so that a row far from the Gaussian adds
-// 0 and not 0 times infinity.  A Gaussian outside these limits (steep) is
-// evaluated voxel by voxel.
+// 0 and not 0 times infinity; a Gaussian that would widen the band below too far
+// (kMaxSpread) or whose opacity is not finite is left out as well.  A Gaussian
+// outside these limits (steep) is evaluated voxel by voxel.
 constexpr float kRowFall = 20.f, kRowSlope = 60.f;
 
-// Voxels whose density falls this close to theta (relative) are summed again
-// voxel by voxel in candidate order, so that the masks never hang on the
-// rounding of the factored form or of the warps' partial sums: those differ
-// from those sums by a few 1e-6 (a term's exponent by a few units of 2^-24 of
-// its partial sums).
-constexpr float kThetaBand = 1e-4f;
+// Voxels whose density may lie on either side of theta, depending on the rounding
+// of the factored form and of the warps' partial sums, are summed again voxel by
+// voxel in candidate order, so that the masks are those of that sum to the last
+// bit.  Steep Gaussians' terms are that sum's, bit for bit.  A factored term's
+// exponent differs from that sum's by at most u = 2^-24 times
+//   11 X G + 6 Q + 150,   X = |dx|, G = |M01| |dy| + |M02| |dz| + 2 |M00| |dx|,
+//                         Q = |M11| dy^2 + |M12 dy dz| + |M22| dz^2,
+// each at its largest over the tile: roundings of dx, xm (1 and 2.5 u X, each times
+// the slope G), of the x coefficient (2 and 3 u G, times X), of the slope's up to 7
+// half voxels (28 u G h / 2 <= 2 u X G), of the y/z part (3 u Q in each form) and of
+// the sums (exponents to -64 and the middle's 420 beyond it at most; smaller terms
+// are below the slack).  The exponentials and products add 6e-6.  Sums of n
+// positive terms in two orders differ by at most 1.5 n u.  So the band is
+//   kBand + 1.5 n u + max over the tile's factored Gaussians of u (8 X G + 4.5 Q)
+// relative, and 2^-44 alpha^2 a candidate absolute for rows whose middle flushes.
+// On 60 k to 90 k Gaussians of 1 to 20 cm at 2.5 to 5 cm voxels the band is about
+// 1e-3 (one tile in 12 to 50 has a voxel in it, which no time shows) and kMaxSpread
+// makes up to 0.4% of the factored Gaussians steep; 5e-4 makes 1-4% (1.829 -> 1.836
+// ms in all), 3e-4 1.856.
+constexpr float kUnit = 5.9604645e-8f;  // u
+constexpr float kBand = 2e-5f, kMaxSpread = 1e-3f;
 constexpr int kCloseAtOnce = 8;
 
 // One staged candidate.  bx = M01 dy + M02 dz is the x coefficient and
@@ -302,7 +318,7 @@ template <int B, int S, int K>
 __global__ void __launch_bounds__(32 * S)
     k_density(const GaussParams* __restrict__ params, const uint32_t* __restrict__ cand,
               const uint32_t* __restrict__ begin, const uint32_t* __restrict__ end, GridArgs g, float theta,
-              float* __restrict__ out) {
+              float max_spread, float* __restrict__ out) {
   using C = DensityCfg<B>;
   constexpr int NT = 32 * S;
   namespace cg = cooperative_groups;
@@ -331,8 +347,7 @@ __global__ void __launch_bounds__(32 * S)
   const double cz = (double)g.o[2] + (double)(tz * B) * (double)g.h;
   const double mid = (double)(B / 2) * (double)g.h;
   const float hh = 0.5f * g.h, end_d = (float)(B - 1) * hh;
-  const float oy = ((float)y + 0.5f) * g.h;
-  const float oz[2] = {((float)z + 0.5f) * g.h, ((float)(z + B / 2) + 0.5f) * g.h};
+  const float jy = (float)y + 0.5f, jz[2] = {(float)z + 0.5f, (float)(z + B / 2) + 0.5f};
   uint64_t acc[2][B / 2];  // voxel pairs mirrored about the row's middle, innermost first
 #pragma unroll
   for (int r = 0; r < 2; ++r)
@@ -342,17 +357,26 @@ __global__ void __launch_bounds__(32 * S)
   // candidate numbers one batch earlier
   GaussParams P = {};
   uint32_t next = 0;
+  float spread = 0.f, weight = 0.f;  // over the lane's factored candidates: the largest u (8 X G + 4.5 Q) and alpha^2
   if (first + lane < b1) P = params[cand[first + lane]];
   if (first + stride + lane < b1) next = cand[first + stride + lane];
   for (uint32_t c0 = first; c0 < b1; c0 += stride) {
     __syncwarp();  // the batch before this one is summed
     const bool valid = c0 + lane < b1;
     const float dX = (float)(cx - (double)P.a.x), dY = (float)(cy - (double)P.a.y), dZ = (float)(cz - (double)P.a.z);
-    // |g h / 2| over the tile's rows, from above: P^2 stays finite
-    const float most = 2.f * end_d + g.h;  // the tile's edge
-    const float slope = hh * (fabsf(P.b.w) * (fabsf(dY) + most) + fabsf(P.c.x) * (fabsf(dZ) + most) +
-                              2.f * fabsf(P.b.x) * (fabsf(dX) + most));
-    const bool fast = valid && fabsf(P.b.x) * (end_d * end_d) <= kRowFall && slope <= kRowSlope;
+    // the offsets' magnitudes over the tile's voxels, from above
+    const float edge = (float)B * g.h;
+    const float X = fmaxf(fabsf(dX), fabsf(dX + edge)), Y = fmaxf(fabsf(dY), fabsf(dY + edge)),
+                Z = fmaxf(fabsf(dZ), fabsf(dZ + edge));
+    const float G = fabsf(P.b.w) * Y + fabsf(P.c.x) * Z + 2.f * fabsf(P.b.x) * X, slope = hh * G;  // |g h / 2| at most: P^2 stays finite
+    const float Q = fabsf(P.b.y) * (Y * Y) + fabsf(P.c.y) * (Y * Z) + fabsf(P.b.z) * (Z * Z);
+    const float d_spread = kUnit * (8.f * (X * G) + 4.5f * Q);
+    const bool fast = valid && fabsf(P.b.x) * (end_d * end_d) <= kRowFall && slope <= kRowSlope &&
+                      d_spread <= max_spread && P.a.w < INFINITY;
+    if (fast) {
+      spread = fmaxf(spread, d_spread);
+      weight = fmaxf(weight, P.a.w);
+    }
     // the factored ones first, steep ones from the end
     const unsigned fm = __ballot_sync(FULL, fast), sm = __ballot_sync(FULL, valid && !fast);
     const unsigned below = (1u << lane) - 1u;
@@ -378,12 +402,12 @@ __global__ void __launch_bounds__(32 * S)
     for (int i = sub; i < nf; i += C::SUB) {
       const float4 at = st[i].at, m = st[i].m, n = st[i].n;
       const float4 w0 = st[i].c[0], w1 = st[i].c[1];
-      const float dy = at.x + oy;
+      const float dy = __fmaf_rn(jy, g.h, at.x);
       const float ay = (m.x * dy) * dy, by = fmaf(m.w, dy, at.w);
       uint64_t t2[2], PP[2];
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
-        const float dz = at.y + oz[r];
+        const float dz = __fmaf_rn(jz[r], g.h, at.y);
         const float a = fmaf(n.x, dz, by);
         const float qm = fmaf(a, at.z, fmaf(fmaf(m.z, dy, m.y * dz), dz, ay));
         const float gh = fmaf(a, hh, n.y);
@@ -405,18 +429,19 @@ __global__ void __launch_bounds__(32 * S)
 #pragma unroll 1
     for (int i = 31 - sub; i > 31 - ns; i -= C::SUB) {
       const float4 at = st[i].at, m = st[i].m, n = st[i].n;
-      const float dy = at.x + oy;
-      const float ay = (m.x * dy) * dy, by = m.w * dy;
+      const float dy = __fmaf_rn(jy, g.h, at.x);
       const uint64_t M002 = dev::pack2f(n.w, n.w), dX2 = dev::pack2f(at.z, at.z), a22 = dev::pack2f(n.z, n.z);
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
-        const float dz = at.y + oz[r];
-        const float bx = fmaf(n.x, dz, by), syz = fmaf(fmaf(m.z, dy, m.y * dz), dz, ay);
+        // the operations of the voxel-by-voxel sum below, one by one
+        const float dz = __fmaf_rn(jz[r], g.h, at.y);
+        const float syz = __fmaf_rn(__fmaf_rn(m.x, dy, __fmul_rn(m.z, dz)), dy, __fmul_rn(__fmul_rn(m.y, dz), dz));
+        const float bx = __fmaf_rn(m.w, dy, __fmul_rn(n.x, dz));
         const uint64_t bx2 = dev::pack2f(bx, bx), syz2 = dev::pack2f(syz, syz);
 #pragma unroll
         for (int p = 0; p < B / 2; ++p) {
           const uint64_t dx2 =
-              add2(dX2, dev::pack2f(((float)(B / 2 - 1 - p) + 0.5f) * g.h, ((float)(B / 2 + p) + 0.5f) * g.h));
+              add2(dX2, dev::pack2f(__fmul_rn((float)(B / 2 - 1 - p) + 0.5f, g.h), __fmul_rn((float)(B / 2 + p) + 0.5f, g.h)));
           float q0, q1;
           dev::unpack2f(dev::ffma2(dev::ffma2(M002, dx2, bx2), dx2, syz2), q0, q1);  // <= 0
           acc[r][p] = dev::ffma2(a22, dev::pack2f(dev::ex2_approx(q0), dev::ex2_approx(q1)), acc[r][p]);
@@ -424,6 +449,11 @@ __global__ void __launch_bounds__(32 * S)
       }
     }
   }
+  // the warps' largest spread and weight (non-negative floats order as integers)
+  __shared__ float2 s_band[K * S];
+  spread = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(spread)));
+  weight = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(weight)));
+  if (lane == 0) s_band[warp] = make_float2(spread, weight);
   float d[2][B];  // the rows' densities, complete in warp 0's lanes of sub 0
 #pragma unroll
   for (int r = 0; r < 2; ++r)
@@ -472,6 +502,7 @@ __global__ void __launch_bounds__(32 * S)
         for (int k = 1; k < K; ++k) sum += part[k];
         s_part[v] = sum;  // read by nobody else
       }
+      for (int t = S + threadIdx.x; t < K * S; t += NT) s_band[t] = *cl.map_shared_rank(s_band + t % S, t / S);
     }
     cl.sync();  // and the others' memory stays until it is read
     if (rank > 0) return;
@@ -484,7 +515,7 @@ __global__ void __launch_bounds__(32 * S)
   }
   const int gx = tx * B, gy = ty * B + y;
   const bool owner = warp == 0 && sub == 0 && gy < g.dims[1];
-  // the tile's densities; the voxels close to theta are then listed and summed
+  // the tile's densities; the voxels in theta's band are then listed and summed
   // again, kCloseAtOnce at a time: their terms a candidate a thread, each
   // voxel's sum a lane's, in candidate order
   __shared__ uint16_t s_close[C::ROWS * B];
@@ -492,6 +523,14 @@ __global__ void __launch_bounds__(32 * S)
   if (threadIdx.x == 0) s_n_close = 0;
   __syncthreads();
   if (owner) {
+    float band = 0.f, slack = 0.f;
+    for (int t = 0; t < (split ? K * S : S); ++t) {
+      band = fmaxf(band, s_band[t].x);
+      slack = fmaxf(slack, s_band[t].y);
+    }
+    const float n = (float)(b1 - b0);
+    band += kBand + 1.5f * kUnit * n;
+    slack = n * (slack * 0x1p-44f + 0x1p-148f);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const int gz = tz * B + z + r * (B / 2);
@@ -501,7 +540,8 @@ __global__ void __launch_bounds__(32 * S)
       for (int i = 0; i < B; ++i) {
         if (gx + i >= g.dims[0]) break;
         dst[gx + i] = d[r][i];
-        if (b1 > b0 && fabsf(d[r][i] - theta) <= kThetaBand * (fabsf(d[r][i]) + fabsf(theta)))
+        // theta <= 0: a density above it is one in any order
+        if (theta > 0.f && fabsf(d[r][i] - theta) <= band * fmaxf(d[r][i], theta) + slack)
           s_close[atomicAdd(&s_n_close, 1)] = (uint16_t)(((z + r * (B / 2)) * B + y) * B + i);
       }
     }
@@ -551,7 +591,8 @@ __global__ void __launch_bounds__(32 * S)
 
 template <int B, int S, int K>
 cudaError_t launch_density(int64_t n_tiles, const GaussParams* params, const uint32_t* cand, const uint32_t* begin,
-                           const uint32_t* end, const GridArgs& g, float theta, float* out, cudaStream_t s) {
+                           const uint32_t* end, const GridArgs& g, float theta, float max_spread, float* out,
+                           cudaStream_t s) {
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeClusterDimension;
   at.val.clusterDim.x = K;
@@ -562,7 +603,7 @@ cudaError_t launch_density(int64_t n_tiles, const GaussParams* params, const uin
   cfg.stream = s;
   cfg.attrs = &at;
   cfg.numAttrs = K > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k_density<B, S, K>, params, cand, begin, end, g, theta, out);
+  return cudaLaunchKernelEx(&cfg, k_density<B, S, K>, params, cand, begin, end, g, theta, max_spread, out);
 }
 
 // eqs. V_occ, Int, Surf: a warp 32 voxels of a row, a block eight rows of a
@@ -773,12 +814,15 @@ extern "C" fgl_status fgl_gaussian_density(const fgl_gaussians* gs, const fgl_gr
     // eight).  Tiles of 4^3 voxels have fewer candidates each: one block of one
     // warp where there are many (25,000 tiles: 1.60 ms; two blocks 2.33).
     const GaussParams* params = (const GaussParams*)S.params;
+    // where theta is as small as what flushed rows leave out (or 0: any density
+    // counts), every Gaussian is summed voxel by voxel
+    const float max_spread = theta >= 0.f && theta < 0x1p-30f ? -1.f : kMaxSpread;
     const bool few = n_tiles < 152 * 16;
-    if (B == 8 && few) DCUDA((launch_density<8, 8, 4>(n_tiles, params, v0, begin, end, g, theta, out_density, s)));
-    else if (B == 8 && n_tiles < ((int64_t)1 << 30)) DCUDA((launch_density<8, 4, 2>(n_tiles, params, v0, begin, end, g, theta, out_density, s)));
-    else if (B == 8) DCUDA((launch_density<8, 4, 1>(n_tiles, params, v0, begin, end, g, theta, out_density, s)));
-    else if (few) DCUDA((launch_density<4, 4, 4>(n_tiles, params, v0, begin, end, g, theta, out_density, s)));
-    else DCUDA((launch_density<4, 1, 1>(n_tiles, params, v0, begin, end, g, theta, out_density, s)));
+    if (B == 8 && few) DCUDA((launch_density<8, 8, 4>(n_tiles, params, v0, begin, end, g, theta, max_spread, out_density, s)));
+    else if (B == 8 && n_tiles < ((int64_t)1 << 30)) DCUDA((launch_density<8, 4, 2>(n_tiles, params, v0, begin, end, g, theta, max_spread, out_density, s)));
+    else if (B == 8) DCUDA((launch_density<8, 4, 1>(n_tiles, params, v0, begin, end, g, theta, max_spread, out_density, s)));
+    else if (few) DCUDA((launch_density<4, 4, 4>(n_tiles, params, v0, begin, end, g, theta, max_spread, out_density, s)));
+    else DCUDA((launch_density<4, 1, 1>(n_tiles, params, v0, begin, end, g, theta, max_spread, out_density, s)));
     ++launches;
     DCUDA(cudaGetLastError());
     if (timing) DCUDA(cudaEventRecord(S.ev[2], s));
