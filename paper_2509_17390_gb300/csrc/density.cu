@@ -240,9 +240,9 @@ __global__ void k_tile_bounds(const uint32_t* __restrict__ keys, int64_t n, int6
 // density: one block per tile of B^3 voxels.  Each warp of the block sums
 // every S-th batch of 32 candidates over the whole tile (two x-rows a lane, so
 // that a staged candidate is read once for 64 rows); the warps' sums are added
-// in warp order.  A tile of more than 2 x 32 S candidates is shared by the K
-// blocks of a cluster, whose sums the first adds in block order (the others of
-// a smaller tile leave at once).  Bound by instruction issue and the FMA pipe about equally
+// in warp order.  In a grid of few tiles, one of more than 2 x 32 S candidates is
+// shared by the K blocks of a cluster, whose sums the first adds in block order
+// (the others of a smaller tile leave at once).  Bound by instruction issue and the FMA pipe about equally
 // (36 warp instructions for a candidate and 32 rows, of which 3 exponentials;
 // one exponential a voxel took 40, and 8 of them held the MUFU pipe longest).
 // 720 k Gaussians, 10,304 tiles of 2.5 cm voxels: 2.22 -> 1.47 ms; 85 k
@@ -336,6 +336,14 @@ __global__ void __launch_bounds__(32 * S)
   // the tile's batches go round the warps of one block or of the whole cluster
   const bool split = K > 1 && b1 - b0 > 2 * NT;
   if (K > 1 && !split && rank > 0) return;  // all of the cluster's blocks agree
+  if (K == 1 && b0 == b1) {  // nobody's tile: most of a sparse grid's
+    for (int v = threadIdx.x; v < C::ROWS * B; v += NT) {
+      const int x = tx * B + v % B, vy = ty * B + v / B % B, vz = tz * B + v / (B * B);
+      if (x < g.dims[0] && vy < g.dims[1] && vz < g.dims[2])
+        out[((int64_t)vz * g.dims[1] + vy) * g.dims[0] + x] = 0.f;
+    }
+    return;
+  }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t first = b0 + 32 * (split ? rank * S + warp : warp), stride = split ? 32 * S * K : 32 * S;
   const int slot = lane % C::LANES, sub = lane / C::LANES, y = slot % B, z = slot / B;  // rows (y, z), (y, z + B / 2)
@@ -805,21 +813,28 @@ extern "C" fgl_status fgl_gaussian_density(const fgl_gaussians* gs, const fgl_gr
     ++launches;
     DCUDA(cudaGetLastError());
     if (timing) DCUDA(cudaEventRecord(S.ev[1], s));
-    // Warps a tile: four of 32 candidates each even out tiles of unequal counts
-    // (2.25 ms for the pass at 10,304 tiles, 2.53 with two, 2.99 with one), in
-    // two blocks for a tile of many (the call 1.92 -> 1.87 ms; four blocks 1.97,
-    // launching them costs more); a grid of fewer than 16 tiles an SM takes
-    // eight warps in four blocks, or its heaviest tiles would run on alone (630
-    // tiles: the call 0.54 ms in one block, 0.49 in two, 0.475 in four or
-    // eight).  Tiles of 4^3 voxels have fewer candidates each: one block of one
-    // warp where there are many (25,000 tiles: 1.60 ms; two blocks 2.33).
+    // Warps a tile, by the mean of its candidates (wall time of the call, us):
+    //   candidates a tile            0.1    5   16   53  211  729 1885    5, half of them within 10 cm
+    //   two warps                    816  393  457  643 1547  541         776
+    //   four                         917  553  581  727 1473  522 1828    648
+    //   four in each of two blocks,
+    //   a cluster                   1275  895  919 1182 2494  566 1877    852
+    //   (two warps that share every candidate, one exponential a voxel:
+    //                               1155  411  464  827 2216  782 2940    838)
+    // over 262,144 tiles with 2,000 Gaussians, 62,500 with 20 k to 800 k, 6,500 and
+    // 10,304 dense ones: two warps for a sparse grid, four for the others.  A grid of
+    // fewer than 16 tiles an SM takes eight warps in four blocks, or its heaviest
+    // tiles would run on alone (630 tiles: the call 0.54 ms in one block, 0.49 in two,
+    // 0.475 in four or eight).  Tiles of 4^3 voxels have fewer candidates each: one
+    // block of one warp where there are many (25,000 tiles: 1.60 ms; two blocks 2.33).
     const GaussParams* params = (const GaussParams*)S.params;
     // where theta is as small as what flushed rows leave out (or 0: any density
     // counts), every Gaussian is summed voxel by voxel
     const float max_spread = theta >= 0.f && theta < 0x1p-30f ? -1.f : kMaxSpread;
     const bool few = n_tiles < 152 * 16;
+    const bool sparse = (int64_t)n_pairs < 32 * n_tiles;
     if (B == 8 && few) DCUDA((launch_density<8, 8, 4>(n_tiles, params, v0, begin, end, g, theta, max_spread, out_density, s)));
-    else if (B == 8 && n_tiles < ((int64_t)1 << 30)) DCUDA((launch_density<8, 4, 2>(n_tiles, params, v0, begin, end, g, theta, max_spread, out_density, s)));
+    else if (B == 8 && sparse) DCUDA((launch_density<8, 2, 1>(n_tiles, params, v0, begin, end, g, theta, max_spread, out_density, s)));
     else if (B == 8) DCUDA((launch_density<8, 4, 1>(n_tiles, params, v0, begin, end, g, theta, max_spread, out_density, s)));
     else if (few) DCUDA((launch_density<4, 4, 4>(n_tiles, params, v0, begin, end, g, theta, max_spread, out_density, s)));
     else DCUDA((launch_density<4, 1, 1>(n_tiles, params, v0, begin, end, g, theta, max_spread, out_density, s)));
