@@ -593,7 +593,30 @@ bool host_mapped(const void* p, void** dev) {
 
 }  // namespace
 
+namespace {
+
+// The parts of a scene's device buffer and where they lie.
+struct SceneLayout {
+  struct {
+    const void* src;
+    size_t bytes;
+  } part[4];
+  size_t at[5] = {};
+  explicit SceneLayout(const fgl_scene_s& s)
+      : part{{s.bvh.nodes.data(), s.bvh.nodes.size()},
+             {s.bvh.tris.data(), s.bvh.tris.size() * sizeof(float)},
+             {s.cut_tris.data(), s.cut_tris.size() * sizeof(float)},
+             {s.cut, s.has_cut ? sizeof(s.cut) : 0}} {
+    for (int k = 0; k < 4; ++k) at[k + 1] = at[k] + part[k].bytes + (k == 0 ? -part[k].bytes % 256 : 0);
+  }
+};
+
+}  // namespace
+
 namespace fgl {
+
+// Device bytes of a resident scene (server.cu's budget).
+int64_t scene_device_bytes(fgl_scene s) { return (int64_t)SceneLayout(*s).at[4]; }
 
 // Item check + descriptor fill for fgl_cast_batched_static (static_batch.cu):
 // the same rules as check_item/make_desc, with constant messages so that a
@@ -668,15 +691,9 @@ fgl_status fgl_scene_upload(fgl_scene s) {
   // one allocation, and one copy of a small scene (108 triangles: 24 us with two
   // of each and no cut, 40 with the cut's own copies)
   constexpr size_t kStaged = 128 * 1024;
-  const struct {
-    const void* src;
-    size_t bytes;
-  } part[] = {{s->bvh.nodes.data(), s->bvh.nodes.size()},
-              {s->bvh.tris.data(), s->bvh.tris.size() * sizeof(float)},
-              {s->cut_tris.data(), s->cut_tris.size() * sizeof(float)},
-              {s->cut, s->has_cut ? sizeof(s->cut) : 0}};
-  size_t at[5] = {};
-  for (int k = 0; k < 4; ++k) at[k + 1] = at[k] + part[k].bytes + (k == 0 ? -part[k].bytes % 256 : 0);
+  const SceneLayout l(*s);
+  const auto& part = l.part;
+  const auto& at = l.at;
   void* buf = nullptr;
   const cudaError_t ae = cudaMalloc(&buf, at[4]);
   if (ae != cudaSuccess) {

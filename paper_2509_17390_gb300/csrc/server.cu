@@ -51,6 +51,7 @@
 
 namespace fgl {
 void record_error(int status, const char* msg);  // api.cu
+int64_t scene_device_bytes(fgl_scene s);         // api.cu
 }
 
 namespace {
@@ -626,7 +627,7 @@ fgl_status fgl_server_add_scene(fgl_server S, fgl_scene scene, int32_t* scene_id
   std::lock_guard<std::mutex> lk(S->mu);
   SceneEntry e;
   e.scene = scene;
-  e.bytes = st.node_bytes + st.tri_bytes;
+  e.bytes = fgl::scene_device_bytes(scene);  // with the cut behind the records
   e.resident = st.resident != 0;
   if (e.resident) {
     if (!make_room(*S, e.bytes, -1)) {
