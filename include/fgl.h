@@ -374,9 +374,10 @@ typedef struct {
  * all centroids), a stable radix sort, the hierarchy from longest common
  * prefixes (eq. LCP; equal codes ordered by position), then node boxes bottom
  * up; leaf boxes are grown by 2^-17 max(1, max |coord|).  The binary tree is
- * then opened into the 8-wide nodes that the casts walk (91 B a triangle, plus
- * 48 B for the triangles in their order; the build's scratch, about 110 B a
- * triangle, stays with the LBVH for the next rebuild).  Synchronises
+ * then opened into the 8-wide nodes that packets of rays walk (91 B a triangle,
+ * plus 48 B for the triangles in their order; left out where there is no room for
+ * them, casts are then slower).  The build's scratch, about 110 B a triangle,
+ * stays with the LBVH for the next rebuild.  Synchronises
  * `stream` at the end.  Errors: FGL_ERR_INVALID (empty mesh, nt >= 2^30, a
  * vertex id out of range or a non-finite vertex), FGL_ERR_OOM, FGL_ERR_CUDA.
  * A rebuild that fails leaves no tree: casts and exports return
@@ -390,7 +391,8 @@ fgl_status fgl_lbvh_get_stats(fgl_lbvh lbvh, fgl_lbvh_stats* out);
  * Morton order (48 B each, as the wide BVH's leaf records). */
 fgl_status fgl_lbvh_export(fgl_lbvh lbvh, void* nodes, int64_t node_bytes, void* tris,
                            int64_t tri_bytes);
-/* eq. t_j* over an LBVH, with fgl_cast's kernels on its 8-wide nodes: the same
+/* eq. t_j* over an LBVH, packets with fgl_cast's kernels on its 8-wide nodes,
+ * other rays one thread each on the binary nodes: the same
  * returns, bit for bit, as fgl_cast on a wide BVH of the same mesh (same
  * triangle test and (t, id) rule), t in [min_range, max_range]. */
 fgl_status fgl_cast_lbvh(fgl_lbvh lbvh, fgl_sensor sensor, const float* poses, int32_t n_env,

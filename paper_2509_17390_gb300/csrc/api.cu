@@ -916,7 +916,7 @@ fgl_status fgl_cast_lbvh(fgl_lbvh lbvh, fgl_sensor sensor, const float* poses, i
   const Opts o;
   ItemDesc d = lbvh_item(lbvh);
   const int packets =
-      packet_opts(8, o) ? lbvh_packets(sensor->packets, d.n_tris, (int64_t)n_env * sensor->n_rays) : 0;
+      d.nodes && packet_opts(8, o) ? lbvh_packets(sensor->packets, d.n_tris, (int64_t)n_env * sensor->n_rays) : 0;
   if (!packets) {
     FGL_CUDA(launch_lbvh_cast(lbvh, sensor->d_dirs, poses, n_env, sensor->n_rays, min_range, max_range, out_range,
                               out_tri, (cudaStream_t)stream));

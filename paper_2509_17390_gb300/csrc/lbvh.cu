@@ -48,6 +48,7 @@ struct fgl_lbvh_s {
   void* nodes = nullptr;   // (nt - 1) x 64 B
   void* tris = nullptr;    // nt x 48 B, Morton order
   void* wnodes = nullptr;  // wide_capacity(nt) x 256 B, n_wide of them made: what packets walk
+                           // (null: no room for it)
   void* wtris = nullptr;   // nt x 48 B, the wide nodes' leaf runs
   void* work = nullptr;    // build scratch
   size_t work_cap = 0;
@@ -793,11 +794,9 @@ extern "C" fgl_status fgl_lbvh_build(const float* d_verts, int64_t nv, const int
     L->nt = 0;
     cudaError_t e = cudaMalloc(&L->nodes, (size_t)std::max<int64_t>(1, nt - 1) * sizeof(LbvhNode));
     if (e == cudaSuccess) e = cudaMalloc(&L->tris, (size_t)nt * 48);
-    if (e == cudaSuccess) e = cudaMalloc(&L->wnodes, (size_t)wide_capacity(nt) * node_stride(8));
-    if (e == cudaSuccess) e = cudaMalloc(&L->wtris, (size_t)nt * 48);
     if (e != cudaSuccess) {
       cudaGetLastError();
-      for (void** b : {&L->nodes, &L->tris, &L->wnodes, &L->wtris}) {
+      for (void** b : {&L->nodes, &L->tris}) {
         if (*b) cudaFree(*b);
         *b = nullptr;
       }
@@ -830,6 +829,14 @@ extern "C" fgl_status fgl_lbvh_build(const float* d_verts, int64_t nv, const int
       return err(FGL_ERR_OOM, "cannot allocate LBVH build scratch");
     }
     L->work_cap = off;
+  }
+  // The wide form is a third of the LBVH: a mesh that fits without it is built
+  // without it, and its casts take the binary tree.
+  if (!L->wnodes && (cudaMalloc(&L->wnodes, (size_t)wide_capacity(nt) * node_stride(8)) != cudaSuccess ||
+                     cudaMalloc(&L->wtris, (size_t)nt * 48) != cudaSuccess)) {
+    cudaGetLastError();
+    if (L->wnodes) cudaFree(L->wnodes);
+    L->wnodes = L->wtris = nullptr;
   }
   char* w = (char*)L->work;
   float4* tbox = (float4*)(w + o_tbox);
@@ -879,7 +886,7 @@ extern "C" fgl_status fgl_lbvh_build(const float* d_verts, int64_t nv, const int
         (LbvhNode*)L->nodes, par, flags, nbox, lbox, roots, bounds + 9, bounds + 7);
     LCUDA(cudaGetLastError());
   }
-  {
+  if (L->wnodes) {
     WideArgs a{(const LbvhNode*)L->nodes, split, lbox, (const float4*)L->tris, nt, (uint8_t*)L->wnodes,
                (float4*)L->wtris, wroot, bounds + 10, bounds + 16, (int)wide_capacity(nt)};
     int dev = 0, sms = 0, per_sm = 0;
@@ -906,7 +913,7 @@ extern "C" fgl_status fgl_lbvh_build(const float* d_verts, int64_t nv, const int
   }
   L->margin = std::ldexp(std::max(1.f, iord(host[6])), -17);
   L->depth = nt > 1 ? host[7] : 1;
-  L->n_wide = 1;
+  L->n_wide = L->wnodes ? 1 : 0;
   for (int lv = 0; lv < kWideLevels; ++lv) L->n_wide += host[16 + lv];
   L->built = true;
   cudaGetDevice(&L->device);
