@@ -91,63 +91,6 @@ __device__ __forceinline__ void setup_ray(Ray& r, float ox, float oy, float oz, 
   r.Sy = __fmul_rn(sel3(dx, dy, dz, ky), r.Sz);
 }
 
-// The three edge functions in float64 (products of two floats are exact
-// there; one rounding per difference).
-static __device__ __noinline__ float3 edges64(float Ax, float Ay, float Bx, float By, float Cx, float Cy) {
-  return make_float3((float)((double)Cx * (double)By - (double)Cy * (double)Bx),
-                     (float)((double)Ax * (double)Cy - (double)Ay * (double)Cx),
-                     (float)((double)Bx * (double)Ay - (double)By * (double)Ax));
-}
-
-// The test from the translated vertices in the ray's axes: (X, Y, Z) of each
-// vertex are its kx, ky, kz coordinates minus the origin's.
-template <bool kAll>
-__device__ __forceinline__ float tri_hit_axes(const Ray& r, float AX, float AY, float Akz, float BX, float BY,
-                                              float Bkz, float CX, float CY, float Ckz, float tbest) {
-  float Ax = __fsub_rn(AX, __fmul_rn(r.Sx, Akz));
-  float Ay = __fsub_rn(AY, __fmul_rn(r.Sy, Akz));
-  float Bx = __fsub_rn(BX, __fmul_rn(r.Sx, Bkz));
-  float By = __fsub_rn(BY, __fmul_rn(r.Sy, Bkz));
-  float Cx = __fsub_rn(CX, __fmul_rn(r.Sx, Ckz));
-  float Cy = __fsub_rn(CY, __fmul_rn(r.Sy, Ckz));
-  float U = __fsub_rn(__fmul_rn(Cx, By), __fmul_rn(Cy, Bx));
-  float V = __fsub_rn(__fmul_rn(Ax, Cy), __fmul_rn(Ay, Cx));
-  float W = __fsub_rn(__fmul_rn(Bx, Ay), __fmul_rn(By, Ax));
-  const bool zero = U == 0.f || V == 0.f || W == 0.f;
-  if (kAll) {
-    // In a loop that all lanes run together the compiler turns the rare
-    // float64 fallback into predicated work of every test (it kept this chip's
-    // small float64 pipe 86% busy); behind a call it stays a branch.
-    if (__any_sync(0xFFFFFFFFu, zero)) {
-      const float3 e = edges64(Ax, Ay, Bx, By, Cx, Cy);
-      if (zero) {
-        U = e.x;
-        V = e.y;
-        W = e.z;
-      }
-    }
-  } else if (zero) {
-    // products of two floats are exact in double; one rounding per difference
-    double u = (double)Cx * (double)By - (double)Cy * (double)Bx;
-    double v = (double)Ax * (double)Cy - (double)Ay * (double)Cx;
-    double w = (double)Bx * (double)Ay - (double)By * (double)Ax;
-    U = (float)u;
-    V = (float)v;
-    W = (float)w;
-  }
-  const bool miss = (U < 0.f || V < 0.f || W < 0.f) && (U > 0.f || V > 0.f || W > 0.f);
-  if (kAll ? __all_sync(0xFFFFFFFFu, miss) : miss) return -1.f;
-  float det = __fadd_rn(__fadd_rn(U, V), W);
-  float Az = __fmul_rn(r.Sz, Akz), Bz = __fmul_rn(r.Sz, Bkz), Cz = __fmul_rn(r.Sz, Ckz);
-  float T = __fadd_rn(__fadd_rn(__fmul_rn(U, Az), __fmul_rn(V, Bz)), __fmul_rn(W, Cz));
-  // t = T/det must be > 0: same sign, T != 0; certainly beyond tbest:
-  // |T| > tbest*|det|*(1+2^-20) implies fl(T/det) > tbest
-  const bool off = miss || det == 0.f || ((__float_as_uint(T) ^ __float_as_uint(det)) >> 31) || T == 0.f ||
-                   fabsf(T) > __fmul_rn(__fmul_rn(tbest, fabsf(det)), 1.00000095367431640625f);
-  if (off) return -1.f;
-  return __fdiv_rn(T, det);
-}
-
 // Watertight float32 ray/triangle test (Woop, Benthin & Wald 2013, JCGT 2(1)):
 // translate the vertices to the ray origin, shear so the ray is the +z axis
 // of the (kx, ky, kz) frame, and take the signs of the three 2D edge
@@ -159,9 +102,83 @@ __device__ __forceinline__ float tri_hit(const Ray& r, float4 a, float4 b, float
   float A0 = __fsub_rn(a.x, r.ox), A1 = __fsub_rn(a.y, r.oy), A2 = __fsub_rn(a.z, r.oz);
   float B0 = __fsub_rn(b.x, r.ox), B1 = __fsub_rn(b.y, r.oy), B2 = __fsub_rn(b.z, r.oz);
   float C0 = __fsub_rn(c.x, r.ox), C1 = __fsub_rn(c.y, r.oy), C2 = __fsub_rn(c.z, r.oz);
-  return tri_hit_axes<false>(r, sel3(A0, A1, A2, kx), sel3(A0, A1, A2, ky), sel3(A0, A1, A2, kz), sel3(B0, B1, B2, kx),
-                      sel3(B0, B1, B2, ky), sel3(B0, B1, B2, kz), sel3(C0, C1, C2, kx), sel3(C0, C1, C2, ky),
-                      sel3(C0, C1, C2, kz), tbest);
+  float Akz = sel3(A0, A1, A2, kz), Bkz = sel3(B0, B1, B2, kz), Ckz = sel3(C0, C1, C2, kz);
+  float Ax = __fsub_rn(sel3(A0, A1, A2, kx), __fmul_rn(r.Sx, Akz));
+  float Ay = __fsub_rn(sel3(A0, A1, A2, ky), __fmul_rn(r.Sy, Akz));
+  float Bx = __fsub_rn(sel3(B0, B1, B2, kx), __fmul_rn(r.Sx, Bkz));
+  float By = __fsub_rn(sel3(B0, B1, B2, ky), __fmul_rn(r.Sy, Bkz));
+  float Cx = __fsub_rn(sel3(C0, C1, C2, kx), __fmul_rn(r.Sx, Ckz));
+  float Cy = __fsub_rn(sel3(C0, C1, C2, ky), __fmul_rn(r.Sy, Ckz));
+  float U = __fsub_rn(__fmul_rn(Cx, By), __fmul_rn(Cy, Bx));
+  float V = __fsub_rn(__fmul_rn(Ax, Cy), __fmul_rn(Ay, Cx));
+  float W = __fsub_rn(__fmul_rn(Bx, Ay), __fmul_rn(By, Ax));
+  if (U == 0.f || V == 0.f || W == 0.f) {
+    // products of two floats are exact in double; one rounding per difference
+    double u = (double)Cx * (double)By - (double)Cy * (double)Bx;
+    double v = (double)Ax * (double)Cy - (double)Ay * (double)Cx;
+    double w = (double)Bx * (double)Ay - (double)By * (double)Ax;
+    U = (float)u;
+    V = (float)v;
+    W = (float)w;
+  }
+  if ((U < 0.f || V < 0.f || W < 0.f) && (U > 0.f || V > 0.f || W > 0.f)) return -1.f;
+  float det = __fadd_rn(__fadd_rn(U, V), W);
+  if (det == 0.f) return -1.f;
+  float Az = __fmul_rn(r.Sz, Akz), Bz = __fmul_rn(r.Sz, Bkz), Cz = __fmul_rn(r.Sz, Ckz);
+  float T = __fadd_rn(__fadd_rn(__fmul_rn(U, Az), __fmul_rn(V, Bz)), __fmul_rn(W, Cz));
+  // t = T/det must be > 0: same sign, T != 0
+  if (((__float_as_uint(T) ^ __float_as_uint(det)) >> 31) || T == 0.f) return -1.f;
+  // certainly beyond tbest: |T| > tbest*|det|*(1+2^-20) implies fl(T/det) > tbest
+  if (fabsf(T) > __fmul_rn(__fmul_rn(tbest, fabsf(det)), 1.00000095367431640625f)) return -1.f;
+  return __fdiv_rn(T, det);
+}
+
+// The three edge functions in float64 (products of two floats are exact
+// there; one rounding per difference).
+static __device__ __noinline__ float3 edges64(float Ax, float Ay, float Bx, float By, float Cx, float Cy) {
+  return make_float3((float)((double)Cx * (double)By - (double)Cy * (double)Bx),
+                     (float)((double)Ax * (double)Cy - (double)Ay * (double)Cx),
+                     (float)((double)Bx * (double)Ay - (double)By * (double)Ax));
+}
+
+// The same test of one triangle by all 32 lanes, each with its own ray, from the
+// translated vertices in the rays' axes: (X, Y, Z) of each vertex are its kx, ky,
+// kz coordinates minus the origin's.  Written apart because the two do not share a
+// good form: in a loop that all lanes run together the compiler turns the rare
+// float64 fallback into predicated work of every test (it kept this chip's small
+// float64 pipe 86% busy), and behind a call it stays a branch; ray by ray, one
+// expression of all the rejections costs 1-6% of a cast.
+__device__ __forceinline__ float tri_hit_packet(const Ray& r, float AX, float AY, float Akz, float BX, float BY,
+                                                float Bkz, float CX, float CY, float Ckz, float tbest) {
+  float Ax = __fsub_rn(AX, __fmul_rn(r.Sx, Akz));
+  float Ay = __fsub_rn(AY, __fmul_rn(r.Sy, Akz));
+  float Bx = __fsub_rn(BX, __fmul_rn(r.Sx, Bkz));
+  float By = __fsub_rn(BY, __fmul_rn(r.Sy, Bkz));
+  float Cx = __fsub_rn(CX, __fmul_rn(r.Sx, Ckz));
+  float Cy = __fsub_rn(CY, __fmul_rn(r.Sy, Ckz));
+  float U = __fsub_rn(__fmul_rn(Cx, By), __fmul_rn(Cy, Bx));
+  float V = __fsub_rn(__fmul_rn(Ax, Cy), __fmul_rn(Ay, Cx));
+  float W = __fsub_rn(__fmul_rn(Bx, Ay), __fmul_rn(By, Ax));
+  const bool zero = U == 0.f || V == 0.f || W == 0.f;
+  if (__any_sync(0xFFFFFFFFu, zero)) {
+    const float3 e = edges64(Ax, Ay, Bx, By, Cx, Cy);
+    if (zero) {
+      U = e.x;
+      V = e.y;
+      W = e.z;
+    }
+  }
+  const bool miss = (U < 0.f || V < 0.f || W < 0.f) && (U > 0.f || V > 0.f || W > 0.f);
+  if (__all_sync(0xFFFFFFFFu, miss)) return -1.f;
+  float det = __fadd_rn(__fadd_rn(U, V), W);
+  float Az = __fmul_rn(r.Sz, Akz), Bz = __fmul_rn(r.Sz, Bkz), Cz = __fmul_rn(r.Sz, Ckz);
+  float T = __fadd_rn(__fadd_rn(__fmul_rn(U, Az), __fmul_rn(V, Bz)), __fmul_rn(W, Cz));
+  // t = T/det must be > 0: same sign, T != 0; certainly beyond tbest:
+  // |T| > tbest*|det|*(1+2^-20) implies fl(T/det) > tbest
+  const bool off = miss || det == 0.f || ((__float_as_uint(T) ^ __float_as_uint(det)) >> 31) || T == 0.f ||
+                   fabsf(T) > __fmul_rn(__fmul_rn(tbest, fabsf(det)), 1.00000095367431640625f);
+  if (off) return -1.f;
+  return __fdiv_rn(T, det);
 }
 
 // Child keys of a node group: one 16-bit key per child slot, two per 32-bit
@@ -743,7 +760,9 @@ __device__ __forceinline__ PacketEnd packet_phase(Tracer<W, COUNT, TMIN>& tr, fl
   const float toX = sel3(tr.r.ox, tr.r.oy, tr.r.oz, tkx), toY = sel3(tr.r.ox, tr.r.oy, tr.r.oz, tky),
               toZ = sel3(tr.r.ox, tr.r.oy, tr.r.oz, tkz);
 
-  uint32_t tkey = __float_as_uint(tr.best_t) | 7u;  // the farthest best hit of the packet, as a key
+  // the farthest best hit of the packet, as a key; it steers the warp, so all
+  // lanes have to come with one best_t (they start at the item's max_range)
+  uint32_t tkey = __float_as_uint(tr.best_t) | 7u;
   // a box in the packet's frame: the earliest entry of a ray (tn), and whether
   // some ray may meet it (then these differences are all non-negative)
   auto meets = [&](float X0, float X1, float Y0, float Y1, float zn, float zf, float zc, float& tn) {
@@ -775,9 +794,9 @@ __device__ __forceinline__ PacketEnd packet_phase(Tracer<W, COUNT, TMIN>& tr, fl
       const float* py = tp + tky;
       const float* pz = tp + tkz;
       const int32_t id = __ldg((const int32_t*)tp + 3);
-      tr.consider(tri_hit_axes<true>(tr.r, __ldg(px) - toX, __ldg(py) - toY, __ldg(pz) - toZ, __ldg(px + 4) - toX,
-                               __ldg(py + 4) - toY, __ldg(pz + 4) - toZ, __ldg(px + 8) - toX, __ldg(py + 8) - toY,
-                               __ldg(pz + 8) - toZ, tr.best_t),
+      tr.consider(tri_hit_packet(tr.r, __ldg(px) - toX, __ldg(py) - toY, __ldg(pz) - toZ, __ldg(px + 4) - toX,
+                                 __ldg(py + 4) - toY, __ldg(pz + 4) - toZ, __ldg(px + 8) - toX, __ldg(py + 8) - toY,
+                                 __ldg(pz + 8) - toZ, tr.best_t),
                   id);
     }
     return true;
