@@ -164,7 +164,7 @@ def _torch():
 
 
 # A small cast's time is this path's (18 us a call before these, 11.5 now): the
-# the raw handle instead of a Stream object, dtypes compared as objects, torch
+# raw handle instead of a Stream object, dtypes compared as objects, torch
 # looked up once.
 def _stream_handle(stream) -> Optional[int]:
     if stream is None:

@@ -1328,7 +1328,7 @@ __global__ void __launch_bounds__(kMtThreads) k_mt_count(const uint32_t* __restr
     pre[3 * blockIdx.x + 1] = off[1] + run[1];
     pre[3 * blockIdx.x + 2] = (unsigned long long)(off[2] + run[2]) | ((unsigned long long)(off[3] + run[3]) << 32);
   }
-  if constexpr (QUERY) return;
+  if (QUERY) return;
 #pragma unroll
   for (int u = 0; u < PER; ++u) {
     const int pi = mt_pad(tid * PER + u);
@@ -2013,7 +2013,6 @@ extern "C" fgl_status fgl_tsdf(const uint8_t* surf, const fgl_grid* grid, float 
     MCUDA(cudaEventRecord(e0, s));
   }
   int launches = 0;
-  const dim3 vg = voxel_grid(g.nx, g.rows());
   const unsigned rb = word_blocks(g.rows() * 32, 256);
   if (tp.ty) {  // tiles pack the surface themselves
     uint8_t* tile_global = (uint8_t*)S.tiles.p;
