@@ -271,7 +271,7 @@ __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
 // (below 2^-126) the row's largest value is below 2^-45.  P^2 has to stay
 // finite too (|g h / 2| <= kRowSlope), so that a row far from the Gaussian adds
 // 0 and not 0 times infinity; a Gaussian that would widen the band below too far
-// (kMaxSpread) or whose opacity is not finite is left out as well.  A Gaussian
+// (kMaxSpread) or whose alpha^2 is above kMaxWeight is left out as well.  A Gaussian
 // outside these limits (steep) is evaluated voxel by voxel.
 constexpr float kRowFall = 20.f, kRowSlope = 60.f;
 
@@ -280,22 +280,25 @@ constexpr float kRowFall = 20.f, kRowSlope = 60.f;
 // voxel in candidate order, so that the masks are those of that sum to the last
 // bit.  Steep Gaussians' terms are that sum's, bit for bit.  A factored term's
 // exponent differs from that sum's by at most u = 2^-24 times
-//   11 X G + 6 Q + 150,   X = |dx|, G = |M01| |dy| + |M02| |dz| + 2 |M00| |dx|,
-//                         Q = |M11| dy^2 + |M12 dy dz| + |M22| dz^2,
-// each at its largest over the tile: roundings of dx, xm (1 and 2.5 u X, each times
-// the slope G), of the x coefficient (2 and 3 u G, times X), of the slope's up to 7
-// half voxels (28 u G h / 2 <= 2 u X G), of the y/z part (3 u Q in each form) and of
-// the sums (exponents to -64 and the middle's 420 beyond it at most; smaller terms
-// are below the slack).  The exponentials and products add 6e-6.  Sums of n
-// positive terms in two orders differ by at most 1.5 n u.  So the band is
-//   kBand + 1.5 n u + max over the tile's factored Gaussians of u (8 X G + 4.5 Q)
-// relative, and 2^-44 alpha^2 a candidate absolute for rows whose middle flushes.
+//   14.4 X G + 6 Q + 150,   X = |dx|, G = |M01| |dy| + |M02| |dz| + 2 |M00| |dx|,
+//                           Q = |M11| dy^2 + |M12 dy dz| + |M22| dz^2,
+// each at its largest over the tile: roundings of xm and dx (1 and 4 u X, each times
+// the slope G), of the x coefficient (2 and 3 u G, times X), of the slope's up to B - 1
+// half voxels and the middle's value (35 u G h / 2, 15 for B = 4, where X >= B h / 2), of
+// the y/z part (3 u Q in each form) and of the sums (exponents to -64 and the middle's
+// 84 beyond the slope; smaller terms are below the slack).  The exponentials and
+// products add 5e-6.  Sums of n
+// positive terms in candidate order and in N parts err by at most n u and n u / N
+// (and kBand covers the parts' own sum).  So the band is
+//   kBand + (1 + 1 / N) n u + max over the tile's factored Gaussians of u (10.5 X G + 4.5 Q)
+// relative, and 2^-44 kMaxWeight a candidate absolute for rows whose middle flushes.
 // On 60 k to 90 k Gaussians of 1 to 20 cm at 2.5 to 5 cm voxels the band is about
-// 1e-3 (one tile in 12 to 50 has a voxel in it, which no time shows) and kMaxSpread
-// makes up to 0.4% of the factored Gaussians steep; 5e-4 makes 1-4% (1.829 -> 1.836
-// ms in all), 3e-4 1.856.
+// 7e-4 (one tile in 14 to 50 has a voxel in it) and kMaxSpread makes 1-4% of the
+// factored Gaussians steep; twice that, up to 0.4%.  A tile of many candidates with
+// such a voxel can hold up a grid of few tiles (29 k Gaussians, 120 tiles: the call 120
+// us, 141 at twice that), and so do steep Gaussians (243 k: 301 us, 308 at a third).
 constexpr float kUnit = 5.9604645e-8f;  // u
-constexpr float kBand = 2e-5f, kMaxSpread = 1e-3f;
+constexpr float kBand = 2e-5f, kMaxSpread = 6e-4f, kMaxWeight = 4.f;
 constexpr int kCloseAtOnce = 8;
 
 // One staged candidate.  bx = M01 dy + M02 dz is the x coefficient and
@@ -365,7 +368,7 @@ __global__ void __launch_bounds__(32 * S)
   // candidate numbers one batch earlier
   GaussParams P = {};
   uint32_t next = 0;
-  float spread = 0.f, weight = 0.f;  // over the lane's factored candidates: the largest u (8 X G + 4.5 Q) and alpha^2
+  float spread = 0.f;  // the largest u (10.5 X G + 4.5 Q) of the lane's factored candidates
   if (first + lane < b1) P = params[cand[first + lane]];
   if (first + stride + lane < b1) next = cand[first + stride + lane];
   for (uint32_t c0 = first; c0 < b1; c0 += stride) {
@@ -378,13 +381,10 @@ __global__ void __launch_bounds__(32 * S)
                 Z = fmaxf(fabsf(dZ), fabsf(dZ + edge));
     const float G = fabsf(P.b.w) * Y + fabsf(P.c.x) * Z + 2.f * fabsf(P.b.x) * X, slope = hh * G;  // |g h / 2| at most: P^2 stays finite
     const float Q = fabsf(P.b.y) * (Y * Y) + fabsf(P.c.y) * (Y * Z) + fabsf(P.b.z) * (Z * Z);
-    const float d_spread = kUnit * (8.f * (X * G) + 4.5f * Q);
+    const float d_spread = kUnit * (10.5f * (X * G) + 4.5f * Q);
     const bool fast = valid && fabsf(P.b.x) * (end_d * end_d) <= kRowFall && slope <= kRowSlope &&
-                      d_spread <= max_spread && P.a.w < INFINITY;
-    if (fast) {
-      spread = fmaxf(spread, d_spread);
-      weight = fmaxf(weight, P.a.w);
-    }
+                      d_spread <= max_spread && P.a.w <= kMaxWeight;
+    if (fast) spread = fmaxf(spread, d_spread);
     // the factored ones first, steep ones from the end
     const unsigned fm = __ballot_sync(FULL, fast), sm = __ballot_sync(FULL, valid && !fast);
     const unsigned below = (1u << lane) - 1u;
@@ -457,11 +457,9 @@ __global__ void __launch_bounds__(32 * S)
       }
     }
   }
-  // the warps' largest spread and weight (non-negative floats order as integers)
-  __shared__ float2 s_band[K * S];
+  __shared__ float s_band[K * S];  // the warps' largest spread (non-negative floats order as integers)
   spread = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(spread)));
-  weight = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(weight)));
-  if (lane == 0) s_band[warp] = make_float2(spread, weight);
+  if (lane == 0) s_band[warp] = spread;
   float d[2][B];  // the rows' densities, complete in warp 0's lanes of sub 0
 #pragma unroll
   for (int r = 0; r < 2; ++r)
@@ -531,14 +529,10 @@ __global__ void __launch_bounds__(32 * S)
   if (threadIdx.x == 0) s_n_close = 0;
   __syncthreads();
   if (owner) {
-    float band = 0.f, slack = 0.f;
-    for (int t = 0; t < (split ? K * S : S); ++t) {
-      band = fmaxf(band, s_band[t].x);
-      slack = fmaxf(slack, s_band[t].y);
-    }
-    const float n = (float)(b1 - b0);
-    band += kBand + 1.5f * kUnit * n;
-    slack = n * (slack * 0x1p-44f + 0x1p-148f);
+    float band = 0.f;
+    for (int t = 0; t < (split ? K * S : S); ++t) band = fmaxf(band, s_band[t]);
+    const float n = (float)(b1 - b0), slack = n * (max_spread < 0.f ? 0x1p-148f : kMaxWeight * 0x1p-44f);
+    band += kBand + (1.f + 1.f / (float)(C::SUB * S * (split ? K : 1))) * kUnit * n;
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const int gz = tz * B + z + r * (B / 2);
@@ -559,8 +553,12 @@ __global__ void __launch_bounds__(32 * S)
   for (int v0 = 0; v0 < n_close; v0 += kCloseAtOnce) {
     const int n = min(kCloseAtOnce, n_close - v0);
     float sum = 0.f;
+    // a batch's parameters travel while the one before it is summed, its
+    // candidate numbers one batch earlier
     GaussParams Q = {};
+    uint32_t ahead = 0;
     if (b0 + threadIdx.x < b1) Q = params[cand[b0 + threadIdx.x]];
+    if (b0 + NT + threadIdx.x < b1) ahead = cand[b0 + NT + threadIdx.x];
     int buf = 0;
     for (uint32_t c0 = b0; c0 < b1; c0 += NT, buf ^= 1) {
       const bool some = c0 + threadIdx.x < b1;
@@ -578,7 +576,8 @@ __global__ void __launch_bounds__(32 * S)
         const float bx = fmaf(Q.b.w, dy, __fmul_rn(Q.c.x, dz));
         sh.terms[buf][1 + v][threadIdx.x] = some ? dev::ex2_approx(fmaf(fmaf(Q.b.x, dx, bx), dx, syz)) : 0.f;
       }
-      if (c0 + NT + threadIdx.x < b1) Q = params[cand[c0 + NT + threadIdx.x]];
+      if (c0 + NT + threadIdx.x < b1) Q = params[ahead];
+      if (c0 + 2 * NT + threadIdx.x < b1) ahead = cand[c0 + 2 * NT + threadIdx.x];
       __syncthreads();  // and the batch before this one is summed
       if (threadIdx.x < (unsigned)n) {
 #pragma unroll 4
@@ -814,28 +813,32 @@ extern "C" fgl_status fgl_gaussian_density(const fgl_gaussians* gs, const fgl_gr
     DCUDA(cudaGetLastError());
     if (timing) DCUDA(cudaEventRecord(S.ev[1], s));
     // Warps a tile, by the mean of its candidates (wall time of the call, us):
-    //   candidates a tile            0.1    5   16   53  211  729 1885    5, half of them within 10 cm
-    //   two warps                    816  393  457  643 1547  541         776
-    //   four                         917  553  581  727 1473  522 1828    648
-    //   four in each of two blocks,
-    //   a cluster                   1275  895  919 1182 2494  566 1877    852
+    //   candidates a tile          0.1    5   16   53  211  729 1885    5, half of them within 10 cm
+    //   two warps                  816  393  457  643 1547  541         776
+    //   four                       917  553  581  727 1473  522 1828    648
+    //   eight                                   1152 1603  529 1815
+    //   four in each of two
+    //   blocks, a cluster         1275  895  919 1182 2494  566 1877    852
     //   (two warps that share every candidate, one exponential a voxel:
-    //                               1155  411  464  827 2216  782 2940    838)
+    //                             1155  411  464  827 2216  782 2940    838)
     // over 262,144 tiles with 2,000 Gaussians, 62,500 with 20 k to 800 k, 6,500 and
-    // 10,304 dense ones: two warps for a sparse grid, four for the others.  A grid of
-    // fewer than 16 tiles an SM takes eight warps in four blocks, or its heaviest
-    // tiles would run on alone (630 tiles: the call 0.54 ms in one block, 0.49 in two,
-    // 0.475 in four or eight).  Tiles of 4^3 voxels have fewer candidates each: one
-    // block of one warp where there are many (25,000 tiles: 1.60 ms; two blocks 2.33).
+    // 10,304 dense ones: two warps for a sparse grid, eight for a dense one, whose
+    // heaviest tiles they even out best (5,000 tiles of 400 k Gaussians 790 us, four
+    // 828).  A grid of fewer than 16 tiles an SM takes eight warps in four blocks, or
+    // its heaviest tiles would run on alone (630 tiles: the call 0.54 ms in one block,
+    // 0.49 in two, 0.475 in four or eight).  Tiles of 4^3 voxels have fewer candidates
+    // each: one block of one warp where there are many (25,000 tiles: 1.60 ms; two
+    // blocks 2.33).
     const GaussParams* params = (const GaussParams*)S.params;
+    const bool few = n_tiles < 152 * 16;
     // where theta is as small as what flushed rows leave out (or 0: any density
     // counts), every Gaussian is summed voxel by voxel
     const float max_spread = theta >= 0.f && theta < 0x1p-30f ? -1.f : kMaxSpread;
-    const bool few = n_tiles < 152 * 16;
-    const bool sparse = (int64_t)n_pairs < 32 * n_tiles;
+    const int64_t mean = (int64_t)n_pairs / n_tiles;
     if (B == 8 && few) DCUDA((launch_density<8, 8, 4>(n_tiles, params, v0, begin, end, g, theta, max_spread, out_density, s)));
-    else if (B == 8 && sparse) DCUDA((launch_density<8, 2, 1>(n_tiles, params, v0, begin, end, g, theta, max_spread, out_density, s)));
-    else if (B == 8) DCUDA((launch_density<8, 4, 1>(n_tiles, params, v0, begin, end, g, theta, max_spread, out_density, s)));
+    else if (B == 8 && mean < 32) DCUDA((launch_density<8, 2, 1>(n_tiles, params, v0, begin, end, g, theta, max_spread, out_density, s)));
+    else if (B == 8 && mean < 256) DCUDA((launch_density<8, 4, 1>(n_tiles, params, v0, begin, end, g, theta, max_spread, out_density, s)));
+    else if (B == 8) DCUDA((launch_density<8, 8, 1>(n_tiles, params, v0, begin, end, g, theta, max_spread, out_density, s)));
     else if (few) DCUDA((launch_density<4, 4, 4>(n_tiles, params, v0, begin, end, g, theta, max_spread, out_density, s)));
     else DCUDA((launch_density<4, 1, 1>(n_tiles, params, v0, begin, end, g, theta, max_spread, out_density, s)));
     ++launches;
