@@ -318,12 +318,15 @@ void build_table(const fgl_cast_item* items, int n, const Opts& o, std::vector<G
     Group g;
     g.W = W;
     int64_t together = 0, rays = 0;  // packets of items that gain less those of the others
-    for (int i = 0; i < n; ++i) {
-      if (items[i].scene->bvh.width != W || items[i].n_env == 0) continue;
-      const int64_t packets = (int64_t)items[i].n_env * ((items[i].sensor->n_rays + 31) / 32);
-      together += batch_packets(items[i].sensor->packets, items[i].scene->bvh.n_tris) ? packets : -packets;
-      rays += (int64_t)items[i].n_env * items[i].sensor->n_rays;
-    }
+    auto each = [&](auto f) {
+      for (int i = 0; i < n; ++i)
+        if (items[i].scene->bvh.width == W && items[i].n_env > 0) f(items[i], (int64_t)items[i].n_env);
+    };
+    each([&](const fgl_cast_item& it, int64_t envs) { rays += envs * it.sensor->n_rays; });
+    each([&](const fgl_cast_item& it, int64_t envs) {
+      const int64_t packets = envs * ((it.sensor->n_rays + 31) / 32);
+      together += batch_packets(it.sensor->packets, walk_cost(it.scene->bvh), rays) ? packets : -packets;
+    });
     g.packets = together >= 0 && packet_opts(W, o);
     const int P = g.packets && !o.own_packet ? batch_packet_rays(rays) : o.packet;
     g.packet_rays = P;
@@ -621,7 +624,8 @@ int64_t scene_device_bytes(fgl_scene s) { return (int64_t)SceneLayout(*s).at[4];
 // Item check + descriptor fill for fgl_cast_batched_static (static_batch.cu):
 // the same rules as check_item/make_desc, with constant messages so that a
 // valid item costs no allocation.  Returns nullptr when the item is valid.
-const char* static_item_desc(const fgl_cast_item& it, ItemDesc* d, int* width, bool* together) {
+const char* static_item_desc(const fgl_cast_item& it, ItemDesc* d, int* width, int* packets,
+                             float* cost) {
   if (!it.scene || !it.sensor) return "null scene or sensor in an item";
   if (it.n_env < 0) return "n_env < 0 in an item";
   if (!(std::isfinite(it.max_range) && it.max_range > 0.f))
@@ -636,7 +640,8 @@ const char* static_item_desc(const fgl_cast_item& it, ItemDesc* d, int* width, b
     return "instances and return points need fgl_cast_batched";
   *d = make_desc(it);
   *width = it.scene->bvh.width;
-  *together = batch_packets(it.sensor->packets, it.scene->bvh.n_tris);
+  *packets = it.sensor->packets;
+  *cost = walk_cost(it.scene->bvh);
   return nullptr;
 }
 
@@ -870,7 +875,7 @@ fgl_status fgl_cast(fgl_scene scene, fgl_sensor sensor, const float* poses, int3
   Opts o;
   ItemDesc d = make_desc(it);
   const int packets = packet_opts(scene->bvh.width, o)
-                          ? cast_packets(sensor->packets, scene->bvh.n_tris, (int64_t)n_env * sensor->n_rays)
+                          ? cast_packets(sensor->packets, walk_cost(scene->bvh), (int64_t)n_env * sensor->n_rays)
                           : 0;
   FGL_CUDA(launch_plain(scene->bvh.width, false, packets, false, d, nullptr, o.block, o.sdepth, o.tri_mode,
                         o.postpone, (cudaStream_t)stream));
@@ -890,7 +895,7 @@ fgl_status fgl_cast_opts(fgl_scene scene, fgl_sensor sensor, const float* poses,
   ItemDesc d = make_desc(it);
   // the refill threshold has no meaning here
   const int packets = o.tri_mode == 0 && packets_fit(scene->bvh.width, o.block, o.sdepth)
-                          ? cast_packets(sensor->packets, scene->bvh.n_tris, (int64_t)n_env * sensor->n_rays)
+                          ? cast_packets(sensor->packets, walk_cost(scene->bvh), (int64_t)n_env * sensor->n_rays)
                           : 0;
   FGL_CUDA(launch_plain(scene->bvh.width, o.count != 0, packets, false, d, nullptr, o.block, o.sdepth, o.tri_mode,
                         o.postpone, (cudaStream_t)stream));

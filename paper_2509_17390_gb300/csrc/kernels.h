@@ -14,36 +14,51 @@ size_t stack_smem_bytes(int W, int block, int sdepth);
 
 // How a cast walks the tree: packets of this many consecutive rays of an
 // environment a warp, together (16 or 32), or each ray for itself (0).  By what the
-// sensor's packets are like (see sensor_packets), the scene's triangles and the
-// rays; the figures are shares of the time ray by ray, over sensors of 5 to 128
-// beams and 91 to 2048 columns and rooms of 108 to 1 M triangles:
-//   sensor   close packets 0.6-1.05 at any number of rays; fair ones 0.9-1.05 from 220 k
-//            rays on, up to 1.15 at 100 k; narrow ones 1.01-1.15
-//   tris     where a walk is short there is little to share: rooms of up to
-//            1,084 triangles 0.75-1.35 up to 220 k rays, from 800 k on 0.65-1.0
-//   16 rays  half of the lanes idle, but a packet ends sooner, which counts when
-//            packets of 16 come to at most two for each of the 28 warps an SM
-//            holds (1 M triangles, 57,600 rays 42 -> 35 us, 131,072 51 -> 44;
-//            184,320 would take 82 instead of 75).  Fair and narrow ones gain up
-//            to half as many rays, on 9,868 triangles and more (0.66-1.05)
+// sensor's packets are like (see sensor_packets), the scene's walk cost and the
+// rays; the figures are shares of the time ray by ray, over sensors of 4 to 128
+// beams and 91 to 2048 columns, rooms with one object (108 to 2,796 triangles, cost
+// 5-6) to cluttered ones (300 to 1 M, 7-60) and 1,000 to 13 M rays:
+//   close  0.55-0.95 from 400 k rays on in any scene; below, 0.7-1.1, but 1.0-1.4 in
+//          rooms of cost 5, whose walks have little to share
+//   fair   0.85-1.03 from 400 k rays on, 0.95-1.1 from 68 k to 220 k
+//   narrow 0.9-1.1 from 400 k rays on, 1.0-1.25 from 68 k to 220 k
+// Packets of 16 leave half of the lanes idle, but one ends sooner, which counts when
+// they come to at most two for each of the 28 warps an SM holds (1 M triangles,
+// 57,600 rays 42 -> 35 us, 131,072 51 -> 44; 184,320 would take 82 instead of 75).
+// Fair ones gain (0.8-1.1) up to half as many rays, narrow ones (0.85-1.1) a quarter.
 constexpr int64_t kSmallCastRays = 16 * 2 * 28 * 152;
 inline bool small_cast(int64_t rays) { return rays <= kSmallCastRays; }
 
 enum SensorPackets { kSpreadPackets = 0, kNarrowPackets = 1, kFairPackets = 2, kClosePackets = 3 };
 
-inline int cast_packets(int sensor, int64_t n_tris, int64_t rays) {
-  if (sensor == kClosePackets && n_tris >= 2048) return small_cast(rays) ? 16 : 32;
-  if (sensor == kSpreadPackets) return 0;
-  if (2 * rays <= kSmallCastRays) return n_tris >= 8192 ? 16 : 0;
-  return sensor >= kFairPackets && rays >= (n_tris < 2048 ? 1 << 19 : 1 << 18) ? 32 : 0;
+// A tree's expected node visits and triangle tests (SAH), as of an 8-wide one.
+inline float walk_cost(const HostBVH& b) { return (float)(b.width == 8 ? b.sah_cost : 0.8 * b.sah_cost); }
+
+inline int cast_packets(int sensor, float cost, int64_t rays) {
+  switch (sensor) {
+    case kClosePackets:
+      return cost < 5.5f && rays < (1 << 19) ? 0 : small_cast(rays) ? 16 : 32;
+    case kFairPackets:
+      return rays >= (1 << 18) ? (cost < 5.5f && rays < (1 << 19) ? 0 : 32)
+                               : cost >= 5.5f && 2 * rays <= kSmallCastRays ? 16 : 0;
+    case kNarrowPackets:
+      return cost >= 7.f && 4 * rays <= kSmallCastRays ? 16 : 0;
+    default:
+      return 0;
+  }
 }
 
-// The same for a batch, whose rays go through one launch: its other kernel hands
-// fresh rays to idle lanes, which a walk in packets has to make up for.  Scenes of
-// 9,868 triangles 0.85-1.13 of the time without packets, 30,012 and more 0.65-1.0,
-// whether close or narrow.  Packets of 16 up to one a warp slot (65,536 rays
-// 0.8-0.9, packets of 32 0.85-1.0; 130,000 rays 0.9-1.1 and 0.8-0.95).
-inline bool batch_packets(int sensor, int64_t n_tris) { return sensor != kSpreadPackets && n_tris >= 16384; }
+// The same for a batch, whose rays go through one launch.  Its other kernel hands
+// fresh rays to idle lanes, which a walk in packets has to make up for, and draws
+// packets one by one, which bounds it where walks are short and rays many: packets
+// take 0.65-0.95 of its time from 5 M rays on, 0.75-1.05 up to 400 k, and between
+// 0.75-1.05 at a cost of 8 and more (narrow ones 0.85-1.05 at 9.5), 1.0-1.2 below.
+// Packets of 16 up to one a warp slot (65,536 rays 0.8-0.9, packets of 32 0.85-1.0;
+// 130,000 rays 0.9-1.1 and 0.8-0.95).
+inline bool batch_packets(int sensor, float cost, int64_t rays) {
+  if (sensor == kSpreadPackets) return false;
+  return rays <= (1 << 19) || rays >= (1 << 22) || cost >= (sensor == kNarrowPackets ? 9.5f : 8.f);
+}
 inline int batch_packet_rays(int64_t rays) { return 2 * rays <= kSmallCastRays ? 16 : 32; }
 
 // The same over a GPU-built LBVH, whose other kernel walks the binary tree ray by

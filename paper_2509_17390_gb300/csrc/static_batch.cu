@@ -28,7 +28,7 @@
 namespace fgl {
 // Allocation-free item check + descriptor fill, and launch-option defaults and
 // checks (api.cu); both return a constant message, or nullptr when valid.
-const char* static_item_desc(const fgl_cast_item& it, ItemDesc* d, int* width, bool* together);
+const char* static_item_desc(const fgl_cast_item& it, ItemDesc* d, int* width, int* packets, float* cost);
 const char* launch_opts(const fgl_batch_opts* o, int* packet, int* block, int* sdepth, int* bpsm,
                         int* graph, int* refill, int* postpone, int* count, int* tri_mode);
 }  // namespace fgl
@@ -117,10 +117,10 @@ extern "C" fgl_status fgl_cast_batched_static(const fgl_cast_item* items, int32_
   // item descriptors, checked once each, then grouped by BVH width straight
   // into the image
   ItemDesc descs[kStaticMaxItems];
-  int widths[kStaticMaxItems];
-  bool gains[kStaticMaxItems];
+  int widths[kStaticMaxItems], kinds[kStaticMaxItems];  // of the trees and of the sensors' packets
+  float costs[kStaticMaxItems];
   for (int i = 0; i < n_items; ++i) {
-    const char* msg = static_item_desc(items[i], &descs[i], &widths[i], &gains[i]);
+    const char* msg = static_item_desc(items[i], &descs[i], &widths[i], &kinds[i], &costs[i]);
     if (msg) return err(FGL_ERR_INVALID, msg);
   }
   StaticImage img;
@@ -139,11 +139,12 @@ extern "C" fgl_status fgl_cast_batched_static(const fgl_cast_item* items, int32_
     int n_in = 0;
     int64_t packets = 0, rays = 0;
     bool tmin = false;
+    for (int i = 0; i < n_items; ++i)
+      if (widths[i] == W) rays += (int64_t)descs[i].n_env * descs[i].n_rays;
     for (int i = 0; i < n_items; ++i) {
       if (widths[i] != W) continue;
       const int64_t warps = (int64_t)descs[i].n_env * ((descs[i].n_rays + 31) / 32);
-      together += gains[i] ? warps : -warps;
-      rays += (int64_t)descs[i].n_env * descs[i].n_rays;
+      together += batch_packets(kinds[i], costs[i], rays) ? warps : -warps;
     }
     const bool walk = together >= 0 && tri_mode == 0 && refill == 32 && packets_fit(W, block, sdepth);
     const int per = walk && !(opts && opts->packet_rays) ? batch_packet_rays(rays) : packet;

@@ -1,7 +1,7 @@
 """Which casts walk packets of rays together: the sizes on either side of each
 line of the rule -- sensors of few rays and of half-empty packets, coarse and fine
-ones, scenes of 108 to 64,000 triangles, casts of up to 136,192 rays, of more and of
-524,288 -- return what the lane-serial form returns, bit for bit, over the host-built
+ones, scenes of 108 to 64,000 triangles, nearly empty and cluttered, and of 5,000 to
+4,300,000 rays -- return what the lane-serial form returns, bit for bit, over the host-built
 tree, alone, in a batch and without allocations, and over the GPU-built one."""
 
 import numpy as np
@@ -24,7 +24,7 @@ def field(rows, cols):
 def sensor(name):
     if name.startswith("field"):
         return field(*map(int, name[5:].split("x")))
-    return fgl.Sensor.from_table(synth.grid_sensor(*{"16x360": (16, -15, 15, 360), "5x91": (5, -20, 15, 91),
+    return fgl.Sensor.from_table(synth.grid_sensor(*{"16x360": (16, -15, 15, 360), "5x91": (5, -20, 15, 91), "16x180": (16, -15, 15, 180),
                                                      "5x2048": (5, -20, 15, 2048)}[name]))
 
 
@@ -33,8 +33,10 @@ SCENES = {}
 
 def scene(kind):
     if kind not in SCENES:
-        if kind == "room":
-            v, t, obs = synth.tiny_room_scene(3)
+        if kind in ("room", "boxes"):
+            v, t, obs = synth.tiny_room_scene(3, n_boxes=8 if kind == "room" else 90)
+        elif kind == "ball":
+            v, t, obs = synth.indoor_scene(5, n_spheres=1, n_boxes=0)
         else:
             v, t, obs = synth.indoor_scene(5, n_spheres={"5k": 9, "10k": 20, "64k": 120}[kind],
                                            n_boxes={"5k": 5, "10k": 9, "64k": 60}[kind])
@@ -44,8 +46,10 @@ def scene(kind):
     return SCENES[kind]
 
 
-@pytest.mark.parametrize("kind", ["room", "5k", "10k", "64k"])
-@pytest.mark.parametrize("name,rays", [("16x360", 5760), ("16x360", 140_000), ("16x360", 530_000), ("5x2048", 60_000),
+@pytest.mark.parametrize("kind", ["room", "boxes", "ball", "5k", "10k", "64k"])
+@pytest.mark.parametrize("name,rays", [("16x360", 5760), ("16x360", 140_000), ("16x360", 530_000), ("16x360", 4_300_000),
+                                       ("16x180", 30_000), ("16x180", 300_000), ("5x2048", 60_000),
+                                       ("5x91", 30_000),
                                        ("5x91", 60_000), ("5x91", 80_000), ("field4x4", 4000), ("field3x11", 70_000),
                                        ("field7x8", 70_000), ("field1x27", 5000), ("field1x28", 5000)])
 def test_rule(kind, name, rays):
