@@ -191,8 +191,8 @@ typedef struct {
 } fgl_cast_item;
 
 typedef struct {
-  int32_t packet_rays;    /* rays per work packet (0 = 32, or 16 in a batch of at most 136,192
-                             rays of narrow packets; multiple of 32) */
+  int32_t packet_rays;    /* rays per work packet (0 = 32, or 16 where a batch of at most
+                             68,096 rays is walked in packets; multiple of 32) */
   int32_t block_threads;  /* threads per block (0 = 128; multiple of 32, <= 512) */
   int32_t stack_smem;     /* traversal stack entries kept in shared memory (0 = 6) */
   int32_t blocks_per_sm;  /* persistent blocks per SM (0 = as many as fit) */

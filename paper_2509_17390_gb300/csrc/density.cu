@@ -245,9 +245,9 @@ __global__ void k_tile_bounds(const uint32_t* __restrict__ keys, int64_t n, int6
 // (the others of a smaller tile leave at once).  Bound by instruction issue and the FMA pipe about equally
 // (36 warp instructions for a candidate and 32 rows, of which 3 exponentials;
 // one exponential a voxel took 40, and 8 of them held the MUFU pipe longest).
-// 720 k Gaussians, 10,304 tiles of 2.5 cm voxels: 2.22 -> 1.47 ms; 85 k
-// Gaussians, 630 tiles of 5 cm, up to 11,400 candidates a tile: 0.63 -> 0.10 ms
-// (0.23 without the clusters and with the voxels close to theta one at a time).
+// 720 k Gaussians, 10,304 tiles of 2.5 cm voxels: 2.16 ms with one exponential a
+// voxel, 1.41 so; 85 k Gaussians, 630 tiles of 5 cm, up to 11,400 candidates a
+// tile: 0.67 and 0.11 ms (the least of eight 0.670 and 0.109).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   uint64_t d;

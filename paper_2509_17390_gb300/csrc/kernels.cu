@@ -398,10 +398,11 @@ __global__ void __maxnreg__(72) k_plain_packets(const ItemDesc it, int sdepth, u
 // the rays of each 32 at a time.  Bound, like k_persistent, by instruction
 // issue (0.70-0.75 of it), but with 140 instead of 224 warp instructions a ray:
 // 4096 x 5760 rays on 1 M triangles of a cluttered room 4.91 -> 3.46 ms, a fleet
-// of dense sensors on 3 cm triangles 1.86 -> 1.59 ms, one 57,600-ray scan (alone,
-// packets of 16 rays) 54 -> 35 us.  Under the 72-register cap 52 bytes a thread spill; 64 (more
-// spills) and 80 (fewer warps) are 1-5% slower, and sharing the loop with k_persistent's
-// refill of partly idle warps keeps so much alive that most of the gain is lost.
+// of dense sensors on 3 cm triangles 1.86 -> 1.59 ms; k_plain_packets takes 35 us
+// for one scan of 57,600 rays (packets of 16; 42 with 32, a call 51 -> 38 us).  Under
+// the 72-register cap 52 bytes a thread spill; 64 (more spills) and 80 (fewer warps)
+// are 1-5% slower, and sharing the loop with k_persistent's refill of partly idle
+// warps keeps so much alive that most of the gain is lost.
 //
 // The queue's counter hands out a draw every 2.6 ns, which bounds cheap
 // packets (368,640 on 20 k triangles took 0.99 ms), so a warp draws three at

@@ -47,8 +47,8 @@ static_assert(kStaticBytes % 16 == 0, "scratch is copied in 16-byte words");
 // its device address comes from cudaGetSymbolAddress below.
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
 
-// The table image travels as a kernel parameter (16 + 2 * 64 + 256 * 96 =
-// 24,720 bytes, within the 32,764-byte parameter limit), so no host staging
+// The table image travels as a kernel parameter (16 + 2 * 64 + 256 * 112 =
+// 28,816 bytes, within the 32,764-byte parameter limit), so no host staging
 // buffer is needed either.
 struct StaticImage {
   uint32_t n_words;
