@@ -243,8 +243,9 @@ __global__ void k_tile_bounds(const uint32_t* __restrict__ keys, int64_t n, int6
 // in warp order.  In a grid of few tiles, one of more than 2 x 32 S candidates is
 // shared by the K blocks of a cluster, whose sums the first adds in block order
 // (the others of a smaller tile leave at once).  Bound by instruction issue and the FMA pipe about equally
-// (36 warp instructions for a candidate and 32 rows, of which 3 exponentials;
-// one exponential a voxel took 40, and 8 of them held the MUFU pipe longest).
+// (32 warp instructions for a candidate and 32 rows, counted over a launch, of which
+// 3 exponentials; one exponential a voxel took 40, and 8 of them held the MUFU pipe
+// longest).
 // 720 k Gaussians, 10,304 tiles of 2.5 cm voxels: 2.16 ms with one exponential a
 // voxel, 1.41 so; 85 k Gaussians, 630 tiles of 5 cm, up to 11,400 candidates a
 // tile: 0.67 and 0.11 ms (the least of eight 0.670 and 0.109).
